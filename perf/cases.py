@@ -1,0 +1,358 @@
+"""The work that a program using this framework has it do, as cases that can be timed and compared.
+
+A serving program keeps a corpus on the GPU, builds one ``EmbedRetrieveStage``
+(or a graph of it) over it, and sends batches through; a scheduler around it
+merges token rows, fans results out, reranks candidates and sums priorities
+with the single calls.  Every case goes through those entry points.
+
+  step      stage.step: chunk merge and merged retrieval of one batch of workflows
+  retrieve  stage.retrieve: the query path alone, batch by batch
+  graph     RetrieveGraph.run: the same captured once, for the smallest latency
+  topk      hs_retrieve_topk: unmerged queries near a corpus's clusters, large k
+  merge     hs_merge_rows, then hs_scatter_results of the unique rows' results
+  unique    hs_fingerprint with a seed, then hs_unique_inverse (node signatures
+            that a caller continues from its own)
+  rerank    hs_rerank_topk with the fan-out to the merged queries
+  cached    stage.retrieve with a result cache that holds the batch already
+  priority  hs_segment_sum of the rows merged into each node
+
+The data are synthetic: Gaussian unit vectors in bf16 and token ids below
+32,000, with planted copies (a share of the rows copies earlier rows, or rows
+are drawn Zipf(1.1) from a pool).
+"""
+import math
+
+import numpy as np
+import torch
+
+import paper_2607_22578_gb300 as hs
+
+VOCAB = 32000
+ZIPF = 1.1
+
+LISTED = [
+    # A handful of small workflows on a small corpus: launches and host work are all there is.
+    dict(name="step_tiny", kind="step", queries=32, q_dup=0.25, rows=256, stride=128,
+         copies=0.5, N=4096, d=384, k=10),
+    # 64 concurrent workflows over a million chunks: the whole stage at its ordinary size.
+    dict(name="step_rag_mix", kind="step", queries=2048, q_dup=0.3, rows=65536, stride=256,
+         copies=0.4, N=1048576, d=768, k=10),
+    # One interactive query, captured as a graph: the lowest latency that the stage offers.
+    dict(name="graph_b1", kind="graph", queries=1, q_dup=0.0, N=2097152, d=768, k=10),
+    # A small online batch: bound by reading the corpus.
+    dict(name="retrieve_b64", kind="retrieve", queries=64, q_dup=0.2, N=2097152, d=768, k=10),
+    # A middle batch: between the memory's and the tensor cores' bound.
+    dict(name="retrieve_b512", kind="retrieve", queries=512, q_dup=0.2, N=2097152, d=768, k=10),
+    # An offline pass of many queries over a large clustered corpus, k = 100.
+    dict(name="topk_large", kind="topk", queries=4096, N=8388608, d=1024, k=100, clusters=1024),
+    # Popular documents: ragged chunk rows drawn Zipf from a pool, an embedding fanned out to each.
+    dict(name="merge_zipf", kind="merge", rows=400000, stride=512, shortest=64, pool=100000,
+         copies=0.0, shared=0, payload=1536),
+    # Mostly distinct rows (a tenth are copies) that begin with one of 16 prompt templates.
+    dict(name="merge_sparse", kind="merge", rows=100003, stride=256, shortest=32, pool=0,
+         copies=0.1, shared=24, payload=80),
+    # Rows at an odd stride, hashed from a caller's seed: no 16-byte alignment.
+    dict(name="unique_odd", kind="unique", rows=20011, stride=333, shortest=1, pool=0,
+         copies=0.3, shared=0),
+    # The second stage of RAG with rerank: top-12 rescored, top-8 kept.
+    dict(name="rerank", kind="rerank", queries=2048, q_dup=0.3, N=1048576, d=1024, k1=12, k=8),
+    # A batch whose results are in the cache from an earlier one.
+    dict(name="cached", kind="cached", queries=2048, q_dup=0.3, N=262144, d=768, k=10,
+         capacity=65536),
+    # Scheduling weights of the nodes that 400,000 rows merge into.
+    dict(name="priority", kind="priority", rows=400000, pool=100000),
+]
+
+
+def listed():
+    return [dict(c) for c in LISTED]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["step", "retrieve", "retrieve", "graph", "topk", "merge", "merge",
+                       "unique", "rerank", "cached", "priority"])
+    dup = round(rng.uniform(0.0, 0.5), 3)
+    d = 8 * _log(rng, 8, 128)
+    if kind == "step":
+        return dict(kind=kind, queries=_log(rng, 8, 2048), q_dup=dup, rows=_log(rng, 64, 65536),
+                    stride=_log(rng, 16, 512), copies=round(rng.uniform(0.05, 0.9), 3),
+                    N=_log(rng, 1000, 1 << 20), d=d, k=_log(rng, 1, 100))
+    if kind in ("retrieve", "graph"):
+        most = 4096 if kind == "retrieve" else 256
+        return dict(kind=kind, queries=_log(rng, 1, most), q_dup=dup, N=_log(rng, 1000, 2 << 20),
+                    d=d, k=_log(rng, 1, 100))
+    if kind == "topk":
+        return dict(kind=kind, queries=_log(rng, 8, 4096), N=_log(rng, 70000, 2 << 20), d=d,
+                    k=_log(rng, 10, 200), clusters=_log(rng, 16, 256))
+    if kind in ("merge", "unique"):
+        stride = _log(rng, 16, 512)
+        zipf = rng.random() < 0.5
+        rows = _log(rng, 1000, 400000 if kind == "merge" else 100000)
+        case = dict(kind=kind, rows=rows, stride=stride, shortest=rng.randint(1, stride),
+                    pool=max(4, rows // rng.randint(2, 8)) if zipf else 0,
+                    copies=0.0 if zipf else round(rng.uniform(0.05, 0.9), 3),
+                    shared=rng.choice([0, stride // 8, stride // 3]))
+        if kind == "merge":
+            case["payload"] = rng.choice([4, 16]) * _log(rng, 2, 100)
+        return case
+    if kind == "rerank":
+        k1 = rng.randint(4, 32)
+        return dict(kind=kind, queries=_log(rng, 8, 4096), q_dup=dup, N=_log(rng, 1000, 1 << 20),
+                    d=d, k1=k1, k=rng.randint(1, k1))
+    if kind == "cached":
+        q = _log(rng, 8, 2048)
+        return dict(kind=kind, queries=q, q_dup=dup, N=_log(rng, 1000, 1 << 18), d=d,
+                    k=_log(rng, 1, 100), capacity=64 * q)
+    return dict(kind=kind, rows=_log(rng, 1000, 1000000), pool=_log(rng, 100, 200000))
+
+
+# ---- inputs ------------------------------------------------------------------------------------
+def _gen(seed):
+    return torch.Generator(device="cuda").manual_seed(seed)
+
+
+def _unit(n, d, g, centres=None, of=None):
+    """n unit-norm bf16 rows; rows with of[i] >= 0 lie near centres[of[i]]."""
+    out = torch.empty((n, d), dtype=torch.bfloat16, device="cuda")
+    for i in range(0, n, 1 << 19):
+        x = torch.randn((min(1 << 19, n - i), d), generator=g, device="cuda")
+        if of is not None:
+            at = (of[i:i + len(x)] >= 0).nonzero()[:, 0]
+            x[at] = centres[of[i + at]] + x[at] * (0.05 / math.sqrt(d))
+        out[i:i + len(x)] = x / x.norm(dim=1, keepdim=True)
+    return out
+
+
+def _roots(n, copies, g):
+    """root[i]: the row that row i repeats; a share `copies` of them copies a distinct earlier row."""
+    base = torch.ones(n, dtype=torch.bool, device="cuda")
+    m = int(round(copies * (n - 1)))
+    base[1 + torch.randperm(n - 1, generator=g, device="cuda")[:m]] = False
+    first = base.nonzero()[:, 0]
+    before = base.cumsum(0)                       # distinct rows up to and with i
+    pick = (torch.rand(n, generator=g, device="cuda", dtype=torch.float64) * before).long()
+    return torch.where(base, torch.arange(n, device="cuda"), first[torch.minimum(pick, before - 1)])
+
+
+def _zipf(n, pool, g):
+    p = torch.arange(1, pool + 1, device="cuda", dtype=torch.float64).pow(-ZIPF).cumsum(0)
+    u = torch.rand(n, generator=g, device="cuda", dtype=torch.float64) * p[-1]
+    return torch.searchsorted(p, u).clamp_(max=pool - 1)
+
+
+def _queries(case, g):
+    q = _unit(case["queries"], case["d"], g)
+    return q[_roots(len(q), case["q_dup"], g)].contiguous()
+
+
+def _tokens(rows, stride, g, shortest=None, pool=0, copies=0.0, shared=0):
+    """Token rows and their lengths (None: all of `stride`): zeros past the length; with `shared`,
+    the first `shared` tokens of a row are one of 16 templates."""
+    n = pool or rows
+    tokens = torch.randint(0, VOCAB, (n, stride), generator=g, device="cuda", dtype=torch.int32)
+    if shared:
+        head = torch.randint(0, VOCAB, (16, shared), generator=g, device="cuda", dtype=torch.int32)
+        tokens[:, :shared] = head[torch.randint(0, 16, (n,), generator=g, device="cuda")]
+    lens = None
+    if shortest is not None:
+        lens = torch.randint(shortest, stride + 1, (n,), generator=g, device="cuda",
+                             dtype=torch.int32)
+        tokens.masked_fill_(torch.arange(stride, device="cuda")[None, :] >= lens[:, None], 0)
+    root = _zipf(rows, pool, g) if pool else _roots(rows, copies, g)
+    return tokens[root].contiguous(), None if lens is None else lens[root].contiguous()
+
+
+def _chunk_args(case):
+    return {k: case[k] for k in ("shortest", "pool", "copies", "shared") if k in case}
+
+
+def prepare(case, seed):
+    g, kind = _gen(seed), case["kind"]
+    s = {"kind": kind, "k": case.get("k")}
+    if kind in ("step", "retrieve", "graph", "cached"):
+        corpus = _unit(case["N"], case["d"], g)
+        s["queries"] = _queries(case, g)
+        s["stage"] = hs.EmbedRetrieveStage(corpus, case["k"], case["queries"],
+                                           case.get("rows", 0),
+                                           cache_capacity=case.get("capacity", 0))
+        if kind == "step":
+            s["tokens"], _ = _tokens(case["rows"], case["stride"], g, copies=case["copies"])
+        elif kind == "graph":
+            s["graph"] = hs.RetrieveGraph(s["stage"], case["queries"])
+        elif kind == "cached":
+            s["stage"].retrieve(s["queries"])      # the earlier batch
+    elif kind == "topk":
+        centres = _unit(case["clusters"], case["d"], g).float()
+        of = torch.full((case["N"],), -1, dtype=torch.long, device="cuda")
+        at = torch.randperm(case["N"], generator=g, device="cuda")[:128 * case["clusters"]]
+        of[at] = torch.arange(len(at), device="cuda") % case["clusters"]
+        s["corpus"] = _unit(case["N"], case["d"], g, centres, of)
+        near = torch.randint(0, case["clusters"], (case["queries"],), generator=g, device="cuda")
+        s["queries"] = _unit(case["queries"], case["d"], g, centres, near)
+        s["workspace"] = torch.empty(hs.hs_retrieve_topk_workspace(
+            case["queries"], case["N"], case["d"], case["k"]), dtype=torch.uint8, device="cuda")
+    elif kind in ("merge", "unique"):
+        s["tokens"], s["lens"] = _tokens(case["rows"], case["stride"], g, **_chunk_args(case))
+        if kind == "merge":
+            s["workspace"] = torch.empty(hs.hs_merge_rows_workspace(case["rows"]),
+                                         dtype=torch.uint8, device="cuda")
+            s["results"] = torch.randint(-2 ** 31, 2 ** 31 - 1, (case["rows"], case["payload"] // 4),
+                                         generator=g, device="cuda", dtype=torch.int32)
+        else:
+            s["seed_state"] = seed * 0x9E3779B97F4A7C15 % 2 ** 64
+            s["workspace"] = torch.empty(hs.hs_unique_inverse_workspace(case["rows"]),
+                                         dtype=torch.uint8, device="cuda")
+    elif kind == "rerank":
+        q, n = case["queries"], case["queries"] - int(round(case["q_dup"] * (case["queries"] - 1)))
+        s["corpus"] = _unit(case["N"], case["d"], g)
+        s["queries"] = _unit(q, case["d"], g)
+        s["candidates"] = torch.randint(0, case["N"], (q, case["k1"]), generator=g, device="cuda",
+                                        dtype=torch.int32)
+        s["count"] = torch.tensor([n], dtype=torch.int32, device="cuda")
+        s["inverse"] = torch.randint(0, n, (q,), generator=g, device="cuda", dtype=torch.int32)
+    elif kind == "priority":
+        group = _zipf(case["rows"], case["pool"], g)
+        first = torch.full((case["pool"],), case["rows"], device="cuda").scatter_reduce_(
+            0, group, torch.arange(case["rows"], device="cuda"), "amin")
+        s["inverse"] = first.argsort().argsort()[group].int()      # ordinals by first occurrence
+        s["count"] = (first < case["rows"]).sum().int().reshape(1)
+        s["phi"] = torch.rand(case["rows"], generator=g, device="cuda", dtype=torch.float64)
+    return s
+
+
+def run(s):
+    kind = s["kind"]
+    if kind == "step":
+        return s["stage"].step(s["tokens"], s["queries"])
+    if kind in ("retrieve", "cached"):
+        return s["stage"].retrieve(s["queries"])
+    if kind == "graph":
+        return s["graph"].run(s["queries"])
+    if kind == "topk":
+        return hs.hs_retrieve_topk(s["queries"], s["corpus"], s["k"], workspace=s["workspace"])
+    if kind == "merge":
+        fp, n, unique, inverse = hs.hs_merge_rows(s["tokens"], s["lens"],
+                                                  workspace=s["workspace"])
+        return fp, n, unique, inverse, hs.hs_scatter_results(s["results"], inverse)
+    if kind == "unique":
+        fp = hs.hs_fingerprint(s["tokens"], s["lens"], s["seed_state"])
+        return (fp,) + hs.hs_unique_inverse(fp, s["tokens"], s["lens"], workspace=s["workspace"])
+    if kind == "rerank":
+        return hs.hs_rerank_topk(s["queries"], s["corpus"], s["candidates"], s["k"], s["count"],
+                                 s["inverse"])
+    return hs.hs_segment_sum(s["phi"], s["inverse"], len(s["phi"]), s["count"])
+
+
+# ---- what a pass cannot do without -------------------------------------------------------------
+def _unique_rows(case):
+    if case.get("pool"):
+        p = np.arange(1, case["pool"] + 1, dtype=np.float64) ** -ZIPF
+        return float(-np.expm1(case["rows"] * np.log1p(-p / p.sum())).sum())
+    return case["rows"] - round(case["copies"] * (case["rows"] - 1))
+
+
+def _merge_bytes(case):
+    words = case["stride"]
+    if "shortest" in case:
+        words = (case["shortest"] + case["stride"]) / 2 + 1
+    return case["rows"] * (4.0 * words + 8 + 4 + 4)
+
+
+def work(case):
+    kind = case["kind"]
+    if kind == "priority":
+        return {"bytes": 12.0 * case["rows"] + 8.0 * case["rows"], "flops": 1.0 * case["rows"]}
+    if kind in ("merge", "unique"):
+        b = _merge_bytes(case)
+        if kind == "merge":
+            b += case["payload"] * (case["rows"] + _unique_rows(case))
+        return {"bytes": b, "flops": 0.0}
+    q, d, k, n = case["queries"], case["d"], case["k"], case["N"]
+    if kind == "topk":
+        return {"bytes": 2.0 * d * (n + q) + 8.0 * q * k, "flops": 2.0 * q * n * d}
+    merged = q - round(case["q_dup"] * (q - 1))
+    if kind == "rerank":
+        rows = min(float(n), merged * float(case["k1"]))
+        return {"bytes": 2.0 * d * (rows + merged) + 4.0 * q + 4.0 * merged * case["k1"] + 8.0 * q * k,
+                "flops": 2.0 * merged * case["k1"] * d}
+    if kind == "cached":                           # the batch, its entries, its results
+        return {"bytes": 2.0 * d * (q + merged) + 8.0 * merged * k + 8.0 * q * k, "flops": 0.0}
+    b = 2.0 * d * (n + q) + 8.0 * q * k
+    if kind == "step":
+        b += _merge_bytes(case)
+    return {"bytes": b, "flops": 2.0 * merged * n * d}
+
+
+# ---- how far another correct implementation may be off -----------------------------------------
+def tolerance(case):
+    kind = case["kind"]
+    if kind in ("merge", "unique"):
+        return "exact"                             # fingerprints, partitions and copied bytes
+    if kind == "priority":
+        return {"rel": 3e-14, "max": 4e-14}        # fp64 sums in another order: 7e-15 seen
+    # fp32 sums of bf16 products in another order, and ids that swap where two scores tie within
+    # that.  Seen against 64 bits: rerank 8e-8; unmerged queries inside clusters, whose hundred
+    # best lie within 1e-3, 2e-6 (and up to 4 % of the ids: the sums' order is kept here, so 1 % is let pass); else 9e-7.
+    if kind == "rerank":
+        return {"rel": 4e-7, "max": 2e-6, "differ": 0.0002}
+    if kind == "topk":
+        return {"rel": 8e-6, "max": 1.2e-5, "differ": 0.01}
+    return {"rel": 4e-6, "max": 8e-6, "differ": 0.0002}
+
+
+# ---- the same in 64 bits -----------------------------------------------------------------------
+def _ordered(scores, ids, k):
+    """The first k of each row by score descending, ties to the lower id."""
+    ids, at = ids.sort(dim=1)
+    scores, at = scores.gather(1, at).sort(dim=1, descending=True, stable=True)
+    return scores[:, :k].contiguous(), ids.gather(1, at)[:, :k].int().contiguous()
+
+
+def _rescored(queries, corpus, ids):
+    out = torch.empty(ids.shape, dtype=torch.float64, device="cuda")
+    for i in range(0, len(ids), 128):
+        rows = corpus[ids[i:i + 128].long()].double()
+        out[i:i + 128] = torch.einsum("qd,qkd->qk", queries[i:i + 128].double(), rows)
+    return out
+
+
+def _exact_topk(queries, corpus, k):
+    """Scores in 64 bits of the rows that lead in 32 bits, with 28 more than asked for in reserve."""
+    keep, best_s, best_i = k + 28, None, None
+    q = queries.float()
+    for i in range(0, len(corpus), 1 << 18):
+        s, j = (q @ corpus[i:i + (1 << 18)].float().T).topk(min(keep, len(corpus) - i, 1 << 18))
+        j = j + i
+        if best_s is not None:
+            s, j = torch.cat([best_s, s], 1), torch.cat([best_i, j], 1)
+            s, at = s.topk(min(keep, s.shape[1]))
+            j = j.gather(1, at)
+        best_s, best_i = s, j
+    return _ordered(_rescored(queries, corpus, best_i), best_i, k)
+
+
+def exact(case, seed):
+    """What run() returns, its scores and sums in 64 bits; None in the place of the merge's whole
+    numbers and of copied bytes."""
+    kind = case["kind"]
+    if kind in ("merge", "unique"):
+        return None
+    s = prepare(case, seed)
+    if kind == "priority":
+        return torch.from_numpy(np.bincount(s["inverse"].cpu().numpy(), s["phi"].cpu().numpy(),
+                                            case["rows"]))
+    if kind == "topk":
+        return _exact_topk(s["queries"], s["corpus"], case["k"])
+    if kind == "rerank":
+        of = s["inverse"].long()
+        scores, ids = _ordered(_rescored(s["queries"], s["corpus"], s["candidates"]),
+                               s["candidates"], case["k"])
+        return scores[of], ids[of]
+    scores, ids = _exact_topk(s["queries"], s["stage"].corpus, case["k"])
+    if kind == "step":
+        return (None, None, None, None), (scores, ids, None)
+    return scores, ids, None

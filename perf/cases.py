@@ -128,7 +128,7 @@ def _unit(n, d, g, centres=None, of=None):
 
 
 def _roots(n, copies, g):
-    """root[i]: the row that row i repeats; a share `copies` of them copies a distinct earlier row."""
+    """root[i]: the row that row i repeats (a share `copies` of them: a distinct earlier row)."""
     base = torch.ones(n, dtype=torch.bool, device="cuda")
     m = int(round(copies * (n - 1)))
     base[1 + torch.randperm(n - 1, generator=g, device="cuda")[:m]] = False
@@ -200,8 +200,9 @@ def prepare(case, seed):
         if kind == "merge":
             s["workspace"] = torch.empty(hs.hs_merge_rows_workspace(case["rows"]),
                                          dtype=torch.uint8, device="cuda")
-            s["results"] = torch.randint(-2 ** 31, 2 ** 31 - 1, (case["rows"], case["payload"] // 4),
-                                         generator=g, device="cuda", dtype=torch.int32)
+            s["results"] = torch.randint(-2 ** 31, 2 ** 31 - 1,
+                                         (case["rows"], case["payload"] // 4), generator=g,
+                                         device="cuda", dtype=torch.int32)
         else:
             s["seed_state"] = seed * 0x9E3779B97F4A7C15 % 2 ** 64
             s["workspace"] = torch.empty(hs.hs_unique_inverse_workspace(case["rows"]),
@@ -277,8 +278,8 @@ def work(case):
     merged = q - round(case["q_dup"] * (q - 1))
     if kind == "rerank":
         rows = min(float(n), merged * float(case["k1"]))
-        return {"bytes": 2.0 * d * (rows + merged) + 4.0 * q + 4.0 * merged * case["k1"] + 8.0 * q * k,
-                "flops": 2.0 * merged * case["k1"] * d}
+        return {"bytes": 2.0 * d * (rows + merged) + 4.0 * q + 4.0 * merged * case["k1"]
+                + 8.0 * q * k, "flops": 2.0 * merged * case["k1"] * d}
     if kind == "cached":                           # the batch, its entries, its results
         return {"bytes": 2.0 * d * (q + merged) + 8.0 * merged * k + 8.0 * q * k, "flops": 0.0}
     b = 2.0 * d * (n + q) + 8.0 * q * k
@@ -296,7 +297,7 @@ def tolerance(case):
         return {"rel": 3e-14, "max": 4e-14}        # fp64 sums in another order: 7e-15 seen
     # fp32 sums of bf16 products in another order, and ids that swap where two scores tie within
     # that.  Seen against 64 bits: rerank 8e-8; unmerged queries inside clusters, whose hundred
-    # best lie within 1e-3, 2e-6 (and up to 4 % of the ids: the sums' order is kept here, so 1 % is let pass); else 9e-7.
+    # best lie within 1e-3, 2e-6 (and up to 4 % of the ids: here 1 % is let pass); else 9e-7.
     if kind == "rerank":
         return {"rel": 4e-7, "max": 2e-6, "differ": 0.0002}
     if kind == "topk":

@@ -2,10 +2,8 @@
 // part of the node semantic signature Sig(v) (Section 3.3, Eq. 2).
 //
 // FNV-1a is a serial chain over the octets of one row, so parallelism comes
-// from rows: each lane of a warp owns one row at a time.  Rows are split into
-// full chunks of 32 tokens, hashed in registers by the chunk kernel with a
-// straight-line, predicate-free loop, and a tail of L mod 32 tokens, finished
-// by a one-thread-per-row tail kernel from the partial state.
+// from rows: each lane of a warp owns one row at a time and hashes it in
+// chunks of 32 tokens, straight-line from registers.
 // The octet rounds themselves are in fnv.cuh.
 #include "fnv.cuh"
 #include "hs_internal.cuh"
@@ -15,21 +13,29 @@ namespace {
 
 using namespace fnv;
 
-// ---- vector path: full chunks in registers, tails in a second kernel -------------
-// A warp owns 32 rows at a time, one per lane.  The chunk kernel hashes only
-// FULL chunks of T = 32 tokens: tokens [0, floor(L/T)*T) of every row with
-// L >= T.  Each lane loads its next chunk with 16- or 32-byte vector loads
+// A lane loads its next chunk of T = 32 tokens with 16- or 32-byte loads
 // straight into registers one chunk ahead of the chunk it hashes (NB register
-// buffers), so every lane runs the same straight-line hash over T tokens: no
-// per-token predicates and no masking.  After its last full chunk a row's
-// state goes to fp_out: the final fingerprint when T divides L, otherwise the
-// partial state, which the tail kernel finishes with the last L mod T tokens
-// (one thread per row, so the few short tails run with the whole GPU's
-// parallelism instead of serially at the end of each warp).  Rows shorter
-// than T and rows with an invalid length are left entirely to the tail
-// kernel.  A lane that has issued its row's last chunk claims the next
+// buffers).  A lane that has issued its row's last chunk claims the next
 // unclaimed row of its warp's range (lengths prefetched 64 rows ahead and
 // handed out by shuffle).
+//
+// Chunks start on a 16-byte boundary, so a row that does not gets up to three
+// tokens of the chunk before its first, and its last chunk may run past its
+// length.  Both are hashed as zeros: a round on a zero octet is a plain
+// multiply by the prime, which is odd and so has an inverse mod 2^64.  The
+// state is multiplied by the inverse once per padding octet (a table of
+// powers), before a row's first chunk and after its last, and comes out
+// exactly as if the padding had not been there.  So every lane runs the same
+// straight-line hash whatever its row's start and length, in one pass.
+//
+// Bound by the memory system: 16 warps an SM each keep one 128-byte chunk per
+// lane in flight, in as many places as there are rows.  400,000 rows of 64 to
+// 512 tokens: 115 us, 4.0 TB/s (116 us as a pass over full chunks and a second
+// one over the rests); 200,000 rows of 512: 82 us, 5.0 TB/s (86); 400,000 rows
+// of at most 36: 20 us (26); 20,011 rows at a stride of 333: 23 us cold (132 us
+// hashing word by word).  Rests queued and hashed 32 at a time, steps left
+// out by a vote of the warp, and loads with a 256-byte prefetch or a bulk
+// prefetch to L2 were each slower.
 //
 // A chunk whose tokens are all below 65536 (in every live lane) takes the
 // two-round small-token hash; otherwise the whole chunk takes the octet-wise
@@ -49,8 +55,199 @@ __device__ __forceinline__ void load_vec(const int32_t* p, uint32_t* x) {
   }
 }
 
-constexpr int kTailChunk = 32;  // T: tokens per full chunk
+constexpr int kChunk = 32;      // T: tokens per chunk
+constexpr int kStep = 8;        // tokens per step that rows shorter than a chunk can leave out
+constexpr int kFpThreads = 256;
 
+// kUnpad.v[t] = prime^-(4 t): undoes t zero tokens.
+struct Unpad {
+  uint64_t v[kChunk + 1];
+};
+constexpr Unpad make_unpad() {
+  uint64_t inv = kPrime;                       // x = inv solves x * prime = 1 (mod 8)
+  for (int i = 0; i < 5; ++i) inv *= 2 - kPrime * inv;   // Newton: the exact bits double
+  Unpad u{};
+  u.v[0] = 1;
+  for (int t = 1; t <= kChunk; ++t) u.v[t] = u.v[t - 1] * inv * inv * inv * inv;
+  return u;
+}
+static_assert(make_unpad().v[1] * kPrime * kPrime * kPrime * kPrime == 1, "inverse of the prime");
+__constant__ Unpad kUnpad = make_unpad();
+
+// VB bytes per load, K loads per chunk, NB register buffers.  MASK: a chunk
+// may hold tokens that are not the row's (lengths, or a stride that is no
+// multiple of T); HEAD: and rows may start off a 16-byte boundary (4-byte
+// aligned), VB is then 16.
+template <int VB, int K, int NB, bool MASK, bool HEAD>
+__global__ void __launch_bounds__(kFpThreads) fingerprint_kernel(
+    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
+    const int32_t* __restrict__ lens, uint64_t seed, uint64_t* __restrict__ fp_out,
+    int64_t rows_per_warp, unsigned* err) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int W = VB / 4;  // tokens per vector load
+  constexpr int T = W * K;   // tokens per chunk
+  static_assert(T == kChunk && (!HEAD || (MASK && W == 4)), "chunk of 32 tokens, offsets below 4");
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t r_begin = warp * rows_per_warp;
+  if (r_begin >= n) return;
+  const int64_t r_end = min(n, r_begin + rows_per_warp);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t seed_lo = (uint32_t)seed, seed_hi = (uint32_t)(seed >> 32);
+  const int32_t* const tokens_end = tokens + n * (int64_t)stride;
+  // Rows of fewer than T tokens (the same for every row): steps past them are
+  // left out.
+  const int used = MASK ? min(T, (stride + (HEAD ? 3 : 0) + kStep - 1) / kStep * kStep) : T;
+
+  // Issue side: the row being loaded, its next chunk's first token (-3 ... -1
+  // in a first chunk that starts before the row), its length.
+  int64_t irow = -1;
+  int32_t ipos = 0, ilen = 0;
+  uint32_t buf[NB][T];
+  int64_t brow[NB];
+  int32_t bend[NB];              // tokens [pad, bend) of the buffer are the row's ...
+  int32_t bpos[NB];              // ... with pad = max(0, -bpos)
+  bool blast[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    brow[b] = -1;
+    bend[b] = bpos[b] = 0;
+    blast[b] = false;
+  }
+  uint32_t lo = seed_lo, hi = seed_hi;
+
+  int64_t next = r_begin;
+  int64_t wbase = r_begin;
+  auto len_of = [&](int64_t r) -> int32_t {
+    return r < r_end ? (lens ? __ldg(lens + r) : stride) : 0;
+  };
+  int32_t len_a = len_of(wbase + lane), len_b = len_of(wbase + 32 + lane);
+
+  auto claim = [&]() {
+    unsigned need = __ballot_sync(0xffffffffu, irow < 0);
+    while (need != 0u && next < r_end) {
+      const int64_t avail = r_end - next;
+      const int rank = __popc(need & lanemask_lt());
+      const int off = (int)(next - wbase) + (irow < 0 ? rank : 0);
+      const int32_t La = __shfl_sync(0xffffffffu, len_a, off & 31);
+      const int32_t Lb = __shfl_sync(0xffffffffu, len_b, off & 31);
+      if (irow < 0 && rank < avail) {
+        const int32_t L = off < 32 ? La : Lb;
+        if (L < 0 || L > stride) {                       // reported, fingerprint 0
+          set_error(err, kErrInvalidArg);
+          fp_out[next + rank] = 0ull;
+        } else if (L == 0) {
+          fp_out[next + rank] = seed;
+        } else {
+          irow = next + rank;
+          ilen = L;
+          ipos = 0;
+          if (HEAD)
+            ipos = -(int32_t)((reinterpret_cast<uintptr_t>(tokens + irow * (int64_t)stride) >> 2) & 3u);
+        }
+      }
+      next += min((int64_t)__popc(need), avail);
+      if (next - wbase >= 32) {
+        wbase += 32;
+        len_a = len_b;
+        len_b = len_of(wbase + 32 + lane);
+      }
+      need = __ballot_sync(0xffffffffu, irow < 0);
+    }
+  };
+
+  // Load this lane's next chunk into buffer b: the pieces that hold one of
+  // the row's tokens.  A piece that would leave the token array (only before
+  // the first row's start and past the last row's end) is read word by word.
+  auto issue = [&](int b) {
+    brow[b] = irow;
+    if (irow >= 0) {
+      const int32_t* src = tokens + irow * (int64_t)stride + ipos;
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const int32_t* p = src + j * W;
+        if (!MASK || ipos + j * W < ilen) {
+          if (!HEAD || (p >= tokens && p + W <= tokens_end)) {
+            load_vec<VB>(p, &buf[b][j * W]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < W; ++i)
+              buf[b][j * W + i] = p + i >= tokens && p + i < tokens_end ? (uint32_t)__ldg(p + i) : 0u;
+          }
+        }
+      }
+      bpos[b] = ipos;
+      bend[b] = min(T, ilen - ipos);
+      ipos += T;
+      blast[b] = ipos >= ilen;
+      if (blast[b]) irow = -1;
+    }
+  };
+
+  // Hash buffer b (every lane, live or not: an idle lane's result is dropped).
+  auto consume = [&](int b) {
+    const bool live = brow[b] >= 0, first = live && bpos[b] <= 0;
+    lo = first ? seed_lo : lo;
+    hi = first ? seed_hi : hi;
+    if (HEAD && first) {
+      const uint64_t h = seed * kUnpad.v[-bpos[b]];
+      lo = (uint32_t)h;
+      hi = (uint32_t)(h >> 32);
+    }
+    if (MASK) {
+      uint32_t own = bend[b] >= T ? 0xffffffffu : (1u << bend[b]) - 1u;
+      if (HEAD && bpos[b] < 0) own &= 0xffffffffu << -bpos[b];
+#pragma unroll
+      for (int t = 0; t < T; ++t)
+        if (!((own >> t) & 1u)) buf[b][t] = 0u;
+    }
+    uint32_t any = 0;
+#pragma unroll
+    for (int t = 0; t < T; ++t) any |= buf[b][t];
+    if (__all_sync(0xffffffffu, !live || (any >> 16) == 0u)) {
+#pragma unroll
+      for (int t0 = 0; t0 < T; t0 += kStep)
+        if (!MASK || t0 < used) {
+#pragma unroll
+          for (int t = t0; t < t0 + kStep; ++t) hash_word_small(lo, hi, buf[b][t]);
+        }
+    } else {
+#pragma unroll
+      for (int t0 = 0; t0 < T; t0 += kStep)
+        if (!MASK || t0 < used) {
+#pragma unroll
+          for (int t = t0; t < t0 + kStep; ++t) hash_word_full(lo, hi, buf[b][t]);
+        }
+    }
+    if (live && blast[b]) {
+      const uint64_t h = ((uint64_t)hi << 32) | lo;
+      fp_out[brow[b]] = MASK ? h * kUnpad.v[used - bend[b]] : h;
+    }
+    brow[b] = -1;
+  };
+
+  // Chunks 0 .. NB-2 in flight before the first hash; then each step loads
+  // chunk c + NB - 1 and hashes chunk c.
+#pragma unroll
+  for (int b = 0; b < NB - 1; ++b) {
+    claim();
+    issue(b);
+  }
+  for (;;) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      claim();
+      issue((b + NB - 1) % NB);
+      consume(b);
+    }
+    bool pending = irow >= 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) pending |= brow[b] >= 0;
+    if (!__any_sync(0xffffffffu, pending) && next >= r_end) break;
+  }
+}
+
+// ---- full chunks only (the first pass of hs_merge_rows) -----------------------------------
 template <int VB, int K, int NB>
 __global__ void __launch_bounds__(256) fingerprint_chunks_kernel(
     const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
@@ -60,7 +257,7 @@ __global__ void __launch_bounds__(256) fingerprint_chunks_kernel(
   pdl_trigger();
   constexpr int W = VB / 4;  // tokens per vector load
   constexpr int T = W * K;   // tokens per chunk
-  static_assert(T == kTailChunk, "chunk size shared with the tail kernel");
+  static_assert(T == kChunk, "chunk size shared with the tail pass");
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t r_begin = warp * rows_per_warp;
   if (r_begin >= n) return;
@@ -169,123 +366,35 @@ __global__ void __launch_bounds__(256) fingerprint_chunks_kernel(
   }
 }
 
-// The last L mod T tokens of every row (the whole row when L < T), one thread
-// per row, continuing from the partial state the chunk kernel left in fp_out.
-// Also the row-length checks: an invalid length sets the error flag and a
-// zero fingerprint; an empty row gets the seed.  Needs 16-byte aligned rows.
-__global__ void __launch_bounds__(256) fingerprint_tails_kernel(
-    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
-    const int32_t* __restrict__ lens, uint64_t seed, uint64_t* __restrict__ fp_out,
-    unsigned* err) {
-  pdl_wait();
-  pdl_trigger();
-  constexpr int T = kTailChunk;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t L = lens ? __ldg(lens + r) : stride;
-    if (L < 0 || L > stride) {
-      set_error(err, kErrInvalidArg);
-      fp_out[r] = 0ull;
-      continue;
-    }
-    const int32_t m = L % T;
-    if (m == 0 && L > 0) continue;  // the chunk kernel wrote the final value
-    uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-    if (L >= T) {
-      const uint64_t st = fp_out[r];
-      lo = (uint32_t)st;
-      hi = (uint32_t)(st >> 32);
-    }
-    const int32_t* src = tokens + r * (int64_t)stride + (L - m);
-    uint4 v[T / 4];
-#pragma unroll
-    for (int q = 0; q < T / 4; ++q)
-      if (4 * q < m) v[q] = __ldg(reinterpret_cast<const uint4*>(src + 4 * q));
-#pragma unroll
-    for (int q = 0; q < T / 4; ++q) {
-      if (4 * q < m) hash_word(lo, hi, v[q].x);
-      if (4 * q + 1 < m) hash_word(lo, hi, v[q].y);
-      if (4 * q + 2 < m) hash_word(lo, hi, v[q].z);
-      if (4 * q + 3 < m) hash_word(lo, hi, v[q].w);
-    }
-    fp_out[r] = ((uint64_t)hi << 32) | lo;
+template <int VB, int K, int NB, bool MASK, bool HEAD>
+hs_status launch_rows(const int32_t* tokens, int64_t n, int32_t stride, const int32_t* lens,
+                      uint64_t seed, uint64_t* fp_out, unsigned* err, cudaStream_t stream) {
+  // Resident warps per SM at this kernel's register count (queried once per
+  // device).
+  static std::atomic<int> per_device[kMaxDeviceOrdinals];
+  const int dev = device_ordinal();
+  int warps_per_sm = dev >= 0 ? per_device[dev].load() : 0;
+  if (warps_per_sm == 0) {
+    int blocks = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &blocks, fingerprint_kernel<VB, K, NB, MASK, HEAD>, kFpThreads, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "fingerprint occupancy");
+    warps_per_sm = blocks > 0 ? blocks * (kFpThreads / 32) : 8;
+    if (dev >= 0) per_device[dev].store(warps_per_sm);
   }
+  const int64_t sms = num_sms();
+  const int64_t warps_target = sms * warps_per_sm;
+  int64_t rpw = (n + warps_target - 1) / warps_target;
+  if (rpw < 32) rpw = 32;
+  const int64_t warps = (n + rpw - 1) / rpw;
+  // Few warps: one-warp blocks, so they spread over all SMs.
+  const int threads = warps >= sms * 8 ? kFpThreads : 32;
+  const int64_t blocks = (warps * 32 + threads - 1) / threads;
+  launch_pdl(fingerprint_kernel<VB, K, NB, MASK, HEAD>, dim3((unsigned)blocks), dim3(threads), 0, stream,
+             tokens, n, stride, lens, seed, fp_out, rpw, err);
+  count_launches(1);
+  return cuda_fail(cudaGetLastError(), "fingerprint launch");
 }
-
-// ---- word path (tokens not 16-byte aligned, or row_stride % 4 != 0) -------------------
-__global__ void __launch_bounds__(256) fingerprint_words_kernel(
-    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
-    const int32_t* __restrict__ lens, uint64_t seed, uint64_t* __restrict__ fp_out,
-    int64_t rows_per_warp, unsigned* err) {
-  pdl_wait();
-  pdl_trigger();
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t r_begin = warp * rows_per_warp;
-  if (r_begin >= n) return;
-  const int64_t r_end = min(n, r_begin + rows_per_warp);
-  const uint32_t seed_lo = (uint32_t)seed, seed_hi = (uint32_t)(seed >> 32);
-  bool busy = false;
-  int64_t row = 0;
-  int32_t len = 0, pos = 0;
-  uint32_t lo = seed_lo, hi = seed_hi;
-  const int32_t* src = tokens;
-  int64_t next = r_begin;
-  const uint32_t lane = threadIdx.x & 31u;
-  int64_t wbase = r_begin;
-  auto len_of = [&](int64_t r) -> int32_t {
-    return r < r_end ? (lens ? __ldg(lens + r) : stride) : 0;
-  };
-  int32_t len_a = len_of(wbase + lane), len_b = len_of(wbase + 32 + lane);
-  for (;;) {
-    unsigned idle = __ballot_sync(0xffffffffu, !busy);
-    while (idle != 0u && next < r_end) {
-      const int64_t avail = r_end - next;
-      const int rank = __popc(idle & lanemask_lt());
-      const int off = (int)(next - wbase) + (!busy ? rank : 0);
-      const int32_t La = __shfl_sync(0xffffffffu, len_a, off & 31);
-      const int32_t Lb = __shfl_sync(0xffffffffu, len_b, off & 31);
-      if (!busy && rank < avail) {
-        const int64_t r = next + rank;
-        const int32_t L = off < 32 ? La : Lb;
-        if (L < 0 || L > stride) {
-          set_error(err, kErrInvalidArg);
-          fp_out[r] = 0ull;
-        } else if (L == 0) {
-          fp_out[r] = seed;
-        } else {
-          row = r;
-          pos = 0;
-          len = L;
-          lo = seed_lo;
-          hi = seed_hi;
-          src = tokens + r * (int64_t)stride;
-          busy = true;
-        }
-      }
-      next += min((int64_t)__popc(idle), avail);
-      if (next - wbase >= 32) {
-        wbase += 32;
-        len_a = len_b;
-        len_b = len_of(wbase + 32 + lane);
-      }
-      idle = __ballot_sync(0xffffffffu, !busy);
-    }
-    if (!__any_sync(0xffffffffu, busy)) break;
-    if (busy) {
-      const int32_t rem = len - pos;
-      const int32_t m = rem < 16 ? rem : 16;
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (j < m) hash_word(lo, hi, (uint32_t)__ldg(src + pos + j));
-      pos += m;
-      if (pos >= len) {
-        fp_out[row] = ((uint64_t)hi << 32) | lo;
-        busy = false;
-      }
-    }
-  }
-}
-
 
 template <int VB, int K, int NB>
 hs_status launch_chunks(const int32_t* tokens, int64_t n, int32_t stride, const int32_t* lens,
@@ -325,7 +434,7 @@ hs_status launch_fingerprint_chunks(const int32_t* tokens, int64_t n, int32_t st
                                     const int32_t* lens, uint64_t seed, uint64_t* fp_out,
                                     bool* ran, cudaStream_t stream) {
   *ran = false;
-  if (stride < kTailChunk) return HS_OK;
+  if (stride < kChunk) return HS_OK;
   const bool vec32 = (reinterpret_cast<uintptr_t>(tokens) & 31u) == 0 && stride % 8 == 0;
   const int64_t sms = num_sms();
   const hs_status st =
@@ -335,40 +444,20 @@ hs_status launch_fingerprint_chunks(const int32_t* tokens, int64_t n, int32_t st
   return st;
 }
 
+// 32-byte loads where every row starts on such a boundary, else 16-byte loads.
 hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
                              const int32_t* lens, uint64_t seed, uint64_t* fp_out,
                              cudaStream_t stream) {
-  const uintptr_t base = reinterpret_cast<uintptr_t>(tokens);
-  const bool vec32 = (base & 31u) == 0 && stride % 8 == 0;
-  const bool vec16 = (base & 15u) == 0 && stride % 4 == 0;
   unsigned* err = device_error_word();
   if (!err) return fail(HS_ERR_CUDA, "could not resolve the device error word");
-  const int64_t sms = num_sms();
-  if (vec16) {
-    if (stride >= kTailChunk) {
-      const hs_status st =
-          vec32 ? launch_chunks<32, 4, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream)
-                : launch_chunks<16, 8, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream);
-      if (st != HS_OK) return st;
-    }
-    if (lens || stride % kTailChunk != 0 || stride == 0) {
-      int64_t blocks = (n + 255) / 256;
-      if (blocks > sms * 64) blocks = sms * 64;
-      launch_pdl(fingerprint_tails_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, tokens, n,
-                 stride, lens, seed, fp_out, err);
-      count_launches(1);
-    }
-  } else {
-    const int64_t warps_target = sms * 32;
-    int64_t rpw = (n + warps_target - 1) / warps_target;
-    if (rpw < 32) rpw = 32;
-    const int64_t warps = (n + rpw - 1) / rpw;
-    const int64_t blocks = (warps + 7) / 8;
-    launch_pdl(fingerprint_words_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, tokens, n,
-               stride, lens, seed, fp_out, rpw, err);
-    count_launches(1);
-  }
-  return cuda_fail(cudaGetLastError(), "fingerprint launch");
+  const uintptr_t base = reinterpret_cast<uintptr_t>(tokens);
+  const bool whole = !lens && stride % kChunk == 0 && stride > 0;   // no masks needed
+  if ((base & 31u) == 0 && stride % 8 == 0)
+    return whole ? launch_rows<32, 4, 2, false, false>(tokens, n, stride, lens, seed, fp_out, err, stream)
+                 : launch_rows<32, 4, 2, true, false>(tokens, n, stride, lens, seed, fp_out, err, stream);
+  if ((base & 15u) == 0 && stride % 4 == 0)
+    return launch_rows<16, 8, 2, true, false>(tokens, n, stride, lens, seed, fp_out, err, stream);
+  return launch_rows<16, 8, 2, true, true>(tokens, n, stride, lens, seed, fp_out, err, stream);
 }
 
 }  // namespace hs

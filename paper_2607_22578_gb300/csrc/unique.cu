@@ -27,6 +27,7 @@
 // its share of the rows, and the last CTA to finish resolves the collision
 // list, scans and writes the outputs.
 #include <mutex>
+#include <type_traits>
 
 #include "fnv.cuh"
 #include "hs_internal.cuh"
@@ -342,34 +343,6 @@ __global__ void __launch_bounds__(256) insert_kernel(const uint64_t* __restrict_
   }
 }
 
-template <bool VEC>
-__global__ void __launch_bounds__(256) verify_kernel(
-    const uint64_t* __restrict__ fp, int64_t n, const uint64_t* __restrict__ keys,
-    const uint32_t* __restrict__ idx, int log2T, const int32_t* __restrict__ tokens,
-    int32_t stride, const int32_t* __restrict__ lens, int32_t* __restrict__ rep,
-    int32_t* coll_list, uint32_t* ctr, unsigned* err) {
-  pdl_wait();
-  pdl_trigger();
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int64_t p0 = w * 32; p0 < n; p0 += warps * 32) {
-    const int64_t a = p0 + lane;
-    const bool valid = a < n;
-    int64_t r = a;
-    if (valid) {
-      const uint32_t v = idx[find_key(keys, __ldg(fp + a), log2T)];
-      if (v < (uint32_t)n) r = v;
-      else set_error(err, kErrInvalidArg);   // not reached: every row was inserted
-    }
-    const bool merged = verify_warp<VEC>(tokens, stride, lens, valid, a, r, err);
-    if (valid) {
-      rep[a] = merged ? (int32_t)r : -1;
-      if (!merged) coll_list[atomicAdd(ctr + kCtrColl, 1u)] = (int32_t)a;
-    }
-  }
-}
-
 // The collision list, after verify: the table is free again (verify was its
 // last reader) and so is uid (the scan writes it next), which holds list2.
 template <bool VEC>
@@ -532,23 +505,33 @@ __global__ void __launch_bounds__(256) finalize_kernel(const int32_t* __restrict
 // Verify of 32 consecutive rows per warp against their representatives (the
 // table's smallest row with the same fingerprint).  The rows that need a
 // comparison (representative another row, lengths equal) are compared as
-// one flat list of 16-byte piece pairs: the warp's pairs are laid end to
-// end (a prefix sum of their piece counts in shared memory), and each lane
-// takes every 32nd piece pair, kVerifyPieces of them in flight per round,
-// so a warp's rows cost about (their bytes / 4 KB) round trips whatever
-// their lengths.  The tokens of a pair's last piece past its length are
-// masked.  Needs 16-byte aligned rows (stride % 4 == 0).  Verifies rows
-// [row0, row_end) of n (row indices, the table and rep are global).
-constexpr int kVerifyPieces = 4;
+// one flat list of piece pairs: the warp's pairs are laid end to end (a
+// prefix sum of their piece counts in shared memory), and each lane takes
+// every 32nd piece pair, kPieces of them in flight per round, so a warp's
+// rows cost about as many round trips as their bytes need whatever their
+// lengths.  VEC: pieces of 16 bytes (16-byte aligned rows, stride % 4 == 0),
+// the tokens of a pair's last piece past its length masked.  Otherwise the
+// rows may start on any word and a piece is one word, coalesced over the
+// lanes, with twice as many in flight: 20,011 rows at a stride of 333, a third
+// of them copies, take 21 us cold (40 us as two rows per warp round).
 constexpr int kVerifyThreads = 256;
 
+// Do the first `live` tokens of two 16-byte pieces, or two words, differ?
+__device__ __forceinline__ bool piece_differs(const uint4& x, const uint4& y, int live) {
+  return (x.x != y.x) | ((live > 1) & (x.y != y.y)) | ((live > 2) & (x.z != y.z)) |
+         ((live > 3) & (x.w != y.w));
+}
+__device__ __forceinline__ bool piece_differs(uint32_t x, uint32_t y, int) { return x != y; }
+
+template <bool VEC>
 __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
-    const uint64_t* __restrict__ fp, uint64_t key_mask, int64_t n, int64_t row0, int64_t row_end,
+    const uint64_t* __restrict__ fp, uint64_t key_mask, int64_t n,
     const uint64_t* __restrict__ keys, const uint32_t* __restrict__ idx, int log2T,
     const int32_t* __restrict__ tokens, int32_t stride, const int32_t* __restrict__ lens,
     int32_t* __restrict__ rep, int32_t* coll_list, uint32_t* ctr, unsigned* err) {
   pdl_wait();
   pdl_trigger();
+  constexpr int kPieces = VEC ? 4 : 8;
   __shared__ int32_t s_pre[kVerifyThreads / 32][32];
   __shared__ int32_t s_a[kVerifyThreads / 32][32];
   __shared__ int32_t s_b[kVerifyThreads / 32][32];
@@ -556,9 +539,9 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int64_t p0 = row0 + w * 32; p0 < row_end; p0 += warps * 32) {
+  for (int64_t p0 = w * 32; p0 < n; p0 += warps * 32) {
     const int64_t a = p0 + lane;
-    const bool valid = a < row_end;
+    const bool valid = a < n;
     int64_t r = a;
     int32_t la = 0, lr = 0;
     if (valid) {
@@ -569,7 +552,9 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
       lr = r != a ? clamp_len(lens, r, stride, err) : la;
     }
     const bool need = valid && r != a && la == lr;
-    int32_t incl = need ? (la + 3) >> 2 : 0;
+    // The list's length fits 32 bits: this path takes more than 4096 rows,
+    // so 32 of them hold less than 2^31 words in any memory there is.
+    int32_t incl = need ? (VEC ? (la + 3) >> 2 : la) : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -583,30 +568,26 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
     __syncwarp();
     uint32_t differ = 0;                       // bit t: a piece of pair t differs
     int t = 0;                                 // this lane's current pair (only moves forward)
-    for (int32_t g0 = 0; g0 < total; g0 += 32 * kVerifyPieces) {
-      uint4 x[kVerifyPieces], y[kVerifyPieces];
-      int tt[kVerifyPieces], vt[kVerifyPieces];
+    for (int32_t g0 = 0; g0 < total; g0 += 32 * kPieces) {
+      using Piece = typename std::conditional<VEC, uint4, uint32_t>::type;
+      Piece x[kPieces], y[kPieces];
+      int tt[kPieces], vt[kPieces];
 #pragma unroll
-      for (int u = 0; u < kVerifyPieces; ++u) {
+      for (int u = 0; u < kPieces; ++u) {
         const int32_t g = g0 + u * 32 + lane;
         tt[u] = -1;
         if (g < total) {
           while (s_pre[wl][t] <= g) ++t;
           const int32_t j = g - (t > 0 ? s_pre[wl][t - 1] : 0);
-          x[u] = __ldg(reinterpret_cast<const uint4*>(tokens + (int64_t)s_a[wl][t] * stride) + j);
-          y[u] = __ldg(reinterpret_cast<const uint4*>(tokens + (int64_t)s_b[wl][t] * stride) + j);
+          x[u] = __ldg(reinterpret_cast<const Piece*>(tokens + (int64_t)s_a[wl][t] * stride) + j);
+          y[u] = __ldg(reinterpret_cast<const Piece*>(tokens + (int64_t)s_b[wl][t] * stride) + j);
           tt[u] = t;
-          vt[u] = s_len[wl][t] - 4 * j;        // live tokens in this piece (>= 1)
+          vt[u] = s_len[wl][t] - 4 * j;        // VEC: live tokens in this piece (>= 1)
         }
       }
 #pragma unroll
-      for (int u = 0; u < kVerifyPieces; ++u) {
-        if (tt[u] >= 0) {
-          const bool d = (x[u].x != y[u].x) | ((vt[u] > 1) & (x[u].y != y[u].y)) |
-                         ((vt[u] > 2) & (x[u].z != y[u].z)) | ((vt[u] > 3) & (x[u].w != y[u].w));
-          if (d) differ |= 1u << tt[u];
-        }
-      }
+      for (int u = 0; u < kPieces; ++u)
+        if (tt[u] >= 0 && piece_differs(x[u], y[u], vt[u])) differ |= 1u << tt[u];
     }
     differ = __reduce_or_sync(0xffffffffu, differ);
     __syncwarp();                              // shared lists free for the next rows
@@ -874,14 +855,10 @@ hs_status launch_unique_inverse(const uint64_t* fp, const int32_t* tokens, int64
   if (e != cudaSuccess) return cuda_fail(e, "hash table clear");
   launch_pdl(insert_kernel, dim3(grid_for(n, 256, sms * 8)), dim3(256), 0, stream, fp, n, keys, idx,
              L.log2T);
-  const unsigned vgrid = grid_for(n, 256, sms * 8);   // one warp per 32 rows
-  if (vec)
-    launch_pdl(verify_flat_kernel, dim3(vgrid), dim3(kVerifyThreads), 0, stream, fp, ~0ull, n,
-               (int64_t)0, n, (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens,
-               stride, lens, rep, coll_list, ctr, err);
-  else
-    launch_pdl(verify_kernel<false>, dim3(vgrid), dim3(256), 0, stream, fp, n, keys, idx, L.log2T,
-               tokens, stride, lens, rep, coll_list, ctr, err);
+  launch_pdl(vec ? verify_flat_kernel<true> : verify_flat_kernel<false>,
+             dim3(grid_for(n, kVerifyThreads, sms * 8)), dim3(kVerifyThreads), 0, stream, fp,
+             ~0ull, n, (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride, lens,
+             rep, coll_list, ctr, err);
   if (vec)
     launch_pdl(resolve_kernel<true>, dim3(1), dim3(kResolveThreads), 0, stream, fp, tokens, stride,
                lens, rep, coll_list, ctr, keys, idx, uid, err);
@@ -944,8 +921,8 @@ hs_status launch_merge_rows(const int32_t* tokens, int64_t n, int32_t stride, co
   if (st != HS_OK) return st;
   launch_pdl(tails_insert_kernel, dim3(grid_for(n, 256, sms * 16)), dim3(256), 0, stream, tokens,
              (int64_t)0, n, stride, lens, seed, ran, mask, fp_out, keys, idx, L.log2T, err);
-  launch_pdl(verify_flat_kernel, dim3(grid_for(n, kVerifyThreads, sms * 8)), dim3(kVerifyThreads),
-             0, stream, (const uint64_t*)fp_out, mask, n, (int64_t)0, n, (const uint64_t*)keys,
+  launch_pdl(verify_flat_kernel<true>, dim3(grid_for(n, kVerifyThreads, sms * 8)),
+             dim3(kVerifyThreads), 0, stream, (const uint64_t*)fp_out, mask, n, (const uint64_t*)keys,
              (const uint32_t*)idx, L.log2T, tokens, stride, lens, rep, coll_list, ctr, err);
   launch_pdl(resolve_kernel<true>, dim3(1), dim3(kResolveThreads), 0, stream,
              (const uint64_t*)fp_out, tokens, stride, lens, rep, (const int32_t*)coll_list,

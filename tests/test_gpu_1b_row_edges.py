@@ -1,0 +1,85 @@
+"""Fingerprints (Section 3.3, Eq. 2) and the exact merge (Section 3.3 (I)) at
+the edges of the 32-token chunks and 16-byte pieces: every word offset of a
+row's start, lengths around them, both ends of the token array, tokens above
+and below 65536."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_22578_gb300 as hs
+from hs_testutil import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def rows_at(offset, n, stride, rng, big):
+    """n rows whose first word lies `offset` words past a 256-byte boundary,
+    in an array with nothing after its last word."""
+    flat = rng.integers(0, 1 << 31 if big else 65536, size=offset + n * stride).astype(np.int32)
+    dev = to_dev(flat)
+    return flat[offset:].reshape(n, stride), dev[offset:].view(n, stride)
+
+
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("stride", [1, 3, 4, 7, 8, 31, 32, 33, 36, 63, 64, 65, 96, 333])
+def test_fingerprint_at_every_offset(stride, big):
+    rng = np.random.default_rng(stride + big)
+    for offset in range(9):
+        tokens, dev = rows_at(offset, 77, stride, rng, big)
+        lens = rng.integers(0, stride + 1, size=77).astype(np.int32)
+        lens[[0, 76]] = stride                       # the array's first and last words
+        for L in (None, lens):
+            for seed in (hs.HS_FNV64_OFFSET_BASIS, 0x0123456789ABCDEF):
+                fp = hs.hs_fingerprint(dev, None if L is None else to_dev(L), seed)
+                hs.hs_get_device_error()
+                want = oracle.fingerprint(tokens, L, seed=seed)
+                assert (fp.cpu().numpy().view(np.uint64) == want).all(), (offset, L is None)
+
+
+def test_fingerprint_mixes_small_and_large_tokens_and_bad_lengths():
+    rng = np.random.default_rng(9)
+    tokens, dev = rows_at(2, 5000, 75, rng, False)
+    tokens = tokens.copy()
+    tokens[rng.random(tokens.shape) < 0.01] = -1     # some chunks take the octet-wise rounds
+    dev.copy_(to_dev(tokens))
+    lens = rng.integers(0, 76, size=5000).astype(np.int32)
+    want = oracle.fingerprint(tokens, lens)
+    bad = lens.copy()
+    bad[[0, 31, 4999]] = [-1, 76, 1 << 30]
+    fp = hs.hs_fingerprint(dev, to_dev(bad))
+    with pytest.raises(hs.HsError) as e:
+        hs.hs_get_device_error()
+    assert e.value.status == hs.HS_ERR_INVALID_ARG
+    want[[0, 31, 4999]] = 0
+    assert (fp.cpu().numpy().view(np.uint64) == want).all()
+
+
+@pytest.mark.parametrize("stride", [1, 5, 33, 127, 130])
+def test_merge_of_rows_on_any_word(stride):
+    rng = np.random.default_rng(stride)
+    n = 4097 + stride
+    for offset in (0, 1, 3):
+        tokens, dev = rows_at(offset, n, stride, rng, True)
+        tokens = tokens.copy()
+        src = rng.integers(0, n, size=n)
+        copy = rng.random(n) < 0.5
+        tokens[copy] = tokens[src[copy]]
+        near = rng.integers(0, n, size=n // 8)       # rows that differ in one word only
+        tokens[near] = tokens[0]
+        tokens[near, rng.integers(0, stride, size=len(near))] ^= 1 << 20
+        dev.copy_(to_dev(tokens))
+        lens = np.where(rng.random(n) < 0.5, stride, rng.integers(0, stride + 1, size=n))
+        lens = lens.astype(np.int32)
+        for L in (None, lens):
+            d = None if L is None else to_dev(L)
+            ou, oi = oracle.unique_inverse(tokens, L)
+            fp, nu, u, i = hs.hs_merge_rows(dev, d)
+            nu2, u2, i2 = hs.hs_unique_inverse(fp, dev, d)
+            hs.hs_get_device_error()
+            assert (fp.cpu().numpy().view(np.uint64) == oracle.fingerprint(tokens, L)).all()
+            for count, uniq, inv in ((nu, u, i), (nu2, u2, i2)):
+                assert int(count.item()) == len(ou)
+                assert (uniq.cpu().numpy()[:len(ou)] == ou).all()
+                assert (uniq.cpu().numpy()[len(ou):] == 0).all()
+                assert (inv.cpu().numpy() == oi).all()

@@ -47,6 +47,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True) -> ctypes.CDLL:
     """Load libhs.so (building it first if it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if build_if_missing:
@@ -120,8 +122,16 @@ def _check(status: int) -> None:
         raise HsError(status, load().hs_last_error().decode())
 
 
+# The current stream's handle without a Stream object: 0.2 us of a call's host
+# time where torch.cuda.current_stream() takes 2.9.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
@@ -138,6 +148,11 @@ def _cuda(t: torch.Tensor, name: str) -> torch.Tensor:
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
     return t
+
+
+def _rows(t: torch.Tensor, n: int) -> torch.Tensor:
+    """The first n rows of t: t itself where it has no more."""
+    return t if t.shape[0] == n else t[:n]
 
 
 def hs_version() -> str:
@@ -183,13 +198,12 @@ def hs_unique_inverse(fp: torch.Tensor, tokens: torch.Tensor, lens: torch.Tensor
                torch.empty(max(n, 1), dtype=torch.int32, device=dev),
                torch.empty(max(n, 1), dtype=torch.int32, device=dev))
     nu, uidx, inv = out
-    need = hs_unique_inverse_workspace(n)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
+        workspace = torch.empty(hs_unique_inverse_workspace(n), dtype=torch.uint8, device=dev)
     _check(load().hs_unique_inverse(_ptr(fp), _ptr(tokens), n, stride, _ptr(lens), _ptr(nu),
                                     _ptr(uidx), _ptr(inv), _ptr(workspace), workspace.numel(),
                                     _stream(stream)))
-    return nu, uidx[:n], inv[:n]
+    return nu, _rows(uidx, n), _rows(inv, n)
 
 
 def hs_merge_rows_workspace(n_rows: int) -> int:
@@ -211,13 +225,12 @@ def hs_merge_rows(tokens: torch.Tensor, lens: torch.Tensor | None = None,
                torch.empty(max(n, 1), dtype=torch.int32, device=dev),
                torch.empty(max(n, 1), dtype=torch.int32, device=dev))
     fp, nu, uidx, inv = out
-    need = hs_merge_rows_workspace(n)
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
+        workspace = torch.empty(hs_merge_rows_workspace(n), dtype=torch.uint8, device=dev)
     _check(load().hs_merge_rows(_ptr(tokens), n, stride, _ptr(lens), int(seed_state), _ptr(fp),
                                 _ptr(nu), _ptr(uidx), _ptr(inv), _ptr(workspace),
                                 workspace.numel(), _stream(stream)))
-    return fp[:n], nu, uidx[:n], inv[:n]
+    return _rows(fp, n), nu, _rows(uidx, n), _rows(inv, n)
 
 
 def hs_debug_merge_key_mask(mask: int = 0) -> None:
@@ -266,7 +279,7 @@ def hs_unique_inverse_noalloc(fp: torch.Tensor, tokens: torch.Tensor,
     nu, uidx, inv = out
     _check(load().hs_unique_inverse_noalloc(_ptr(fp), _ptr(tokens), n, stride, _ptr(lens),
                                             _ptr(nu), _ptr(uidx), _ptr(inv), _stream(stream)))
-    return nu, uidx[:n], inv[:n]
+    return nu, _rows(uidx, n), _rows(inv, n)
 
 
 def hs_retrieve_topk_workspace(n_queries: int, n_corpus: int, dim: int, k: int) -> int:
@@ -396,7 +409,7 @@ def hs_merge_queries(queries: torch.Tensor, seed_state: int = HS_FNV64_OFFSET_BA
     _check(load().hs_merge_queries(_ptr(queries), n, d, seed_state & (2**64 - 1), _ptr(fp_in),
                                    _ptr(fp), _ptr(nu), _ptr(uidx), _ptr(inv), _ptr(uq),
                                    _stream(stream)))
-    return fp[:n], nu, uidx[:n], inv[:n], uq[:n]
+    return _rows(fp, n), nu, _rows(uidx, n), _rows(inv, n), _rows(uq, n)
 
 
 def hs_scatter_results(src: torch.Tensor, mapping: torch.Tensor, dst: torch.Tensor | None = None,
@@ -407,7 +420,11 @@ def hs_scatter_results(src: torch.Tensor, mapping: torch.Tensor, dst: torch.Tens
     if mapping.dtype != torch.int32:
         raise TypeError("map must be int32")
     n = mapping.numel()
-    row_bytes = src[0].numel() * src.element_size() if src.dim() > 1 else src.element_size()
+    row_bytes = src.element_size()
+    if src.dim() > 1:
+        if src.shape[0] == 0:
+            raise IndexError("src has no rows")
+        row_bytes *= src.numel() // src.shape[0]
     if dst is None:
         dst = torch.empty((n,) + tuple(src.shape[1:]), dtype=src.dtype, device=src.device)
     _check(load().hs_scatter_results(_ptr(src), src.shape[0], row_bytes, _ptr(mapping), n,
@@ -548,7 +565,7 @@ def hs_segment_sum(phi: torch.Tensor, inverse: torch.Tensor, max_groups: int,
         out = torch.empty(max(int(max_groups), 1), dtype=torch.float64, device=phi.device)
     _check(load().hs_segment_sum(_ptr(phi), _ptr(inverse), phi.numel(), _ptr(n_groups_dev),
                                  int(max_groups), _ptr(out), _stream(stream)))
-    return out[: int(max_groups)]
+    return _rows(out, int(max_groups))
 
 
 def hs_launch_count() -> int:

@@ -79,6 +79,22 @@ class EmbedRetrieveStage:
                                     device=dev)
             self.r_scores = torch.empty((mq, self.rerank_k), dtype=torch.float32, device=dev)
             self.r_ids = torch.empty((mq, self.rerank_k), **i32)
+        self._views = {}
+
+    def _first(self, name: str, n: int):
+        """The first n rows of the buffers `name` (an attribute: a tensor or a
+        tuple of them).  Views of the last few batch sizes are kept: a slice
+        is 1.1 us of host time, and a cached batch takes about twenty.  They
+        stay inside the stage: what a call returns is a slice of its own."""
+        key = (name, n)
+        v = self._views.get(key)
+        if v is None:
+            if len(self._views) >= 256:
+                self._views.clear()
+            b = getattr(self, name)
+            v = tuple(t[:n] for t in b) if isinstance(b, tuple) else b[:n]
+            self._views[key] = v
+        return v
 
     def capture(self, tokens: torch.Tensor, queries: torch.Tensor,
                 lens: torch.Tensor | None = None) -> "StepGraph":
@@ -88,10 +104,14 @@ class EmbedRetrieveStage:
     def dedup_chunks(self, tokens: torch.Tensor, lens: torch.Tensor | None = None):
         """Fingerprint + exact unique of chunk rows.  Returns (n_unique_dev,
         unique_idx, inverse, fp) as device tensors."""
+        return self._dedup_chunks(tokens, lens, None)
+
+    def _dedup_chunks(self, tokens, lens, stream):
         n = tokens.shape[0]
         nu_b, uidx_b, inv_b = self.c_out
         fp, nu, uidx, inv = _lib.hs_merge_rows(
-            tokens, lens, workspace=self.ws_c, out=(self.c_fp[:n], nu_b, uidx_b[:n], inv_b[:n]))
+            tokens, lens, workspace=self.ws_c, out=(self.c_fp[:n], nu_b, uidx_b[:n], inv_b[:n]),
+            stream=stream)
         return nu, uidx, inv, fp
 
     def retrieve(self, queries: torch.Tensor, events: tuple | None = None):
@@ -110,19 +130,20 @@ class EmbedRetrieveStage:
         """Lookup of the merged queries, retrieval of the misses only, insert
         of their results, fan-out to every query."""
         Q = inv.shape[0]
-        fp, uidx = self.q_fp[:Q], self.q_out[1][:Q]
-        out = (self.c_s[:Q], self.c_i[:Q])
-        miss = (self.miss[0][:Q], self.miss[1], self.miss[2][:Q])
+        fp, uidx = self._first("q_fp", Q), self._first("q_out", Q)[1]
+        out = (self._first("c_s", Q), self._first("c_i", Q))
+        m_s, m_i = self._first("m_s", Q), self._first("m_i", Q)
+        first = self._first("miss", Q)
+        miss = (first[0], self.miss[1], first[2])
         _lib.hs_cache_lookup(self.cache, uq, fp, fp_rows=uidx, n_queries_dev=nu, out=out,
                              miss=miss)
         if events is not None:
             events[0].record()
         _lib.hs_retrieve_topk_n(miss[2], miss[1], self.corpus, self.k, workspace=self.ws_r,
-                                out=(self.m_s[:Q], self.m_i[:Q]))
+                                out=(m_s, m_i))
         if events is not None:
             events[1].record()
-        _lib.hs_cache_insert(self.cache, miss, fp, self.m_s[:Q], self.m_i[:Q], out,
-                             fp_rows=uidx)
+        _lib.hs_cache_insert(self.cache, miss, fp, m_s, m_i, out, fp_rows=uidx)
         scores = _lib.hs_scatter_results(out[0], inv, dst=self.scores[:Q])
         ids = _lib.hs_scatter_results(out[1], inv, dst=self.ids[:Q])
         return scores, ids
@@ -143,11 +164,12 @@ class EmbedRetrieveStage:
         if Q > self.max_queries or rerank_queries.shape[0] != Q:
             raise ValueError("batch larger than max_queries or rerank rows differ")
         nu, inv, uq = self._merge_queries(queries)
-        uidx = self.q_out[1][:Q]
+        uidx = self._first("q_out", Q)[1]
+        i_u = self._first("i_u", Q)
         _lib.hs_retrieve_topk_n(uq, nu, self.corpus, self.k, workspace=self.ws_r,
-                                out=(self.s_u[:Q], self.i_u[:Q]))
-        rq = _lib.hs_scatter_results(rerank_queries, uidx, dst=self.rq_u[:Q])
-        scores, ids = _lib.hs_rerank_topk(rq, self.rerank_corpus, self.i_u[:Q], self.rerank_k,
+                                out=(self._first("s_u", Q), i_u))
+        rq = _lib.hs_scatter_results(rerank_queries, uidx, dst=self._first("rq_u", Q))
+        scores, ids = _lib.hs_rerank_topk(rq, self.rerank_corpus, i_u, self.rerank_k,
                                           n_queries_dev=nu, inverse=inv,
                                           out=(self.r_scores[:Q], self.r_ids[:Q]))
         return scores, ids, nu
@@ -156,15 +178,17 @@ class EmbedRetrieveStage:
         """Merged query nodes of a batch: (n_unique_dev, inverse, unique
         query rows)."""
         Q = queries.shape[0]
-        nu_b, uidx_b, inv_b = self.q_out
+        nu_b = self.q_out[0]
+        _, uidx_b, inv_b = self._first("q_out", Q)
+        fp_b, uq_b = self._first("q_fp", Q), self._first("uq", Q)
         if Q <= _lib.HS_MERGE_QUERIES_MAX:
-            _, nu, _, inv, uq = _lib.hs_merge_queries(
-                queries, out=(self.q_fp[:Q], nu_b, uidx_b[:Q], inv_b[:Q], self.uq[:Q]))
+            _, nu, _, inv, uq = _lib.hs_merge_queries(queries,
+                                                      out=(fp_b, nu_b, uidx_b, inv_b, uq_b))
             return nu, inv, uq
         qi32 = queries.view(torch.int32)
-        _, nu, uidx, inv = _lib.hs_merge_rows(
-            qi32, workspace=self.ws_q, out=(self.q_fp[:Q], nu_b, uidx_b[:Q], inv_b[:Q]))
-        uq = _lib.hs_scatter_results(queries, uidx, dst=self.uq[:Q])
+        _, nu, uidx, inv = _lib.hs_merge_rows(qi32, workspace=self.ws_q,
+                                              out=(fp_b, nu_b, uidx_b, inv_b))
+        uq = _lib.hs_scatter_results(queries, uidx, dst=uq_b)
         return nu, inv, uq
 
     def _retrieve_merged(self, uq, nu, inv, events):
@@ -194,8 +218,7 @@ class EmbedRetrieveStage:
             self._join = torch.cuda.Event()
         self._fork.record(main)
         self._side.wait_event(self._fork)
-        with torch.cuda.stream(self._side):
-            chunk = self.dedup_chunks(tokens, lens)
+        chunk = self._dedup_chunks(tokens, lens, self._side)
         self._join.record(self._side)
         if queries.shape[0] > self.max_queries:
             raise ValueError("batch larger than max_queries")

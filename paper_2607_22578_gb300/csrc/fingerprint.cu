@@ -5,7 +5,9 @@
 // from rows: each lane of a warp owns one row at a time and hashes it in
 // chunks of 32 tokens, straight-line from registers.
 // The octet rounds themselves are in fnv.cuh.
-#include "fnv.cuh"
+#include <algorithm>
+
+#include "fnv_warp.cuh"
 #include "hs_internal.cuh"
 
 namespace hs {
@@ -64,11 +66,9 @@ struct Unpad {
   uint64_t v[kChunk + 1];
 };
 constexpr Unpad make_unpad() {
-  uint64_t inv = kPrime;                       // x = inv solves x * prime = 1 (mod 8)
-  for (int i = 0; i < 5; ++i) inv *= 2 - kPrime * inv;   // Newton: the exact bits double
   Unpad u{};
   u.v[0] = 1;
-  for (int t = 1; t <= kChunk; ++t) u.v[t] = u.v[t - 1] * inv * inv * inv * inv;
+  for (int t = 1; t <= kChunk; ++t) u.v[t] = u.v[t - 1] * power(inverse_prime(), 4);
   return u;
 }
 static_assert(make_unpad().v[1] * kPrime * kPrime * kPrime * kPrime == 1, "inverse of the prime");
@@ -244,6 +244,34 @@ __global__ void __launch_bounds__(kFpThreads) fingerprint_kernel(
 #pragma unroll
     for (int b = 0; b < NB; ++b) pending |= brow[b] >= 0;
     if (!__any_sync(0xffffffffu, pending) && next >= r_end) break;
+  }
+}
+
+// ---- few rows: a warp per row -------------------------------------------------------------
+// Bound by the latency of one row, which a warp cuts to eight prefix xors and
+// 32 rounds per 1024 octets (fnv.cuh).  It costs about three times the
+// instructions of a lane per row, so it is for batches that leave most of the
+// GPU idle.  A row of
+// 1536 octets takes 3.5 us with its launch where the chain takes 14.4.
+template <bool VEC>
+__global__ void __launch_bounds__(128) fingerprint_warp_kernel(
+    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
+    const int32_t* __restrict__ lens, uint64_t seed, uint64_t* __restrict__ fp_out,
+    unsigned* err) {
+  pdl_wait();
+  pdl_trigger();
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const int32_t L = lens ? __ldg(lens + r) : stride;
+    const bool bad = L < 0 || L > stride;                  // reported, fingerprint 0
+    uint64_t h = 0;
+    if (!bad)
+      h = hash_row_warp<VEC>(reinterpret_cast<const uint32_t*>(tokens + r * (int64_t)stride), L,
+                             seed);
+    if ((threadIdx.x & 31) == 0) {
+      if (bad) set_error(err, kErrInvalidArg);
+      fp_out[r] = h;
+    }
   }
 }
 
@@ -451,11 +479,27 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
   unsigned* err = device_error_word();
   if (!err) return fail(HS_ERR_CUDA, "could not resolve the device error word");
   const uintptr_t base = reinterpret_cast<uintptr_t>(tokens);
+  const bool vec16 = (base & 15u) == 0 && stride % 4 == 0;
+  // A warp per row takes 0.7 ns per row and 256 tokens at full size; a lane
+  // per row the chain of the longest row, 17 ns per token (33 where rows are
+  // not aligned), while that many lanes fit the GPU.  Measured, us, warp / lane:
+  // 4096 rows of 256 tokens 4.9 / 6.6, 8192 7.4 / 6.6; 2048 of 384 (octet-wise)
+  // 5.1 / 14.4; 2048 of 64 3.1 / 2.8; 1024 of 64 2.7 / 2.7; 8192 of 333 on any
+  // word 13.1 / 18.3, 16384 23.4 / 18.4.
+  const int64_t work = n * (((int64_t)stride + 255) / 256);
+  if (n < (1 << 20) && work <= (vec16 ? 24 : 48) * (int64_t)stride) {
+    const int64_t blocks = (n + 3) / 4;
+    launch_pdl(vec16 ? fingerprint_warp_kernel<true> : fingerprint_warp_kernel<false>,
+               dim3((unsigned)std::min<int64_t>(blocks, num_sms() * 64)), dim3(128), 0, stream,
+               tokens, n, stride, lens, seed, fp_out, err);
+    count_launches(1);
+    return cuda_fail(cudaGetLastError(), "fingerprint launch");
+  }
   const bool whole = !lens && stride % kChunk == 0 && stride > 0;   // no masks needed
   if ((base & 31u) == 0 && stride % 8 == 0)
     return whole ? launch_rows<32, 4, 2, false, false>(tokens, n, stride, lens, seed, fp_out, err, stream)
                  : launch_rows<32, 4, 2, true, false>(tokens, n, stride, lens, seed, fp_out, err, stream);
-  if ((base & 15u) == 0 && stride % 4 == 0)
+  if (vec16)
     return launch_rows<16, 8, 2, true, false>(tokens, n, stride, lens, seed, fp_out, err, stream);
   return launch_rows<16, 8, 2, true, true>(tokens, n, stride, lens, seed, fp_out, err, stream);
 }

@@ -37,6 +37,23 @@ def test_fingerprint_at_every_offset(stride, big):
                 assert (fp.cpu().numpy().view(np.uint64) == want).all(), (offset, L is None)
 
 
+@pytest.mark.parametrize("big", [False, True])
+@pytest.mark.parametrize("stride", [1, 8, 33, 255, 256, 257, 513, 1280])
+def test_fingerprint_on_both_sides_of_the_row_count(stride, big):
+    """Few rows are hashed by a warp each (1024 octets at a time), many by a
+    lane each."""
+    rng = np.random.default_rng(stride + big)
+    for offset, n in ((0, 1), (0, 33), (1, 33), (0, 13000), (3, 13000)):
+        tokens, dev = rows_at(offset, n, stride, rng, big)
+        lens = rng.integers(0, stride + 1, size=n).astype(np.int32)
+        lens[[0, n - 1]] = stride
+        for L in (None, lens):
+            fp = hs.hs_fingerprint(dev, None if L is None else to_dev(L), 0xFFFFFFFFFFFFFFFF)
+            hs.hs_get_device_error()
+            want = oracle.fingerprint(tokens, L, seed=0xFFFFFFFFFFFFFFFF)
+            assert (fp.cpu().numpy().view(np.uint64) == want).all(), (offset, n)
+
+
 def test_fingerprint_mixes_small_and_large_tokens_and_bad_lengths():
     rng = np.random.default_rng(9)
     tokens, dev = rows_at(2, 5000, 75, rng, False)

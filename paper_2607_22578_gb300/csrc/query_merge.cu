@@ -9,21 +9,30 @@
 // hs_scatter_results(queries, unique_idx) called in turn.
 //
 // Small batches are latency-bound: each of those calls is a few microseconds
-// of launch and dependency latency around very little work.  Here every CTA
-// runs the whole merge on its own — the fingerprints of all rows (one thread
-// per row), the hash table in shared memory, the verification, the scan —
-// so the CTAs never wait for one another, and they split only the final
-// gather.  The redundant work is cheap at these sizes: at most 256 rows,
-// read from L2.  CTA 0 alone writes fingerprints, unique_idx, inverse and the
-// unique count.
+// of launch and dependency latency around very little work.  Here every merging
+// CTA runs the whole merge on its own — a key of every row, the hash table in
+// shared memory, the verification, the scan — so the CTAs never wait for one
+// another, and they split only the final gather.  The redundant work is cheap
+// at these sizes: at most 256 rows, read from L2.  CTA 0 alone writes
+// unique_idx, inverse and the unique count.
 //
-// Exactness: rows are grouped by fingerprint (the table keeps the smallest
-// row index per fingerprint), then every row whose group leader is another
-// row is compared with it in full.  A row that differs from its leader (a
-// fingerprint collision) is re-grouped by a warp in ascending row order:
-// its leader is the first earlier row with the same fingerprint that leads
-// its own group and has equal contents, else itself.
-#include "fnv.cuh"
+// The merge does not need the fingerprints, whose hash is the longest chain
+// here (a warp per row, fnv_warp.cuh): its key is a hash of the whole row that
+// a warp takes in one round of loads (multiply-xorshift of each 16-byte piece
+// with its place, added up), and further CTAs of the same launch compute the
+// fingerprints meanwhile.  Given fingerprints are taken as the keys.
+//
+// Bound by the launch and its dependent round trips (keys, verify, gather); at
+// 256 rows of 768 by each CTA's reading of all rows.  us with the launch, where
+// one thread hashed each row first: 1 row of 768 3.6 (15.0), 64 rows 7.0
+// (17.6), 256 rows 16.6 (28.1).  256 threads instead of 512: 64 rows 8.6.
+//
+// Exactness: rows are grouped by key (the table keeps the smallest row index
+// per key), then every row whose group leader is another row is compared with
+// it in full.  A row that differs from its leader (a collision) is re-grouped
+// by a warp in ascending row order: its leader is the first earlier row with
+// the same key that leads its own group and has equal contents, else itself.
+#include "fnv_warp.cuh"
 #include "hs_internal.cuh"
 #include "row_table.cuh"
 
@@ -32,24 +41,47 @@ namespace {
 
 using namespace table;
 
-constexpr int kQmThreads = 256;             // one thread per query row
-constexpr int kQmMaxRows = kQmThreads;
+constexpr int kQmThreads = 512;
+constexpr int kQmMaxRows = 256;             // the first threads take a row each
+static_assert(kQmMaxRows <= kQmThreads && kQmMaxRows >= HS_MERGE_QUERIES_MAX, "a thread per row");
 constexpr int kQmLog2 = table_log2(kQmMaxRows);
 constexpr int kQmSlots = (1 << kQmLog2) + 1;
 constexpr int kQmMaxCtas = 32;
-constexpr int kQmChunk = 8;                 // 16-byte vectors per register chunk (32 words)
+constexpr int kQmRows = 4;                  // rows a group takes side by side for their keys
+constexpr int kQmPieces = 3;                // 16-byte pieces per lane and row in flight
 constexpr int kQmUnroll = 4;                // independent 16-byte copies in flight per thread
 
 __device__ __forceinline__ bool same4(const uint4& a, const uint4& b) {
   return a.x == b.x && a.y == b.y && a.z == b.z && a.w == b.w;
 }
 
+// Hash of one 16-byte piece at place v of its row; a row's key is the sum of
+// its pieces' hashes, so lanes and rounds add up in any order.
+__device__ __forceinline__ uint64_t piece_key(const uint4& x, int v) {
+  constexpr uint64_t kMul = 0x9E3779B97F4A7C15ull, kFin = 0xD6E8FEB86659FD93ull;
+  uint64_t h = ((((uint64_t)x.y << 32) | x.x) ^ ((uint64_t)(v + 1) * kFin)) * kMul;
+  h = (h ^ (h >> 32) ^ (((uint64_t)x.w << 32) | x.z)) * kMul;
+  return h ^ (h >> 29);
+}
+
+// CTAs [0, merge_ctas) merge; the others hash rows (fp_in NULL, fp_out not).
 __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
     const uint4* __restrict__ q, int n, int nv, uint64_t seed, const uint64_t* __restrict__ fp_in,
     uint64_t* __restrict__ fp_out, int32_t* __restrict__ n_unique,
-    int32_t* __restrict__ unique_idx, int32_t* __restrict__ inverse, uint4* __restrict__ uq) {
+    int32_t* __restrict__ unique_idx, int32_t* __restrict__ inverse, uint4* __restrict__ uq,
+    int merge_ctas) {
   pdl_wait();
   pdl_trigger();
+  if ((int)blockIdx.x >= merge_ctas) {
+    const int warps = ((int)gridDim.x - merge_ctas) * (kQmThreads / 32);
+    for (int r = ((int)blockIdx.x - merge_ctas) * (kQmThreads / 32) + (int)(threadIdx.x >> 5);
+         r < n; r += warps) {
+      const uint64_t h = fnv::hash_row_warp<true>(
+          reinterpret_cast<const uint32_t*>(q + (size_t)r * nv), nv * 4, seed);
+      if ((threadIdx.x & 31) == 0) fp_out[r] = h;
+    }
+    return;
+  }
   __shared__ uint64_t s_fp[kQmMaxRows];
   __shared__ uint64_t s_keys[kQmSlots];
   __shared__ uint32_t s_idx[kQmSlots];
@@ -69,45 +101,56 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
     s_keys[s] = kEmpty;
     s_idx[s] = kNoRow;
   }
-  s_diff[tid] = 0;
+  if (tid < kQmMaxRows) s_diff[tid] = 0;
   if (tid == 0) s_nlist = s_ncoll = 0;
 
-  // 1. fingerprint of row tid: FNV-1a over its octets, one chunk of 32 words
-  //    loaded ahead of the chunk being hashed
-  uint64_t f = 0;
-  if (row) {
-    if (fp_in) {
-      f = __ldg(fp_in + tid);
-    } else {
-      const uint4* r = q + (size_t)tid * nv;
-      uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-      uint4 cur[kQmChunk], nxt[kQmChunk];
-#pragma unroll
-      for (int j = 0; j < kQmChunk; ++j) cur[j] = j < nv ? __ldg(r + j) : make_uint4(0, 0, 0, 0);
-      for (int c0 = 0; c0 < nv; c0 += kQmChunk) {
-#pragma unroll
-        for (int j = 0; j < kQmChunk; ++j)
-          nxt[j] = c0 + kQmChunk + j < nv ? __ldg(r + c0 + kQmChunk + j) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-        for (int j = 0; j < kQmChunk; ++j) {
-          if (c0 + j < nv) {
-            fnv::hash_word_full(lo, hi, cur[j].x);
-            fnv::hash_word_full(lo, hi, cur[j].y);
-            fnv::hash_word_full(lo, hi, cur[j].z);
-            fnv::hash_word_full(lo, hi, cur[j].w);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < kQmChunk; ++j) cur[j] = nxt[j];
-      }
-      f = ((uint64_t)hi << 32) | lo;
+  // 1. every row's key
+  if (fp_in) {
+    if (row) {
+      s_fp[tid] = __ldg(fp_in + tid);
+      if (blockIdx.x == 0 && fp_out) fp_out[tid] = s_fp[tid];
     }
-    s_fp[tid] = f;
-    if (blockIdx.x == 0 && fp_out) fp_out[tid] = f;
+  } else {
+    // A group of lanes per row (fewer than 32 for short rows), and kQmRows
+    // rows side by side.
+    int group = 32;
+    while (group > 1 && group / 2 >= nv) group /= 2;
+    const int groups = kQmThreads / group, gl = tid & (group - 1);
+    for (int base = 0; base < n; base += groups * kQmRows) {     // the same for every lane
+      const int r0 = base + tid / group;
+      uint64_t h[kQmRows];
+#pragma unroll
+      for (int r = 0; r < kQmRows; ++r) h[r] = 0;
+      for (int v0 = 0; v0 < nv; v0 += group * kQmPieces) {
+        uint4 x[kQmRows][kQmPieces];
+#pragma unroll
+        for (int r = 0; r < kQmRows; ++r)
+#pragma unroll
+          for (int p = 0; p < kQmPieces; ++p) {
+            const int v = v0 + p * group + gl;
+            if (r0 + r * groups < n && v < nv)
+              x[r][p] = __ldg(q + (size_t)(r0 + r * groups) * nv + v);
+          }
+#pragma unroll
+        for (int r = 0; r < kQmRows; ++r)
+#pragma unroll
+          for (int p = 0; p < kQmPieces; ++p) {
+            const int v = v0 + p * group + gl;
+            if (r0 + r * groups < n && v < nv) h[r] += piece_key(x[r][p], v);
+          }
+      }
+#pragma unroll
+      for (int r = 0; r < kQmRows; ++r) {
+        if (base + r * groups >= n) break;
+        for (int o = group / 2; o > 0; o >>= 1) h[r] += __shfl_xor_sync(0xffffffffu, h[r], o);
+        if (gl == 0 && r0 + r * groups < n) s_fp[r0 + r * groups] = h[r];
+      }
+    }
   }
   __syncthreads();
+  const uint64_t f = row ? s_fp[tid] : 0ull;
 
-  // 2. table: each fingerprint's smallest row index; rep = that row
+  // 2. table: each key's smallest row index; rep = that row
   insert_row(s_keys, s_idx, log2T, row, f, (uint32_t)tid);
   __syncthreads();
   int32_t rep = tid;
@@ -198,7 +241,7 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
 
   // 6. gather the unique rows, split over the CTAs
   const int gitems = total * nv;
-  const int gstride = gridDim.x * kQmThreads;
+  const int gstride = merge_ctas * kQmThreads;
   for (int b = blockIdx.x * kQmThreads + tid; b < gitems; b += gstride * kQmUnroll) {
     uint4 x[kQmUnroll];
     int dst[kQmUnroll];
@@ -230,9 +273,10 @@ hs_status launch_merge_queries(const uint16_t* queries, int64_t n, int32_t dim, 
   const int64_t work = n * (int64_t)nv;
   int64_t grid = (work + kQmThreads * kQmUnroll - 1) / (kQmThreads * kQmUnroll);
   grid = grid < 1 ? 1 : (grid > kQmMaxCtas ? kQmMaxCtas : grid);
-  launch_pdl(merge_queries_kernel, dim3((unsigned)grid), dim3(kQmThreads), 0, stream,
+  const int hash = !fp_in && fp_out ? (int)((n + kQmThreads / 32 - 1) / (kQmThreads / 32)) : 0;
+  launch_pdl(merge_queries_kernel, dim3((unsigned)(grid + hash)), dim3(kQmThreads), 0, stream,
              reinterpret_cast<const uint4*>(queries), (int)n, nv, seed, fp_in, fp_out, n_unique,
-             unique_idx, inverse, reinterpret_cast<uint4*>(uq));
+             unique_idx, inverse, reinterpret_cast<uint4*>(uq), (int)grid);
   count_launches(1);
   return cuda_fail(cudaGetLastError(), "merge_queries launch");
 }

@@ -774,6 +774,15 @@ __device__ __forceinline__ void unpack_key(uint64_t key, float& s, int32_t& idx)
   idx = (int32_t)(0xffffffffu - (uint32_t)key);
 }
 
+// Largest key of the warp's: the largest high word, then the largest low word
+// among the lanes holding it (two warp reductions).
+__device__ __forceinline__ uint64_t warp_max_key(uint64_t key) {
+  const uint32_t hi = (uint32_t)(key >> 32);
+  const uint32_t mhi = __reduce_max_sync(0xffffffffu, hi);
+  const uint32_t mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? (uint32_t)key : 0u);
+  return ((uint64_t)mhi << 32) | mlo;
+}
+
 // One warp per query runs a tournament over the sorted lists.
 // Lane l owns lists l, l+32, ...; it keeps each list's head and the entry
 // after it (prefetched) in registers.  Each round the warp takes the largest
@@ -842,12 +851,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
           best = head[j];
           bj = j;
         }
-      // Warp maximum of the 64-bit keys: the largest high word, then the
-      // largest low word among the lanes holding it (two warp reductions).
-      const uint32_t bhi = (uint32_t)(best >> 32), blo = (uint32_t)best;
-      const uint32_t mhi = __reduce_max_sync(0xffffffffu, bhi);
-      const uint32_t mlo = __reduce_max_sync(0xffffffffu, bhi == mhi ? blo : 0u);
-      const uint64_t mx = ((uint64_t)mhi << 32) | mlo;
+      const uint64_t mx = warp_max_key(best);
       const unsigned win = __ballot_sync(0xffffffffu, best == mx && mx != 0ull);
       last = mx;
       if (kout <= 32) {
@@ -895,6 +899,87 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
   }
 }
 
+// Few output rows, k <= 32: a block per row, and no tournament.  The heads of
+// the lists are ranked by counting; the k best heads name the only lists that
+// can hold one of the k best entries, and the k-th best head bounds those.
+// What is left of these lists, little more than k entries, is ranked by
+// counting again, and an entry's rank is its place.  Two round trips to memory
+// and two loops over shared memory in place of k dependent rounds.  64 rows of
+// 304 lists, k = 10: 11 us cold, 14.4 with a warp each.
+constexpr int kMrThreads = 256;
+constexpr int kMrLists = 32 * kMaxListsPerLane;
+static_assert(kMrLists <= 2 * kMrThreads, "two heads per thread");
+
+__global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
+                                                                float* __restrict__ out_s,
+                                                                int32_t* __restrict__ out_i,
+                                                                OutRows rows) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ uint64_t s_head[kMrLists], s_cand[32 * 32];
+  __shared__ int32_t s_sel[32];
+  __shared__ int s_nsel, s_ncand;
+  const int64_t Q = query_count(p);
+  const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
+  const int k = p.k, lists = 2 * sp.nsplit, tid = threadIdx.x;
+  const int64_t R = rows.inv ? rows.n_out : Q;
+  for (int64_t o = blockIdx.x; o < R; o += gridDim.x) {
+    const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
+    if (q < 0 || q >= Q) {                         // block-uniform
+      if (tid == 0) set_error(p.err, kErrInvalidArg);
+      continue;
+    }
+    const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
+    const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
+    uint64_t mine[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int l = j * kMrThreads + tid;
+      mine[j] = l < lists ? pack_key(ps[(size_t)l * k], pi[(size_t)l * k]) : 0ull;
+      if (l < lists) s_head[l] = mine[j];
+    }
+    if (tid == 0) s_nsel = s_ncand = 0;
+    __syncthreads();
+    int rank[2] = {0, 0};
+#pragma unroll 8
+    for (int l = 0; l < lists; ++l) {              // (heads of empty lists are alike)
+      const uint64_t h = s_head[l];
+      rank[0] += (h > mine[0]) | ((h == mine[0]) & (l < tid));
+      rank[1] += (h > mine[1]) | ((h == mine[1]) & (l < tid + kMrThreads));
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if (j * kMrThreads + tid < lists && rank[j] < k) {
+        s_sel[rank[j]] = j * kMrThreads + tid;
+        atomicAdd(&s_nsel, 1);
+      }
+    __syncthreads();
+    const int nsel = s_nsel;
+    // the k-th best head; with fewer lists than k every entry counts
+    const uint64_t bound = nsel == k ? s_head[s_sel[k - 1]] : 0ull;
+    for (int i = tid; i < nsel * k; i += kMrThreads) {
+      const size_t e = (size_t)s_sel[i / k] * k + i % k;
+      const uint64_t key = pack_key(ps[e], pi[e]);
+      if (key >= bound) s_cand[atomicAdd(&s_ncand, 1)] = key;
+    }
+    __syncthreads();
+    const int c = s_ncand;
+    for (int i = tid; i < c; i += kMrThreads) {
+      const uint64_t key = s_cand[i];
+      int r = 0;
+      for (int j = 0; j < c; ++j) r += (s_cand[j] > key) | ((s_cand[j] == key) & (j < i));
+      if (r < k) {
+        float sc;
+        int32_t id;
+        unpack_key(key, sc, id);
+        out_s[(size_t)o * k + r] = sc;
+        out_i[(size_t)o * k + r] = id;
+      }
+    }
+    __syncthreads();                               // read before the next row's lists come in
+  }
+}
+
 // ---- K6s: small batches (at most 16 queries) -------------------------------------------
 // With few queries the query block of the main kernel is mostly padding and
 // is re-streamed with every corpus stage.  Here the roles are swapped: the
@@ -907,10 +992,13 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
 // tile, holding its 16 scores.  A score above its query's threshold is
 // appended to that query's candidate buffer in shared memory; after each
 // tile a warp merges each non-empty buffer with the query's sorted top-k list
-// (k rounds of a warp-wide maximum over packed (score, ~row) keys) and resets
+// (a few candidates are put in their places by a ballot each, many go through
+// k rounds of a warp-wide maximum over packed (score, ~row) keys) and resets
 // the threshold to the new k-th best.  Each CTA covers a contiguous range of
 // 128-row tiles and writes one sorted list per query, in the layout of the
-// main kernel's lists, so the same merge kernel finishes the job.
+// main kernel's lists, so the same merge kernels finish the job.  With k rounds
+// for every buffer these bounded the kernel: 16 queries, k = 10, 2,097,152 x
+// 768: 680 -> 476 us; k = 32, 1,048,576 x 1024: 1602 -> 353 us.
 constexpr int SQ_N = 16;                    // queries per MMA (N)
 constexpr int SQ_BM = 128;                  // corpus rows per tile (M)
 constexpr int SQ_STAGES = 10;
@@ -918,6 +1006,7 @@ constexpr int SQ_MAXKB = 16;                // d <= 1024
 constexpr int SQ_TBUF = 4;                  // TMEM accumulators
 constexpr uint32_t SQ_TMEM_COLS = 64;       // SQ_TBUF * SQ_N
 constexpr int SQ_CAP = SQ_BM;               // candidates per query per tile: at most one per row
+constexpr int SQ_INSERT = 16;               // candidates inserted one by one; more are selected
 constexpr int SQ_THREADS = 64 + 128;        // producer, MMA, 4 epilogue warps
 constexpr uint32_t SQ_ABYTES = SQ_BM * BK * 2;   // 16 KB
 constexpr uint32_t SQ_QBYTES = SQ_N * BK * 2;    // 2 KB per k-block
@@ -1112,36 +1201,42 @@ __global__ void __launch_bounds__(SQ_THREADS, 1)
       for (int q = ew; q < nq; q += 4) {
         const int c = min(cnt[q], SQ_CAP);
         if (c == 0) continue;
-        uint64_t held[1 + SQ_CAP / 32];
-        held[0] = lane < k ? lists[q * 32 + lane] : 0ull;
-#pragma unroll
-        for (int j = 0; j < SQ_CAP / 32; ++j) {
-          const int e = j * 32 + lane;
-          held[1 + j] = e < c ? cands[q * SQ_CAP + e] : 0ull;
-        }
-        uint64_t mine = 0ull;
-        for (int rd = 0; rd < k; ++rd) {
-          uint64_t best = held[0];
-          int bj = 0;
-#pragma unroll
-          for (int j = 1; j < 1 + SQ_CAP / 32; ++j)
-            if (held[j] > best) {
-              best = held[j];
-              bj = j;
-            }
-          uint64_t mx = best;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const uint64_t y = __shfl_xor_sync(0xffffffffu, mx, o);
-            mx = y > mx ? y : mx;
+        uint64_t mine = lane < k ? lists[q * 32 + lane] : 0ull;
+        if (c <= SQ_INSERT) {
+          // A few: each goes to its place in the sorted list (keys differ).
+          for (int e = 0; e < c; ++e) {
+            const uint64_t x = cands[q * SQ_CAP + e];
+            const int at = __popc(__ballot_sync(0xffffffffu, mine > x));
+            const uint64_t up = __shfl_up_sync(0xffffffffu, mine, 1);
+            if (lane >= at) mine = lane == at ? x : up;
           }
-          if (lane == rd) mine = mx;
-          if (mx == 0ull) continue;
-          const unsigned win = __ballot_sync(0xffffffffu, best == mx);
-          if (lane == __ffs(win) - 1) {
+          if (lane >= k) mine = 0ull;
+        } else {
+          uint64_t held[1 + SQ_CAP / 32];
+          held[0] = mine;
+          mine = 0ull;
 #pragma unroll
-            for (int j = 0; j < 1 + SQ_CAP / 32; ++j)
-              if (j == bj) held[j] = 0ull;
+          for (int j = 0; j < SQ_CAP / 32; ++j) {
+            const int e = j * 32 + lane;
+            held[1 + j] = e < c ? cands[q * SQ_CAP + e] : 0ull;
+          }
+          for (int rd = 0; rd < k; ++rd) {
+            uint64_t best = held[0];
+            int bj = 0;
+#pragma unroll
+            for (int j = 1; j < 1 + SQ_CAP / 32; ++j)
+              if (held[j] > best) {
+                best = held[j];
+                bj = j;
+              }
+            const uint64_t mx = warp_max_key(best);
+            if (mx == 0ull) break;                 // warp-uniform: nothing left
+            if (lane == rd) mine = mx;
+            if (best == mx) {                      // one lane: keys differ
+#pragma unroll
+              for (int j = 0; j < 1 + SQ_CAP / 32; ++j)
+                if (j == bj) held[j] = 0ull;
+            }
           }
         }
         if (lane < k) lists[q * 32 + lane] = mine;
@@ -1394,6 +1489,19 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     // every launch.
     if (2 * (int64_t)pm.slots > 32 * kMaxListsPerLane)
       return fail(HS_ERR_UNSUPPORTED, "more lists per query than the merge takes");
+    // A block per row while there is an SM for each (256 rows of 152 lists
+    // take 1 to 2 us more than with a warp each) and k is worth it (k = 1: 0.5
+    // to 1 us more).  After the main kernel it is launched in plain stream
+    // order: with its blocks waiting beside it, their shared memory cost the
+    // next retrieval up to 45 us; after the small-batch kernel it does not.
+    if (k >= 4 && k <= 32 && nr <= sms) {
+      if (small)
+        launch_pdl(merge_rank_kernel, dim3((unsigned)nr), dim3(kMrThreads), 0, stream, pm, os, oi,
+                   orows);
+      else
+        merge_rank_kernel<<<dim3((unsigned)nr), dim3(kMrThreads), 0, stream>>>(pm, os, oi, orows);
+      return cuda_fail(cudaGetLastError(), "merge launch");
+    }
     {
       const int64_t blocks = (nr + 7) / 8;          // one warp per row
       const dim3 grid((unsigned)(blocks < sms * 16 ? blocks : sms * 16));

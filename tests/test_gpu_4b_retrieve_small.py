@@ -1,0 +1,72 @@
+"""Retrieval at the edges of what its variants take: candidate counts around
+the insertion limit of the small-batch kernel, corpora of a few tiles for
+k <= 32 and beyond, equal scores everywhere, and merges of few rows (Section
+4.1: the k best chunks per query, ties to the lower index)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_22578_gb300 as hs
+import synth
+from hs_testutil import bf16_f64, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def check(Q, C, k):
+    s, i = hs.hs_retrieve_topk(to_dev(Q).view(torch.bfloat16), to_dev(C).view(torch.bfloat16), k)
+    hs.hs_get_device_error()
+    full = bf16_f64(Q) @ bf16_f64(C).T
+    order = np.lexsort((np.broadcast_to(np.arange(len(C)), full.shape), -full))[:, :k]
+    want = np.take_along_axis(full, order, 1)
+    s, i = s.cpu().numpy(), i.cpu().numpy()
+    assert np.abs(s - want).max() < 1e-3
+    assert np.abs(np.take_along_axis(full, i.astype(np.int64), 1) - want).max() < 1e-3
+    assert all(len(set(r)) == k for r in i.tolist())
+    return s, i, order
+
+
+@pytest.mark.parametrize("k", [1, 3, 4, 10, 16, 17, 32])
+@pytest.mark.parametrize("nq,N", [(1, 127), (5, 129), (16, 5000), (17, 300), (64, 4096),
+                                  (152, 2000), (153, 2000), (300, 777)])
+def test_register_lists_on_small_corpora(nq, N, k):
+    check(synth.unit_rows(nq, 72, nq + k), synth.unit_rows(N, 72, N), k)
+
+
+@pytest.mark.parametrize("nq,N,k", [(3, 40, 33), (20, 256, 64), (5, 300, 64), (130, 1000, 100),
+                                    (260, 2000, 200), (40, 16000, 500), (9, 4096, 1024)])
+def test_large_k_on_few_tiles(nq, N, k):
+    check(synth.unit_rows(nq, 64, nq), synth.unit_rows(N, 64, N + k), k)
+
+
+@pytest.mark.parametrize("k", [5, 32, 100])
+def test_large_k_crowded_into_one_tile(k):
+    """The top k of every query lies in one tile of the corpus: the lists of
+    the optimistic pass are cut, and the blocks run the exact pass."""
+    C = synth.unit_rows(3000, 64, 5)
+    Q = np.tile(synth.unit_rows(1, 64, 6), (150, 1))
+    near = bf16_f64(Q[:1]).astype(np.float32) + np.linspace(0.0, 0.3, 200)[:, None].astype(
+        np.float32) * bf16_f64(C[:200]).astype(np.float32)
+    near /= np.linalg.norm(near, axis=1, keepdims=True)
+    C[520:720] = torch.from_numpy(near).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    check(Q, C, k)
+
+
+@pytest.mark.parametrize("nq", [1, 16, 17, 200])
+@pytest.mark.parametrize("k", [4, 10, 32, 40])
+def test_equal_scores_go_to_the_lowest_rows(nq, k):
+    C = np.tile(synth.unit_rows(1, 64, 1), (1500, 1))
+    s, i, order = check(np.tile(synth.unit_rows(1, 64, 2), (nq, 1)), C, k)
+    assert (i == np.arange(k)).all() and (s == s[0, 0]).all()
+
+
+@pytest.mark.parametrize("nq", [2, 40])
+def test_scores_of_the_lowest_value_and_ascending_rows(nq):
+    """Every row beats the ones before it, and zero rows (score 0) among
+    negative ones: each tile replaces the whole list."""
+    base = bf16_f64(synth.unit_rows(1, 64, 3))[0]
+    scale = np.linspace(-1.0, -0.01, 2000)
+    scale[::97] = 0.0
+    rows = torch.from_numpy((scale[:, None] * base).astype(np.float32)).to(torch.bfloat16)
+    C = rows.view(torch.int16).numpy().view(np.uint16)
+    check(np.tile(synth.unit_rows(1, 64, 3), (nq, 1)), C, 10)

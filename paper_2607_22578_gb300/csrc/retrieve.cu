@@ -212,6 +212,23 @@ __device__ __forceinline__ float chunk_max(const uint32_t (&r)[32]) {
   return fmaxf(max3f(a, b, c), e);
 }
 
+// Sort N (a power of two) values in descending order: a bitonic network.
+template <int N>
+__device__ __forceinline__ void sort_desc(float (&v)[N]) {
+#pragma unroll
+  for (int size = 2; size <= N; size *= 2)
+#pragma unroll
+    for (int d = size / 2; d > 0; d /= 2)
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if ((i & d) == 0) {
+          const float hi = fmaxf(v[i], v[i | d]), lo = fminf(v[i], v[i | d]);
+          const bool down = (i & size) == 0;
+          v[i] = down ? hi : lo;
+          v[i | d] = down ? lo : hi;
+        }
+}
+
 // Insert (s, idx) into a list sorted by score descending.  idx is larger than
 // every index already present, so on equal scores it goes after them.
 template <int KREG>
@@ -565,6 +582,42 @@ __global__ void __launch_bounds__(kThreads, 1)
           Ls[i] = -FLT_MAX;
           Li[i] = -1;
         }
+      }
+      // A list that starts with no threshold would take nearly every score of
+      // its first tile in turn.  The maxima of 16 groups of columns give it one:
+      // the k-th largest is reached by k columns, so the k best of the tile are
+      // not below it (ties with it are kept).  A 17 to 128 query batch over 4096
+      // x 384, k = 10: 31 to 35 -> 22 to 25 us.  (Lists of 32 slots have no
+      // registers for it: the large corpus with k = 100 took 1 % more.)
+      if (KREG > 0 && KREG < 32 && __any_sync(0xffffffffu, valid_q && qf_seen == 0u)) {
+        const uint32_t acc = tile_i & 1u, aphase = (tile_i >> 1) & 1u;
+        if (!mbar_wait_limit(tfull + acc, aphase, abort_flag, lim)) goto epi_done;
+        tc_fence_after();
+        const int64_t col0 = t0 * BN + half * kHalfCols;
+        const bool tail = col0 + kHalfCols > p.N;
+        constexpr int kGroups = 16, kEach = kHalfCols / kGroups;
+        float gm[kGroups];
+#pragma unroll
+        for (int c = 0; c < kHalfCols / 32; ++c) {
+          uint32_t r[32];
+          tmem_ld_32x32b_x32(tmem_base + lane_addr + acc * BN + half * kHalfCols + c * 32, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int g = 0; g < 32 / kEach; ++g) {
+            float m = -FLT_MAX;
+#pragma unroll
+            for (int e = 0; e < kEach; ++e)
+              if (!tail || col0 + c * 32 + g * kEach + e < p.N)
+                m = fmaxf(m, __uint_as_float(r[g * kEach + e]));
+            gm[c * (32 / kEach) + g] = m;
+          }
+        }
+        tc_fence_before();
+        sort_desc<kGroups>(gm);
+        float kth = -FLT_MAX;
+#pragma unroll
+        for (int i = 0; i < kGroups; ++i) kth = i == k - 1 ? gm[i] : kth;
+        if (kth > -FLT_MAX) qf_theta = fmaxf(qf_theta, nextafterf(kth, -INFINITY));
       }
       for (int64_t t = t0; t < t1; ++t, ++tile_i) {
         const uint32_t acc = tile_i & 1u, aphase = (tile_i >> 1) & 1u;

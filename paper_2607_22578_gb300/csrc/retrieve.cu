@@ -1607,7 +1607,7 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   } else if (k <= 32) {
     st = launch_variant<32>(corpus, N, d, mq, prm, stream);
   } else {
-    // Large k.  With at least 64 corpus tiles an optimistic pass runs first:
+    // Large k.  Unless the corpus has few tiles an optimistic pass runs first:
     // the register-list kernel (32 per list, no shared floor: a floor that
     // bounds 32nd-best scores would cut rows of the top k) over the whole
     // corpus, merged to the first k of the union of its lists.  A list whose
@@ -1620,9 +1620,13 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     // pass 2: the large-k kernel over the whole corpus keeping scores >= the
     // floor), and every kernel of it skips the other blocks.  Both passes'
     // lists go through the same workspace; the floors are staged in it.
-    if (tiles >= 64) {
+    // A tile gives a query two lists, so with k <= 32 tiles a list holds 16 of
+    // the top k on average, four deviations below the 32 it keeps; pass 1
+    // needs eight tiles of its own.  4096
+    // x 384, k = 100: 1 query 157 -> 85 us, 2048 queries 1267 -> 171 us.
+    if ((int64_t)k <= 32 * tiles) {
       const int64_t nb = (Qmax + BM - 1) / BM;
-      cudaError_t ze = cudaMemsetAsync(block_flags, 0, (size_t)nb * 4, stream);
+      const cudaError_t ze = cudaMemsetAsync(block_flags, 0, (size_t)nb * 4, stream);
       if (ze != cudaSuccess) return cuda_fail(ze, "flag clear");
       Params pa = prm;
       pa.k = 32;
@@ -1633,12 +1637,14 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       st = merge(pa, k, scores_out, ids_out, rows, block_flags, nullptr);
       if (st != HS_OK) return st;
       count_launches(2);
+      prm.only = block_flags;
+    }
+    if (tiles >= 64 && prm.only) {
       Params p1 = prm;
       p1.tiles = tiles / 8;
       p1.N = p1.tiles * BN;
       p1.k = 32;
       p1.floor = nullptr;
-      p1.only = block_flags;
       st = launch_variant<32>(corpus, N, d, mq, p1, stream);
       if (st != HS_OK) return st;
       st = merge(p1, k, kth, nullptr, OutRows{nullptr, 0}, nullptr, block_flags);
@@ -1647,9 +1653,8 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       prm.floor = kth;
       prm.floor_stride = 1;
       prm.floor_index = 0;
-      prm.only = block_flags;
       // Pass 1's shared floors bound 32nd-best scores, not k-th best: clear.
-      ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
+      const cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
       if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
     }
     st = launch_variant<0>(corpus, N, d, mq, prm, stream);

@@ -530,7 +530,7 @@ uint64_t hs_launch_count(void);
  * Every device-side wait of the library gives up after a limit (2 s by
  * default) and then sets HS_ERR_TIMEOUT in the device error word instead of
  * spinning on.  hs_unique_inverse's scan waits for the status each earlier
- * tile of 16,384 rows publishes (decoupled look-back).  This hook, for tests
+ * tile of 4,096 rows publishes (decoupled look-back).  This hook, for tests
  * only, lowers that wait's limit and can stop one tile from publishing, so
  * that a test can make the wait run out and check that the call returns,
  * that hs_get_device_error reports HS_ERR_TIMEOUT, and that the next call

@@ -38,11 +38,10 @@ namespace {
 
 using namespace table;
 
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 16;
+constexpr int kScanThreads = 512;
+constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 static_assert(kScanThreads % 32 == 0 && kScanThreads <= 1024, "scan block: whole warps, at most 32");
-constexpr int kLookBatch = 8;           // predecessor statuses read per round trip
 constexpr int64_t kSmallRows = 4096;    // single-launch path
 constexpr int kSmallThreads = 512;
 constexpr int kResolveThreads = 512;    // one block for the collision list
@@ -360,10 +359,14 @@ __global__ void __launch_bounds__(kResolveThreads) resolve_kernel(
 }
 
 // Single-pass exclusive sum-scan of "rep[i] == i" with decoupled look-back;
-// the last tile writes the total (the group count).  A predecessor's status
-// is awaited for at most limit_ns of %globaltimer; then the wait gives up,
-// sets kErrTimeout and counts the predecessor as a zero prefix (the call's
-// outputs are then unspecified, but every write stays in bounds).
+// the last tile writes the total (the group count).  A warp looks back over 32
+// predecessors per round trip, so tiles can be small enough to spread a batch
+// over the SMs (400,000 rows: 98 tiles of 4096).  A predecessor's status is
+// awaited for at most limit_ns of %globaltimer; then the wait gives up, sets
+// kErrTimeout and counts the predecessor as a zero prefix (the call's outputs
+// are then unspecified, but every write stays in bounds).
+// Bound by its chain of round trips: 65,536 rows 5.2 us cold (7.2 us in tiles
+// of 16,384 with eight predecessors at a time).
 __device__ __forceinline__ uint64_t wait_status(const volatile unsigned long long* p,
                                                 unsigned* err, uint64_t limit_ns) {
   unsigned long long s = *p;
@@ -382,39 +385,41 @@ __device__ __forceinline__ uint64_t wait_status(const volatile unsigned long lon
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __restrict__ rep,
-                                                            int64_t n, int32_t* __restrict__ uid,
-                                                            unsigned long long* status,
-                                                            uint32_t* ctr, int32_t* total_out,
-                                                            unsigned* err, uint64_t limit_ns,
-                                                            int64_t withhold_tile) {
+__global__ void __launch_bounds__(kScanThreads) scan_kernel(
+    const int32_t* __restrict__ rep, int64_t n, int32_t* __restrict__ uid, unsigned long long* status, uint32_t* ctr, int32_t* total_out, unsigned* err, uint64_t limit_ns, int64_t withhold_tile) {
   pdl_wait();
   pdl_trigger();
+  constexpr int kWarps = kScanThreads / 32;
   __shared__ uint32_t s_tile;
-  __shared__ int32_t s_warp[kScanThreads / 32];
+  __shared__ int32_t s_warp[kWarps];
   __shared__ int32_t s_prefix;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (tid == 0) s_tile = atomicAdd(ctr + kCtrScan, 1u);
   __syncthreads();
   const uint32_t tile = s_tile;
   const int64_t base = (int64_t)tile * kScanTile + (int64_t)tid * kScanItems;
-  int32_t x[kScanItems];
-  int32_t run = 0;
+  int32_t r[kScanItems];
+  if (base + kScanItems <= n) {
 #pragma unroll
-  for (int i = 0; i < kScanItems; i += 4) {
-    const int64_t e = base + i;
-    if (e + 3 < n) {
-      const int4 v = *reinterpret_cast<const int4*>(rep + e);
-      x[i] = v.x == (int32_t)e;
-      x[i + 1] = v.y == (int32_t)(e + 1);
-      x[i + 2] = v.z == (int32_t)(e + 2);
-      x[i + 3] = v.w == (int32_t)(e + 3);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) x[i + j] = (e + j < n) ? (rep[e + j] == (int32_t)(e + j)) : 0;
+    for (int i = 0; i < kScanItems; i += 4) {
+      const int4 v = *reinterpret_cast<const int4*>(rep + base + i);
+      r[i] = v.x;
+      r[i + 1] = v.y;
+      r[i + 2] = v.z;
+      r[i + 3] = v.w;
     }
-    run += x[i] + x[i + 1] + x[i + 2] + x[i + 3];
+  } else {
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) r[i] = base + i < n ? rep[base + i] : 0;
   }
+  int32_t run = 0;
+  uint32_t own = 0;                            // bit i: row base + i is its own representative
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i)
+    if (base + i < n && r[i] == (int32_t)(base + i)) {
+      own |= 1u << i;
+      ++run;
+    }
   int32_t incl = run;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -424,7 +429,6 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __res
   if (lane == 31) s_warp[w] = incl;
   __syncthreads();
   if (w == 0) {
-    constexpr int kWarps = kScanThreads / 32;
     const int32_t v = lane < kWarps ? s_warp[lane] : 0;
     int32_t iv = v;
 #pragma unroll
@@ -433,33 +437,24 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __res
       if (lane >= o) iv += y;
     }
     if (lane < kWarps) s_warp[lane] = iv - v;  // exclusive warp offsets
-    if (lane == 31) {
-      const int32_t tile_total = iv;
-      volatile unsigned long long* st = status;
-      int32_t prefix = 0;
-      // A withheld tile (test hook, -1 in normal use) never publishes, so
-      // its successors' waits run out.
-      const bool publish = (int64_t)tile != withhold_tile;
-      if (tile == 0) {
-        if (publish) st[0] = (2ull << 32) | (uint32_t)tile_total;
-      } else {
-        if (publish) st[tile] = (1ull << 32) | (uint32_t)tile_total;
-        bool done = false;
-        for (int64_t j0 = (int64_t)tile - 1; j0 >= 0 && !done; j0 -= kLookBatch) {
-          unsigned long long sv[kLookBatch];
-#pragma unroll
-          for (int b = 0; b < kLookBatch; ++b) sv[b] = j0 - b >= 0 ? st[j0 - b] : (2ull << 32);
-#pragma unroll
-          for (int b = 0; b < kLookBatch; ++b) {
-            if (done) break;
-            unsigned long long sb = sv[b];
-            if ((sb >> 32) == 0) sb = wait_status(st + (j0 - b), err, limit_ns);
-            if (j0 - b >= 0) prefix += (int32_t)(uint32_t)sb;
-            if ((sb >> 32) == 2ull) done = true;
-          }
-        }
-        if (publish) st[tile] = (2ull << 32) | (uint32_t)(prefix + tile_total);
-      }
+    const int32_t tile_total = __shfl_sync(0xffffffffu, iv, 31);
+    // A withheld tile (test hook, -1 in normal use) never publishes, so its
+    // successors' waits run out.
+    volatile unsigned long long* st = status;
+    const bool publish = lane == 0 && (int64_t)tile != withhold_tile;
+    if (publish) st[tile] = ((tile == 0 ? 2ull : 1ull) << 32) | (uint32_t)tile_total;
+    int32_t prefix = 0;
+    bool done = tile == 0;
+    for (int64_t j0 = (int64_t)tile - 1; !done; j0 -= 32) {
+      const int64_t j = j0 - lane;             // before the first tile: a zero prefix
+      const uint64_t sv = j >= 0 ? wait_status(st + j, err, limit_ns) : 2ull << 32;
+      const unsigned ends = __ballot_sync(0xffffffffu, (sv >> 32) == 2ull);
+      const int last = ends ? __ffs(ends) - 1 : 31;
+      prefix += __reduce_add_sync(0xffffffffu, lane <= last ? (int32_t)(uint32_t)sv : 0);
+      done = ends != 0u;
+    }
+    if (lane == 0) {
+      if (publish && tile > 0) st[tile] = (2ull << 32) | (uint32_t)(prefix + tile_total);
       s_prefix = prefix;
       const int64_t tiles = (n + kScanTile - 1) / kScanTile;
       if ((int64_t)tile == tiles - 1) *total_out = prefix + tile_total;
@@ -471,7 +466,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __res
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     u[i] = acc;
-    acc += x[i];
+    acc += (own >> i) & 1u;
   }
   if (base + kScanItems <= n) {
 #pragma unroll
@@ -502,7 +497,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const int32_t* __restrict
 }
 
 // ---- verify over flat piece lists ------------------------------------------------------------
-// Verify of 32 consecutive rows per warp against their representatives (the
+// Verify of up to 32 consecutive rows per warp against their representatives (the
 // table's smallest row with the same fingerprint).  The rows that need a
 // comparison (representative another row, lengths equal) are compared as
 // one flat list of piece pairs: the warp's pairs are laid end to end (a
@@ -513,7 +508,10 @@ __global__ void __launch_bounds__(256) finalize_kernel(const int32_t* __restrict
 // the tokens of a pair's last piece past its length masked.  Otherwise the
 // rows may start on any word and a piece is one word, coalesced over the
 // lanes, with twice as many in flight: 20,011 rows at a stride of 333, a third
-// of them copies, take 21 us cold (40 us as two rows per warp round).
+// of them copies, take 21 us cold (40 us as two rows per warp round).  Batches
+// that do not fill the GPU with 32 rows per warp take fewer, down to 4, so a
+// warp's chain of rounds is shorter: with the scan's smaller tiles 20,011 rows
+// take 25 us from fingerprints to inverse (35), 65,536 rows of 256 tokens 33 (38).
 constexpr int kVerifyThreads = 256;
 
 // Do the first `live` tokens of two 16-byte pieces, or two words, differ?
@@ -528,7 +526,8 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
     const uint64_t* __restrict__ fp, uint64_t key_mask, int64_t n,
     const uint64_t* __restrict__ keys, const uint32_t* __restrict__ idx, int log2T,
     const int32_t* __restrict__ tokens, int32_t stride, const int32_t* __restrict__ lens,
-    int32_t* __restrict__ rep, int32_t* coll_list, uint32_t* ctr, unsigned* err) {
+    int rows_per_warp, int32_t* __restrict__ rep, int32_t* coll_list, uint32_t* ctr,
+    unsigned* err) {
   pdl_wait();
   pdl_trigger();
   constexpr int kPieces = VEC ? 4 : 8;
@@ -539,9 +538,9 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int64_t p0 = w * 32; p0 < n; p0 += warps * 32) {
+  for (int64_t p0 = w * rows_per_warp; p0 < n; p0 += warps * rows_per_warp) {
     const int64_t a = p0 + lane;
-    const bool valid = a < n;
+    const bool valid = lane < rows_per_warp && a < n;
     int64_t r = a;
     int32_t la = 0, lr = 0;
     if (valid) {
@@ -794,6 +793,14 @@ unsigned grid_for(int64_t items, int per_block, int max_blocks) {
   return (unsigned)b;
 }
 
+// Rows per warp of the verify: 32, or fewer while that leaves over half of the
+// GPU's warps (32 per SM) without any.
+int verify_rows(int64_t n, int sms) {
+  int r = 32;
+  while (r > 4 && n < (int64_t)sms * 16 * r) r /= 2;
+  return r;
+}
+
 template <bool VEC>
 hs_status launch_small(const uint64_t* fp, const int32_t* tokens, int64_t n, int32_t stride,
                        const int32_t* lens, int32_t* n_unique, int32_t* unique_idx,
@@ -855,10 +862,11 @@ hs_status launch_unique_inverse(const uint64_t* fp, const int32_t* tokens, int64
   if (e != cudaSuccess) return cuda_fail(e, "hash table clear");
   launch_pdl(insert_kernel, dim3(grid_for(n, 256, sms * 8)), dim3(256), 0, stream, fp, n, keys, idx,
              L.log2T);
+  const int vr = verify_rows(n, sms);
   launch_pdl(vec ? verify_flat_kernel<true> : verify_flat_kernel<false>,
-             dim3(grid_for(n, kVerifyThreads, sms * 8)), dim3(kVerifyThreads), 0, stream, fp,
-             ~0ull, n, (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride, lens,
-             rep, coll_list, ctr, err);
+             dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)), dim3(kVerifyThreads), 0, stream,
+             fp, ~0ull, n, (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride,
+             lens, vr, rep, coll_list, ctr, err);
   if (vec)
     launch_pdl(resolve_kernel<true>, dim3(1), dim3(kResolveThreads), 0, stream, fp, tokens, stride,
                lens, rep, coll_list, ctr, keys, idx, uid, err);
@@ -921,9 +929,11 @@ hs_status launch_merge_rows(const int32_t* tokens, int64_t n, int32_t stride, co
   if (st != HS_OK) return st;
   launch_pdl(tails_insert_kernel, dim3(grid_for(n, 256, sms * 16)), dim3(256), 0, stream, tokens,
              (int64_t)0, n, stride, lens, seed, ran, mask, fp_out, keys, idx, L.log2T, err);
-  launch_pdl(verify_flat_kernel<true>, dim3(grid_for(n, kVerifyThreads, sms * 8)),
-             dim3(kVerifyThreads), 0, stream, (const uint64_t*)fp_out, mask, n, (const uint64_t*)keys,
-             (const uint32_t*)idx, L.log2T, tokens, stride, lens, rep, coll_list, ctr, err);
+  const int vr = verify_rows(n, sms);
+  launch_pdl(verify_flat_kernel<true>, dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)),
+             dim3(kVerifyThreads), 0, stream, (const uint64_t*)fp_out, mask, n,
+             (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride, lens, vr, rep,
+             coll_list, ctr, err);
   launch_pdl(resolve_kernel<true>, dim3(1), dim3(kResolveThreads), 0, stream,
              (const uint64_t*)fp_out, tokens, stride, lens, rep, (const int32_t*)coll_list,
              (const uint32_t*)ctr, keys, idx, uid, err);

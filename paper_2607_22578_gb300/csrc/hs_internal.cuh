@@ -253,6 +253,21 @@ __device__ __forceinline__ uint32_t cluster_smem_addr(const void* p, uint32_t ra
   return r;
 }
 
+// A word of shared memory given by its cluster address.
+__device__ __forceinline__ uint32_t ld_cluster(uint32_t cluster_addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t cluster_atomic_inc(uint32_t cluster_addr) {
+  uint32_t v;
+  asm volatile("atom.shared::cluster.add.u32 %0, [%1], 1;"
+               : "=r"(v)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+
 // Arrive once on an mbarrier given by its cluster shared-memory address.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)

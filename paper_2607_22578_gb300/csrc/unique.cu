@@ -22,10 +22,7 @@
 //      group its ordinal in first-occurrence order (single pass, decoupled
 //      look-back with bounded spins); the final kernel writes unique_idx and
 //      inverse.
-// Up to kSmallRows rows, one launch does it all: every CTA builds the table
-// for all rows in its own shared memory (the same table in each), verifies
-// its share of the rows, and the last CTA to finish resolves the collision
-// list, scans and writes the outputs.
+// Up to kSmallRows rows, one launch of one cluster does it all.
 #include <mutex>
 #include <type_traits>
 
@@ -42,8 +39,7 @@ constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 static_assert(kScanThreads % 32 == 0 && kScanThreads <= 1024, "scan block: whole warps, at most 32");
-constexpr int64_t kSmallRows = 4096;    // single-launch path
-constexpr int kSmallThreads = 512;
+constexpr int64_t kSmallRows = 4096;    // single-launch path: 1024 threads, four rows each
 constexpr int kResolveThreads = 512;    // one block for the collision list
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -59,7 +55,6 @@ struct Layout {
 // Counters (uint32 each) in the zeroed region.
 constexpr int kCtrColl = 0;   // collision list length
 constexpr int kCtrScan = 1;   // scan tile ticket
-constexpr int kCtrDone = 2;   // CTAs finished (single-launch path)
 
 constexpr Layout layout(int64_t n) {
   Layout L{};
@@ -672,25 +667,36 @@ __global__ void __launch_bounds__(256) tails_insert_kernel(
 }
 
 // ---- single-launch path (n <= kSmallRows) ----------------------------------------------------
+// One cluster of CTAs, each of which builds the whole table in its own shared
+// memory (the same table in each), verifies its share of the rows, and, once
+// the cluster's barrier has shown that no keys collided, scans the whole batch
+// and writes its share of the outputs.  The barrier is the only dependency
+// between CTAs, so the call needs no counters in memory and nothing cleared.
+// A collision list (its length in the first CTA's shared memory) is regrouped
+// by that CTA, which then writes all outputs.  THREADS threads of up to ROWS
+// rows each.
+//
+// Bound by its chain of round trips and barriers.  Fingerprints to inverse, us
+// (CTAs without a cluster, whose last one to finish scanned and wrote alone,
+// after a memset of its counters): 64 rows 5.1 (12.3), 512 rows of 384 words
+// 7.5 (12.7), 2048 rows 14.9 (21.0), 4096 rows of 128 words 23.5 (26.7).
 // Dynamic shared memory: keys[T + 1], idx[T + 1], rep[n], uid[n] (T = 2^log2T).
 constexpr size_t small_smem(int64_t n) {
   const size_t T1 = (size_t(1) << table_log2(n)) + 1;
   return T1 * 8 + T1 * 4 + (size_t)n * 8 + 16;
 }
-static_assert(small_smem(kSmallRows) + kSmallThreads / 32 * 4 + 16 <= 232448,
+static_assert(small_smem(kSmallRows) + 256 <= 232448,
               "one-launch path: the table, rep and uid fit one CTA's shared memory");
 
-template <bool VEC>
-__global__ void __launch_bounds__(kSmallThreads, 1) unique_small_kernel(
-    const uint64_t* __restrict__ fp, int64_t n, const int32_t* __restrict__ tokens,
-    int32_t stride, const int32_t* __restrict__ lens, int32_t* __restrict__ n_unique,
-    int32_t* __restrict__ unique_idx, int32_t* __restrict__ inverse, uint32_t* ctr,
-    int32_t* coll_list, unsigned* err) {
-  pdl_wait();
-  pdl_trigger();
+template <bool VEC, int THREADS, int ROWS>
+__global__ void __launch_bounds__(THREADS, 1) unique_small_kernel(
+    const uint64_t* __restrict__ fp, int n, const int32_t* __restrict__ tokens, int32_t stride,
+    const int32_t* __restrict__ lens, int32_t* __restrict__ n_unique,
+    int32_t* __restrict__ unique_idx, int32_t* __restrict__ inverse, int32_t* coll_list,
+    unsigned* err) {
   extern __shared__ __align__(16) uint8_t sm[];
-  __shared__ bool s_last;
-  __shared__ int32_t s_warp[kSmallThreads / 32];
+  __shared__ uint32_t s_ncoll;
+  __shared__ int32_t s_warp[THREADS / 32];
   const int log2T = table_log2(n);
   const uint32_t T1 = (1u << log2T) + 1u;
   uint64_t* keys = reinterpret_cast<uint64_t*>(sm);
@@ -698,61 +704,70 @@ __global__ void __launch_bounds__(kSmallThreads, 1) unique_small_kernel(
   int32_t* rep = reinterpret_cast<int32_t*>(idx + T1);
   int32_t* uid = rep + n;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  constexpr int kWarps = kSmallThreads / 32;
+  constexpr int kWarps = THREADS / 32;
+  const int ctas = (int)gridDim.x, rank = (int)blockIdx.x;   // the grid is one cluster
 
   // 1. the table for all rows (the same in every CTA)
-  for (uint32_t s = tid; s < T1; s += kSmallThreads) {
+  for (uint32_t s = tid; s < T1; s += THREADS) {
     keys[s] = kEmpty;
     idx[s] = kNoRow;
   }
+  if (tid == 0) s_ncoll = 0;
+  pdl_wait();
+  pdl_trigger();
   __syncthreads();
-  for (int64_t base = 0; base < n; base += kSmallThreads) {
-    const int64_t i = base + tid;
-    const bool valid = i < n;
-    insert_row(keys, idx, log2T, valid, valid ? __ldg(fp + i) : 0ull, (uint32_t)i);
-  }
+  if (ctas > 1) cluster_sync();                // the first CTA's counter is 0
+  uint64_t f[ROWS];                            // all of the thread's rows at once
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) f[u] = u * THREADS + tid < n ? __ldg(fp + u * THREADS + tid) : 0ull;
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u)
+    if (u * THREADS < n)
+      insert_row(keys, idx, log2T, u * THREADS + tid < n, f[u], (uint32_t)(u * THREADS + tid));
   __syncthreads();
-  for (int64_t i = tid; i < n; i += kSmallThreads) {
-    const uint32_t v = idx[find_key(keys, __ldg(fp + i), log2T)];
-    rep[i] = v < (uint32_t)n ? (int32_t)v : (int32_t)i;
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    const int i = u * THREADS + tid;
+    if (i < n) {
+      const uint32_t v = idx[find_key(keys, f[u], log2T)];
+      rep[i] = v < (uint32_t)n ? (int32_t)v : i;
+    }
   }
   __syncthreads();
 
-  // 2. verify this CTA's rows: warp-rounds of 32 rows, dealt round-robin
-  //    over the CTAs first, so every CTA gets a share
-  const int64_t rounds = (n + 31) / 32;
-  for (int64_t rd = (int64_t)w * gridDim.x + blockIdx.x; rd < rounds;
-       rd += (int64_t)gridDim.x * kWarps) {
-    const int64_t a = rd * 32 + lane;
-    const bool valid = a < n;
+  // 2. verify this CTA's rows: rounds of 8 rows per warp (a round is a chain
+  //    of memory round trips, two rows at a time), dealt over all warps
+  constexpr int kRound = 8;
+  const uint32_t count = cluster_smem_addr(&s_ncoll, 0);
+  const int rounds = (n + kRound - 1) / kRound;
+  for (int rd = w * ctas + rank; rd < rounds; rd += ctas * kWarps) {
+    const int a = rd * kRound + lane;
+    const bool valid = lane < kRound && a < n;
     const int64_t r = valid ? rep[a] : a;
     const bool merged = verify_warp<VEC>(tokens, stride, lens, valid, a, r, err);
-    if (valid && !merged) coll_list[atomicAdd(ctr + kCtrColl, 1u)] = (int32_t)a;
+    if (valid && !merged) coll_list[cluster_atomic_inc(count)] = a;
   }
-
-  // 3. the last CTA to finish writes the outputs
   __syncthreads();
-  if (tid == 0) {
+  if (ctas > 1) cluster_sync();                // every row is verified
+  uint32_t m = ld_cluster(count);
+  if (ctas > 1) cluster_sync();                // the counter is read: its CTA may leave
+  if (m > 0) {
+    if (rank != 0) return;
     __threadfence();
-    s_last = atomicAdd(ctr + kCtrDone, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const uint32_t m = *reinterpret_cast<volatile uint32_t*>(ctr + kCtrColl);
-  for (uint32_t c = tid; c < m; c += kSmallThreads) rep[coll_list[c]] = -1;
-  __syncthreads();
-  if (m) {   // the table and uid are free here: uid holds the rows left for peeling
+    for (uint32_t c = tid; c < m; c += THREADS) rep[__ldcg(coll_list + c)] = -1;
+    __syncthreads();
+    // the table and uid are free here: uid holds the rows left for peeling
     const uint32_t m2 =
         regroup_block<VEC>(fp, tokens, stride, lens, rep, coll_list, m, keys, idx, uid, err);
     if (m2) peel_block<VEC>(fp, tokens, stride, lens, rep, uid, m2, err);
+    __syncthreads();
   }
-  __syncthreads();
-  // exclusive scan of rep[i] == i: contiguous items per thread
-  const int64_t per = (n + kSmallThreads - 1) / kSmallThreads;
-  const int64_t b0 = tid * per, b1 = min(n, b0 + per);
+
+  // 3. exclusive scan of rep[i] == i: contiguous items per thread
+  const int per = (n + THREADS - 1) / THREADS;
+  const int b0 = min(n, tid * per), b1 = min(n, b0 + per);
   int32_t run = 0;
-  for (int64_t i = b0; i < b1; ++i) run += rep[i] == (int32_t)i;
+  for (int i = b0; i < b1; ++i) run += rep[i] == i;
   int32_t incl = run;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -762,23 +777,27 @@ __global__ void __launch_bounds__(kSmallThreads, 1) unique_small_kernel(
   if (lane == 31) s_warp[w] = incl;
   __syncthreads();
   int32_t off = 0, total = 0;
+#pragma unroll
   for (int i = 0; i < kWarps; ++i) {
     off += i < w ? s_warp[i] : 0;
     total += s_warp[i];
   }
   int32_t acc = off + incl - run;
-  for (int64_t i = b0; i < b1; ++i) {
+  for (int i = b0; i < b1; ++i) {
     uid[i] = acc;
-    acc += rep[i] == (int32_t)i;
+    acc += rep[i] == i;
   }
   __syncthreads();
-  for (int64_t i = tid; i < n; i += kSmallThreads) {
+
+  // 4. the outputs, every CTA its share
+  const int shares = m > 0 ? 1 : ctas;
+  for (int i = rank * THREADS + tid; i < n; i += shares * THREADS) {
     const int32_t r = rep[i];
     inverse[i] = uid[r];
-    if (r == (int32_t)i) unique_idx[uid[i]] = (int32_t)i;
+    if (r == i) unique_idx[uid[i]] = i;
+    if (i >= total) unique_idx[i] = 0;
   }
-  for (int64_t i = total + tid; i < n; i += kSmallThreads) unique_idx[i] = 0;
-  if (tid == 0) *n_unique = total;
+  if (rank == 0 && tid == 0) *n_unique = total;
 }
 
 // Test hook of the look-back's bounded wait (hs_debug_scan_wait): the wait
@@ -801,27 +820,42 @@ int verify_rows(int64_t n, int sms) {
   return r;
 }
 
-template <bool VEC>
+template <bool VEC, int THREADS, int ROWS>
 hs_status launch_small(const uint64_t* fp, const int32_t* tokens, int64_t n, int32_t stride,
                        const int32_t* lens, int32_t* n_unique, int32_t* unique_idx,
-                       int32_t* inverse, uint32_t* ctr, int32_t* coll_list, unsigned* err,
-                       cudaStream_t stream) {
+                       int32_t* inverse, int32_t* coll_list, unsigned* err, cudaStream_t stream) {
+  auto* kernel = unique_small_kernel<VEC, THREADS, ROWS>;
   const size_t smem = small_smem(n);
   static std::atomic<uint64_t> configured{0};
   if (smem > 48 * 1024) {
     const hs_status cst = once_per_device(configured, [] {
-      return cuda_fail(cudaFuncSetAttribute(unique_small_kernel<VEC>,
+      return cuda_fail(cudaFuncSetAttribute(unique_small_kernel<VEC, THREADS, ROWS>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)small_smem(kSmallRows)),
+                                            (int)small_smem(THREADS * ROWS)),
                        "unique smem attribute");
     });
     if (cst != HS_OK) return cst;
   }
-  // One CTA per 2 warp-rounds of rows (they wait on memory), at most one per SM.
-  const unsigned grid = grid_for((n + 31) / 32, 2, num_sms());
-  launch_pdl(unique_small_kernel<VEC>, dim3(grid), dim3(kSmallThreads), smem, stream, fp, n, tokens,
-             stride, lens, n_unique, unique_idx, inverse, ctr, coll_list, err);
-  return HS_OK;
+  // A CTA per 64 rows, at most the portable cluster size.
+  unsigned ctas = 1;
+  while (ctas < 8 && (int64_t)ctas * 64 < n) ctas *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cuda_fail(cudaLaunchKernelEx(&cfg, kernel, fp, (int)n, tokens, stride,
+                                      lens, n_unique, unique_idx, inverse, coll_list, err),
+                   "unique launch");
 }
 
 }  // namespace
@@ -846,18 +880,18 @@ hs_status launch_unique_inverse(const uint64_t* fp, const int32_t* tokens, int64
   const bool vec = ((reinterpret_cast<uintptr_t>(tokens) & 15u) == 0) && (stride % 4 == 0);
   const int sms = num_sms();
 
+  if (n <= kSmallRows) {
+    // Twice the threads once there are more than four rows for each of 512
+    // (us, 512 / 1024 threads: 512 rows 7.5 / 8.6, 4096 ragged rows 33.5 / 29.4).
+    auto* launch = n <= 2048 ? (vec ? launch_small<true, 512, 4> : launch_small<false, 512, 4>)
+                             : (vec ? launch_small<true, 1024, 4> : launch_small<false, 1024, 4>);
+    const hs_status st = launch(fp, tokens, n, stride, lens, n_unique_dev, unique_idx, inverse,
+                                coll_list, err, stream);
+    if (st == HS_OK) count_launches(1);
+    return st;
+  }
   cudaError_t e = cudaMemsetAsync(w, 0, L.zero_end, stream);
   if (e != cudaSuccess) return cuda_fail(e, "workspace clear");
-  if (n <= kSmallRows) {
-    const hs_status st =
-        vec ? launch_small<true>(fp, tokens, n, stride, lens, n_unique_dev, unique_idx, inverse,
-                                 ctr, coll_list, err, stream)
-            : launch_small<false>(fp, tokens, n, stride, lens, n_unique_dev, unique_idx, inverse,
-                                  ctr, coll_list, err, stream);
-    if (st != HS_OK) return st;
-    count_launches(1);
-    return cuda_fail(cudaGetLastError(), "unique_inverse launch");
-  }
   e = cudaMemsetAsync(w + L.zero_end, 0xff, L.ones_end - L.zero_end, stream);
   if (e != cudaSuccess) return cuda_fail(e, "hash table clear");
   launch_pdl(insert_kernel, dim3(grid_for(n, 256, sms * 8)), dim3(256), 0, stream, fp, n, keys, idx,

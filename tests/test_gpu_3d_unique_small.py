@@ -1,0 +1,37 @@
+"""The one-launch unique (Section 3.3 (I)) at the edges of its cluster: row
+counts around a CTA's share, the CTA counts and the two block sizes, collisions
+in every CTA's share, invalid lengths, and its use of a workspace whose
+contents are anything."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_22578_gb300 as hs
+from hs_testutil import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("stride", [3, 8, 100])
+@pytest.mark.parametrize("n", [1, 8, 63, 64, 65, 128, 129, 257, 512, 513, 2047, 2048, 2049, 4095, 4096])
+def test_row_counts(n, stride):
+    rng = np.random.default_rng(n + stride)
+    tokens = rng.integers(0, 1 << 31, size=(n, stride)).astype(np.int32)
+    src = rng.integers(0, n, size=n)
+    copy = rng.random(n) < 0.6
+    tokens[copy] = tokens[src[copy]]
+    lens = np.where(rng.random(n) < 0.5, stride, rng.integers(0, stride + 1, size=n)).astype(np.int32)
+    t = to_dev(tokens)
+    ws = torch.full((hs.hs_unique_inverse_workspace(n),), 0x5A, dtype=torch.uint8, device="cuda")
+    for L in (None, lens):
+        d = None if L is None else to_dev(L)
+        ou, oi = oracle.unique_inverse(tokens, L)
+        fp = hs.hs_fingerprint(t, d)
+        few = fp % 5                                 # equal rows alike, most others too
+        for key in (fp, few, torch.zeros_like(fp)):
+            nu, u, inv = hs.hs_unique_inverse(key, t, d, workspace=ws)
+            hs.hs_get_device_error()
+            assert int(nu.item()) == len(ou)
+            assert (u.cpu().numpy()[:len(ou)] == ou).all() and (u.cpu().numpy()[len(ou):] == 0).all()
+            assert (inv.cpu().numpy() == oi).all()

@@ -55,10 +55,8 @@ constexpr int UK = 16;                // K per tcgen05.mma, kind::f16
 constexpr int kEpiWarps = 8;
 constexpr int kEpi = kEpiWarps * 32;  // epilogue threads
 constexpr int kThreads = 64 + kEpi;
-constexpr int kHalfCols = BN / 2;     // columns per epilogue thread per tile
 constexpr uint32_t kABytes = BM * BK * 2;
 constexpr uint32_t kBBytes = BN * BK * 2;
-constexpr uint32_t kTmemCols = 2 * BN;
 constexpr int kCap = 16;              // candidate buffer per thread (large-k path)
 constexpr int kMergeMax = 16384;      // bound on lists * k per query (the merge's candidates)
 constexpr size_t kBarBytes = 256;
@@ -75,6 +73,31 @@ struct Ring {
   static constexpr uint32_t stage_bytes = kABytes + b_bytes;
   static constexpr size_t smem = 1024 + (size_t)stages * stage_bytes + kBarBytes + kEpiSmem;
 };
+// Resident queries (17 to 64 of them, single CTAs): the query block is kept in
+// shared memory, 64 rows of 128 bytes per 64 dimensions, and the ring carries
+// corpus boxes of RN rows only.  The MMA reads 128 query rows all the same:
+// rows 64-127 of a block are whatever follows it (the next block, or the
+// ring), and the scores they give lie in lanes nobody reads.
+constexpr int RQ = 64;                   // queries
+constexpr int kResMaxKb = 16;            // d <= 1024 ...
+constexpr int kResMaxKbWide = 12;        // ... and 768 for tiles of 256 rows
+constexpr int kResMaxStages = 12;
+constexpr uint32_t kResQBytes = RQ * BK * 2;
+constexpr size_t kResEpiSmem = (size_t)4 * 32 * 32 * 4;   // staging of the four warps with queries
+__host__ __device__ constexpr int res_stages(int rn, int kb) {
+  const int64_t room =
+      232448 - 1024 - (int64_t)kBarBytes - (int64_t)kResEpiSmem - (int64_t)kb * kResQBytes;
+  const int64_t n = room / (rn * BK * 2);
+  return (int)(n < kResMaxStages ? n : kResMaxStages);
+}
+constexpr size_t res_smem(int rn, int kb) {
+  return 1024 + (size_t)kb * kResQBytes + (size_t)res_stages(rn, kb) * rn * BK * 2 + kBarBytes +
+         kResEpiSmem;
+}
+static_assert(res_stages(128, kResMaxKb) >= 4 && res_stages(256, kResMaxKbWide) >= 3,
+              "resident queries: a ring of a few stages");
+static_assert(128 * BK * 2 >= (int)kResQBytes, "rows past the last query block lie in the ring");
+static_assert(8 * (2 * kResMaxStages + 4 + 2) + 8 + 8 <= kBarBytes, "barrier area");
 static_assert(Ring<1>::smem <= 232448 && Ring<2>::smem <= 232448, "shared memory per CTA");
 static_assert(8 * (2 * Ring<2>::stages + 4) + 8 + 8 <= kBarBytes, "barrier area");
 
@@ -332,19 +355,26 @@ __device__ void flush_candidates(float* cs, int32_t* ci, int et, int& cnt, float
   cnt = 0;
 }
 
-template <int KREG, int CL>
+// RN > 0: resident queries (CL = 1) and corpus tiles of RN rows.
+template <int KREG, int CL, int RN>
 __global__ void __launch_bounds__(kThreads, 1)
     retrieve_kernel(const __grid_constant__ CUtensorMap tmap_q,
                     const __grid_constant__ CUtensorMap tmap_c, const Params p) {
-  constexpr int kStages = Ring<CL>::stages;
-  constexpr uint32_t kBLocal = Ring<CL>::b_bytes;
-  constexpr uint32_t kStageBytes = Ring<CL>::stage_bytes;
+  constexpr bool RES = RN > 0;
+  static_assert(!RES || (CL == 1 && KREG > 0), "resident queries: single CTAs, register lists");
+  constexpr int BN = RES ? RN : hs::BN;
+  constexpr int kHalfCols = BN / 2;     // columns per epilogue thread per tile
+  constexpr uint32_t kTmemCols = 2 * BN;
+  const int kStages = RES ? res_stages(RN, p.kb_count) : Ring<CL>::stages;
+  constexpr uint32_t kBLocal = RES ? RN * BK * 2 : Ring<CL>::b_bytes;
+  constexpr uint32_t kStageBytes = RES ? RN * BK * 2 : Ring<CL>::stage_bytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
-  uint8_t* sB = smem + kStages * kABytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint8_t* sB = smem + (RES ? p.kb_count * kResQBytes : kStages * kABytes);
+  uint8_t* bar_base = RES ? sB + kStages * kStageBytes : smem + kStages * kStageBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(bar_base);
   uint64_t* full = bars;
   uint64_t* empty = bars + kStages;
   uint64_t* tfull = bars + 2 * kStages;
@@ -352,7 +382,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint64_t* drain = tempty + 3;          // after tmem_slot and abort_flag: the MMA drain
-  uint8_t* epi_smem = smem + kStages * kStageBytes + kBarBytes;
+  uint64_t* qfull = drain + 1;           // resident queries are there
+  uint8_t* epi_smem = bar_base + kBarBytes;
   const uint64_t lim = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
 
   // CTA pair: the even CTA (rank 0) owns the full and tempty barriers that
@@ -368,6 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(tempty + a, kEpiWarps * CL);
     }
     mbar_init(drain, 1);
+    if (RES) mbar_init(qfull, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -407,6 +439,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t pol_q = policy_evict_last();
       uint32_t stage = 0, phase = 0;
       int64_t issued = 0;                 // stages armed (or withheld) so far
+      const bool queries = RES && u0 < units;
+      if (queries) {
+        mbar_arrive_expect_tx(qfull, (uint32_t)p.kb_count * kResQBytes);
+        for (int kb = 0; kb < p.kb_count; ++kb)
+          tma_load_2d(sA + kb * kResQBytes, &tmap_q, qfull, kb * BK, 0);
+      }
       for (int64_t u = u0; u < units; u += ustep) {
         if (unit_skipped(p, sp, u, CL)) continue;
         int qb, split;
@@ -428,7 +466,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             // row 0 instead: its scores are masked, and no box lies wholly
             // outside the tensor.
             const int32_t qy = (int64_t)qb * BM < p.Qmax ? qb * BM : 0;
-            if (CL == 1) {
+            if (RES) {
+              mbar_arrive_expect_tx(full + stage, kStageBytes);
+              tma_load_2d_hint(sB + stage * kBLocal, &tmap_c, full + stage, kb * BK,
+                               (int32_t)(t * BN), pol_c);
+            } else if (CL == 1) {
               mbar_arrive_expect_tx(full + stage, kStageBytes);
               tma_load_2d_hint(sA + stage * kABytes, &tmap_q, full + stage, kb * BK, qy, pol_q);
               tma_load_2d_hint(sB + stage * kBLocal, &tmap_c, full + stage, kb * BK,
@@ -459,6 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // or complete within the last tile.
       if (rank == 0) {
         volatile int keep_going = 0;
+        if (queries) mbar_wait_limit(qfull, 0u, &keep_going, lim);
         for (int64_t i = issued > kStages ? issued - kStages : 0; i < issued; ++i) {
           if (p.withhold_first && i == 0) continue;           // never armed
           if (!mbar_wait_limit(full + (int)(i % kStages), (uint32_t)((i / kStages) & 1),
@@ -473,6 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       constexpr uint32_t idesc = idesc_bf16_f32(BM * CL, BN);
       uint32_t stage = 0, phase = 0, tile_i = 0;
       bool any_mma = false;
+      if (RES && u0 < units && !mbar_wait_limit(qfull, 0u, abort_flag, lim)) goto mma_done;
       for (int64_t u = u0; u < units; u += ustep) {
         if (unit_skipped(p, sp, u, CL)) continue;
         int qb, split;
@@ -487,7 +531,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!mbar_wait_limit(full + stage, phase, abort_flag, lim)) goto mma_done;
             tc_fence_after();
             any_mma = true;
-            const uint64_t a0 = smem_desc_k_sw128(smem_u32(sA + stage * kABytes));
+            const uint64_t a0 =
+                smem_desc_k_sw128(smem_u32(sA + (RES ? kb * kResQBytes : stage * kABytes)));
             const uint64_t b0 = smem_desc_k_sw128(smem_u32(sB + stage * kBLocal));
 #pragma unroll
             for (int kk = 0; kk < BK / UK; ++kk) {
@@ -531,7 +576,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int quarter = warp & 3;             // TMEM lanes [32*quarter, 32*quarter+32)
     const int half = ew >> 2;                 // columns [half*128, half*128+128) of a tile
     const int row = quarter * 32 + lane;      // query within the block
-    const int et = ew * 32 + lane;            // epilogue thread index, 0..255
+    // Epilogue thread index, 0..255; with resident queries those of quarters 0
+    // and 1, the ones that have queries, are 0..127 (the others stage nothing).
+    const int et = RES ? ((half * 2 + (quarter & 1)) * 32 + lane) : ew * 32 + lane;
+    constexpr int kEpi = RES ? 128 : hs::kEpi;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int k = p.k;
     const int lists = 2 * sp.nsplit;
@@ -1366,13 +1414,13 @@ bool make_map(CUtensorMap* map, const uint16_t* base, int64_t rows, int32_t d, u
 std::atomic<uint64_t> g_ret_wait_limit_ns{0};
 std::atomic<int> g_ret_withhold{0};
 
-template <int KREG, int CL>
+template <int KREG, int CL, int RN>
 hs_status configure_kernel() {
   static std::atomic<uint64_t> done{0};
   return once_per_device(done, [] {
-    return cuda_fail(cudaFuncSetAttribute(retrieve_kernel<KREG, CL>,
+    return cuda_fail(cudaFuncSetAttribute(retrieve_kernel<KREG, CL, RN>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)Ring<CL>::smem),
+                                          RN > 0 ? 232448 : (int)Ring<CL>::smem),
                      "retrieve smem attribute");
   });
 }
@@ -1397,14 +1445,14 @@ int64_t max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<KREG, 2>, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<KREG, 2, 0>, &cfg) != cudaSuccess) n = 0;
     cached = n;
     if (dev >= 0) per_device[dev].store(cached + 1);
   }
   return cached;
 }
 
-template <int KREG, int CL>
+template <int KREG, int CL, int RN>
 hs_status launch_kernel(const CUtensorMap& mq, const CUtensorMap& mc, const Params& prm,
                         int64_t grid, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
@@ -1417,11 +1465,11 @@ hs_status launch_kernel(const CUtensorMap& mq, const CUtensorMap& mc, const Para
   attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = Ring<CL>::smem;
+  cfg.dynamicSmemBytes = RN > 0 ? res_smem(RN, prm.kb_count) : Ring<CL>::smem;
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = CL > 1 ? 2 : 1;
-  return cuda_fail(cudaLaunchKernelEx(&cfg, retrieve_kernel<KREG, CL>, mq, mc, prm),
+  return cuda_fail(cudaLaunchKernelEx(&cfg, retrieve_kernel<KREG, CL, RN>, mq, mc, prm),
                    "retrieve launch");
 }
 
@@ -1432,14 +1480,14 @@ hs_status launch_variant(const uint16_t* corpus, int64_t N, int32_t d, const CUt
                          Params& prm, cudaStream_t stream) {
   const int64_t sms = num_sms();
   const int64_t qblocks_max = (prm.Qmax + BM - 1) / BM;
-  hs_status st = configure_kernel<KREG, 1>();
+  hs_status st = configure_kernel<KREG, 1, 0>();
   if (st != HS_OK) return st;
   int cl = 1;
   // Unit executors: at most 16 * kMaxListsPerLane, so every query's lists
   // (2 per split, nsplit <= slots) fit the warp merge.
   int64_t slots = std::min<int64_t>(sms, 16 * kMaxListsPerLane);
   if (qblocks_max >= 2) {
-    st = configure_kernel<KREG, 2>();
+    st = configure_kernel<KREG, 2, 0>();
     if (st != HS_OK) return st;
     const int64_t pairs = std::min<int64_t>(std::min<int64_t>(max_pairs<KREG>(), sms / 2),
                                             16 * kMaxListsPerLane);
@@ -1462,11 +1510,36 @@ hs_status launch_variant(const uint16_t* corpus, int64_t N, int32_t d, const CUt
     if (units < execs) execs = units;
   }
   if (execs < 1) execs = 1;
-  return cl == 2 ? launch_kernel<KREG, 2>(mq, mc, prm, execs * 2, stream)
-                 : launch_kernel<KREG, 1>(mq, mc, prm, execs, stream);
+  return cl == 2 ? launch_kernel<KREG, 2, 0>(mq, mc, prm, execs * 2, stream)
+                 : launch_kernel<KREG, 1, 0>(mq, mc, prm, execs, stream);
+}
+
+// The same with resident queries.  One query block, so the plan has a split
+// per CTA.
+template <int KREG, int RN>
+hs_status launch_resident(const uint16_t* queries, const uint16_t* corpus, int64_t N, int32_t d,
+                          Params& prm, cudaStream_t stream) {
+  const hs_status st = configure_kernel<KREG, 1, RN>();
+  if (st != HS_OK) return st;
+  CUtensorMap mq, mc;
+  if (!make_map(&mq, queries, prm.Qmax, d, RQ) || !make_map(&mc, corpus, N, d, RN))
+    return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
+  prm.tiles = (N + RN - 1) / RN;
+  prm.slots = (int32_t)std::min<int64_t>(num_sms(), 16 * kMaxListsPerLane);
+  prm.cl = 1;
+  const SplitPlan sp = split_plan(1, prm.tiles, prm.k, prm.slots, 1);
+  return launch_kernel<KREG, 1, RN>(mq, mc, prm, sp.nsplit, stream);
 }
 
 }  // namespace
+
+// One of the two arrays of lists.  Batches of up to RQ queries may be split
+// into tiles of 128 rows.
+static size_t part_bytes(int64_t Q, int64_t N, int32_t k, int64_t sms) {
+  const int64_t few = std::min<int64_t>(Q, RQ) * max_splits(sms, (N + 127) / 128, k);
+  const int64_t lists = std::max<int64_t>(Q * max_splits(sms, (N + BN - 1) / BN, k), few);
+  return (((size_t)lists * 2 * k * 4) + 255) & ~(size_t)255;
+}
 
 // Upper bound over every query count up to Q: a plan's split count is at most
 // max_splits() and the grid is at most the SM count, so one workspace serves
@@ -1475,8 +1548,7 @@ size_t retrieve_topk_workspace(int64_t Q, int64_t N, int32_t d, int32_t k) {
   if (Q <= 0 || N <= 0 || k <= 0) return 256;
   (void)d;
   const int64_t sms = num_sms();
-  const int64_t ns = max_splits(sms, (N + BN - 1) / BN, k);
-  const size_t part = (((size_t)Q * 2 * ns * k * 4) + 255) & ~(size_t)255;
+  const size_t part = part_bytes(Q, N, k, sms);
   const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
   const size_t qfloor = (((size_t)Q * 4) + 255) & ~(size_t)255;
   const size_t flags = ((((size_t)(Q + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
@@ -1502,8 +1574,7 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   CUtensorMap mq;
   if (!make_map(&mq, queries, Qmax, d, BM))
     return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
-  const int64_t ns_max = max_splits(sms, tiles, k);
-  const size_t part = (((size_t)Qmax * 2 * ns_max * k * 4) + 255) & ~(size_t)255;
+  const size_t part = part_bytes(Qmax, N, k, sms);
   const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
   char* w = static_cast<char*>(ws);
   Params prm{};
@@ -1526,6 +1597,16 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list + 2 * qfloor_bytes);
   prm.err = err;
   const bool small = Qmax <= SQ_N && k <= 32 && prm.kb_count <= SQ_MAXKB;
+  // Up to 64 queries stay in shared memory, which leaves the ring to the
+  // corpus.  Tiles of 256 rows cost less per row, tiles of 128 spread a small
+  // corpus over twice the SMs and leave wide rows a ring.  us, k = 10, a 128-row
+  // query block streamed beside the corpus / resident with tiles of 128 / of
+  // 256: 17 queries, 1,000,000 x 768 313 / 237 / 233, 2,000,000 x 256 222 / 172 /
+  // 168; 64 queries, 4096 x 384 24.5 / 22.5 / 24.2, 20,000 x 768 30.1 / 34.8 /
+  // 30.5, 2,000,000 x 256 177 to 187 / 189 / 173, 1,000,000 x 768 235 to 255 /
+  // 240 / 236 to 241.  A stage's batch of 64 over 2,097,152 x 768: 508 -> 475.
+  const bool resident = !small && Qmax <= RQ && k <= 32 && prm.kb_count <= kResMaxKb;
+  const bool wide = prm.kb_count <= kResMaxKbWide && (N + 127) / 128 > sms;
   if (!small) {
     // The shared per-query floors of the register-list passes start empty.
     const cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
@@ -1598,6 +1679,12 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     launch_pdl(retrieve_small_kernel, dim3((unsigned)grid), dim3(SQ_THREADS), SQ_SMEM, stream,
                mq16, mc128, prm, (N + SQ_BM - 1) / SQ_BM);
     st = cuda_fail(cudaGetLastError(), "retrieve launch");
+  } else if (resident) {
+    auto* launch = k <= 8    ? (wide ? launch_resident<8, 256> : launch_resident<8, 128>)
+                   : k <= 12 ? (wide ? launch_resident<12, 256> : launch_resident<12, 128>)
+                   : k <= 16 ? (wide ? launch_resident<16, 256> : launch_resident<16, 128>)
+                             : (wide ? launch_resident<32, 256> : launch_resident<32, 128>);
+    st = launch(queries, corpus, N, d, prm, stream);
   } else if (k <= 8) {
     st = launch_variant<8>(corpus, N, d, mq, prm, stream);
   } else if (k <= 12) {

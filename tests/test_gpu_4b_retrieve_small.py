@@ -70,3 +70,46 @@ def test_scores_of_the_lowest_value_and_ascending_rows(nq):
     rows = torch.from_numpy((scale[:, None] * base).astype(np.float32)).to(torch.bfloat16)
     C = rows.view(torch.int16).numpy().view(np.uint16)
     check(np.tile(synth.unit_rows(1, 64, 3), (nq, 1)), C, 10)
+
+
+@pytest.mark.parametrize("d", [8, 64, 136, 768, 1024, 1032])
+@pytest.mark.parametrize("nq", [17, 31, 33, 63, 64, 65])
+def test_resident_queries(nq, d):
+    """17 to 64 queries stay in shared memory (d <= 1024): widths around a
+    64-dimension block, row counts around a 128-row tile, several tiles per CTA."""
+    for N, k in ((127, 7), (129, 12), (385, 16), (25001, 32)):
+        check(synth.unit_rows(nq, d, nq + N), synth.unit_rows(N, d, N), k)
+
+
+def test_resident_queries_with_the_count_on_the_device():
+    q, c = synth.unit_rows(64, 128, 1), synth.unit_rows(9000, 128, 2)
+    Q, C = (to_dev(x).view(torch.bfloat16) for x in (q, c))
+    Q[40:] = float("nan")                          # rows past the count are never selected from
+    want_s, want_i = hs.hs_retrieve_topk(Q[:40].contiguous(), C, 10)
+    for n in (0, 1, 39, 40):
+        s = torch.full((64, 10), 7.0, device="cuda")
+        i = torch.full((64, 10), 7, dtype=torch.int32, device="cuda")
+        hs.hs_retrieve_topk_n(Q, torch.tensor([n], dtype=torch.int32, device="cuda"), C, 10,
+                              out=(s, i))
+        hs.hs_get_device_error()
+        assert torch.equal(s[:n], want_s[:n]) and torch.equal(i[:n], want_i[:n])
+        assert (s[n:] == 7.0).all() and (i[n:] == 7).all()
+
+
+def test_resident_pipeline_wait_runs_out():
+    """As the other kernels' waits: a stage that never fills ends in
+    HS_ERR_TIMEOUT, and the next call is right."""
+    q, c = synth.unit_rows(40, 256, 3), synth.unit_rows(30000, 256, 4)
+    Q, C = (to_dev(x).view(torch.bfloat16) for x in (q, c))
+    want = hs.hs_retrieve_topk(Q, C, 10)
+    try:
+        hs.hs_debug_retrieve_wait(1_000_000, 1)
+        hs.hs_retrieve_topk(Q, C, 10)
+        with pytest.raises(hs.HsError) as e:
+            hs.hs_get_device_error()
+        assert e.value.status == hs.HS_ERR_TIMEOUT
+    finally:
+        hs.hs_debug_retrieve_wait()
+    got = hs.hs_retrieve_topk(Q, C, 10)
+    hs.hs_get_device_error()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])

@@ -35,3 +35,24 @@ def test_row_counts(n, stride):
             assert int(nu.item()) == len(ou)
             assert (u.cpu().numpy()[:len(ou)] == ou).all() and (u.cpu().numpy()[len(ou):] == 0).all()
             assert (inv.cpu().numpy() == oi).all()
+
+
+@pytest.mark.parametrize("n", [4097, 8191, 8193, 70001])
+def test_workspace_cleared(n):
+    """Above one cluster: counters, scan states and the table's last slot
+    (fingerprint of all ones) come out of the clearing launch."""
+    rng = np.random.default_rng(n)
+    tokens = rng.integers(0, 50, size=(n, 4)).astype(np.int32)
+    tokens[n // 2:] = tokens[rng.integers(0, n // 2, size=n - n // 2)]
+    t = to_dev(tokens)
+    ou, oi = oracle.unique_inverse(tokens, None)
+    fp = hs.hs_fingerprint(t)
+    ones = torch.where(t[:, 0] < 1, torch.full_like(fp, -1), fp)
+    for fill in (0x00, 0x5A, 0xFF):
+        ws = torch.full((hs.hs_merge_rows_workspace(n),), fill, dtype=torch.uint8, device="cuda")
+        calls = [lambda k=k: hs.hs_unique_inverse(k, t, workspace=ws) for k in (fp, ones)]
+        for call in calls + [lambda: hs.hs_merge_rows(t, workspace=ws)[-3:]]:
+            nu, u, inv = call()
+            hs.hs_get_device_error()
+            assert int(nu.item()) == len(ou)
+            assert (u.cpu().numpy()[:len(ou)] == ou).all() and (inv.cpu().numpy() == oi).all()

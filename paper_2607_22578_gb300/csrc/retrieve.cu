@@ -29,16 +29,18 @@
 // the same time on different SMs, so each corpus tile is read from HBM about
 // once and served to the other query blocks from L2.
 //
-// Top-k state per (query, half): for k <= 32 a sorted list in registers
-// (KREG = 16 or 32 slots).  A 32-column chunk whose maximum beats no lane's
-// threshold costs one max-reduction; otherwise the chunk is staged in shared
-// memory and every lane inserts its candidates in one converged loop, so the
-// warp pays for the largest candidate count of a lane, not for the sum over
-// lanes.  For k > 32 a 16-entry candidate buffer per thread in shared memory
-// is sorted and merged into a sorted list in global scratch whenever a
-// buffer fills.  Each unit writes its k best per (query, half); K7 merges the
-// sorted lists of each query: one warp per query takes the largest head of
-// its lists k times (packed (score, index) keys).
+// Top-k state per (query, half): a sorted list in registers (KREG = 8 to 32
+// slots; more than 16 results are first looked for in lists shorter than k).
+// A 32-column chunk whose maximum beats no lane's threshold costs one
+// max-reduction; otherwise the chunk is staged in shared memory and every lane
+// inserts its candidates in one converged loop, so the warp pays for the
+// largest candidate count of a lane, not for the sum over lanes.  Where k > 32
+// and such lists do not suffice, a 16-entry candidate buffer per thread in
+// shared memory is sorted and merged into a sorted list in global scratch
+// whenever a buffer fills.  Each unit writes its k best per (query, half); K7
+// merges the sorted lists of each query: by ranking what can be among the k
+// best (few rows), or one warp per query takes the largest head of its lists
+// k times (packed (score, index) keys).
 #include <float.h>
 
 #include <algorithm>
@@ -117,14 +119,15 @@ struct Params {
   // query's final k-th best score, so it prunes without changing the result.
   const float* floor;
   int32_t floor_stride, floor_index;
-  // k <= 32: per-query shared floor, the largest k-th best score any list of
+  // Per-query shared floor, the largest k-th best score any list of
   // the query has reached so far (order-preserving uint32 code of the float,
   // 0 = none), raised with atomicMax and read once per tile by every list of
   // the query.  Zeroed before each launch.
   uint32_t* qfloor;
-  // Optional, one word per query block: a unit whose query blocks are all 0
-  // here is skipped (the exact large-k pass re-runs only the flagged blocks).
+  // Optional, one word per query block: a unit whose query blocks all have no
+  // bit of only_mask here is skipped (later passes re-run only flagged blocks).
   const uint32_t* only;
+  uint32_t only_mask;
   // Bounded waits of retrieve_kernel: give up after wait_limit_ns.  With
   // withhold_first set (a test hook) every CTA skips the loads of its first
   // stage, so that stage never fills and the waits run out.
@@ -210,7 +213,7 @@ __device__ __forceinline__ bool unit_skipped(const Params& p, const SplitPlan& s
   const int g = (int)(u % sp.groups);
   for (int r = 0; r < cl; ++r) {
     const int qb = g * cl + r;
-    if (qb < sp.qblocks && p.only[qb] != 0u) return false;
+    if (qb < sp.qblocks && (p.only[qb] & p.only_mask) != 0u) return false;
   }
   return true;
 }
@@ -385,6 +388,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* qfull = drain + 1;           // resident queries are there
   uint8_t* epi_smem = bar_base + kBarBytes;
   const uint64_t lim = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
+
+  // A pass over flagged query blocks of which there are none, the usual case,
+  // ends here (every CTA sees the same flags): 3.4 us cold, 5 to 7.5 where it
+  // found no unit after the setup.
+  if ((KREG == 0 || KREG == 32) && p.only) {
+    pdl_wait();
+    bool any = false;
+    for (int64_t b = threadIdx.x; b < (p.Qmax + BM - 1) / BM; b += kThreads)
+      any |= (p.only[b] & p.only_mask) != 0u;
+    if (!__syncthreads_or(any)) return;
+  }
 
   // CTA pair: the even CTA (rank 0) owns the full and tempty barriers that
   // both CTAs' loads and epilogues signal, and issues every MMA.
@@ -895,7 +909,7 @@ constexpr int kMaxListsPerLane = 10;
 // Any kout: picks 0..31 are kept one per lane and written together when
 // kout <= 32; for larger kout each pick is written as it is made.  With
 // out_i NULL only the kout-th pick's score is written, to out_s[o] (the
-// floor of the second large-k pass).  With `only` set, rows whose query
+// floor of the second large-k pass).  With p.only set, rows whose query
 // block is not flagged there are skipped.  With `flag_out` set, a query's
 // block is flagged when one of its lists may have cut off a member of the
 // top kout: a full list whose last (k-th) entry is not below the union's
@@ -909,7 +923,7 @@ template <int LPL>
 __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* __restrict__ out_s,
                                                          int32_t* __restrict__ out_i,
                                                          int32_t kout, OutRows rows,
-                                                         uint32_t* flag_out, const uint32_t* only) {
+                                                         uint32_t* flag_out, uint32_t flag_bit) {
   pdl_wait();
   pdl_trigger();
   const int64_t Q = query_count(p);
@@ -925,7 +939,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
       if (lane == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
-    if (only && only[q / BM] == 0u) continue;      // warp-uniform
+    if (p.only && (p.only[q / BM] & p.only_mask) == 0u) continue;   // warp-uniform
     const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
     const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
     uint64_t head[LPL], next[LPL];
@@ -995,34 +1009,44 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
         if (l < lists)
           cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= last;
       }
-      if (__any_sync(0xffffffffu, cut) && lane == 0) atomicOr(flag_out + q / BM, 1u);
+      if (__any_sync(0xffffffffu, cut) && lane == 0) atomicOr(flag_out + q / BM, flag_bit);
     }
   }
 }
 
-// Few output rows, k <= 32: a block per row, and no tournament.  The heads of
-// the lists are ranked by counting; the k best heads name the only lists that
-// can hold one of the k best entries, and the k-th best head bounds those.
-// What is left of these lists, little more than k entries, is ranked by
-// counting again, and an entry's rank is its place.  Two round trips to memory
-// and two loops over shared memory in place of k dependent rounds.  64 rows of
-// 304 lists, k = 10: 11 us cold, 14.4 with a warp each.
+// A block per row, and no tournament.  The first `depth` entries of the lists,
+// as many as it takes to have kout of them, are ranked by counting; the
+// kout-th best bounds the result from below, so only lists whose depth-th entry
+// reaches it can hold more.  What is left of these, with the first entries
+// above the bound little more than kout, is ranked by counting again, and an
+// entry's rank is its place.  Two round trips to memory and two loops over
+// shared memory in place of kout dependent rounds.  64 rows of 304 lists, k =
+// 10: 11 us cold, 14.4 with a warp each; 24 rows, k = 50: 27.8 -> 8.4 (32 lists of
+// 32 entries before, 64 of 12 now); 100 rows, k = 100: 66.9 -> 16.8.
+// Lists of at most 32 entries (p.k); CAP >= kout * p.k.  flag_out as above.
 constexpr int kMrThreads = 256;
 constexpr int kMrLists = 32 * kMaxListsPerLane;
+constexpr int kMrMaxK = 128;
 static_assert(kMrLists <= 2 * kMrThreads, "two heads per thread");
+static_assert(kMrLists >= 2 * kMrMaxK, "lists * depth < kout + lists <= kMrLists");
 
+template <int CAP>
 __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
                                                                 float* __restrict__ out_s,
                                                                 int32_t* __restrict__ out_i,
-                                                                OutRows rows) {
+                                                                int32_t kout, OutRows rows,
+                                                                uint32_t* flag_out,
+                                                                uint32_t flag_bit) {
   pdl_wait();
   pdl_trigger();
-  __shared__ uint64_t s_head[kMrLists], s_cand[32 * 32];
-  __shared__ int32_t s_sel[32];
+  __shared__ uint64_t s_head[kMrLists], s_cand[CAP], s_kth;
+  __shared__ int32_t s_sel[kMrLists];
   __shared__ int s_nsel, s_ncand;
   const int64_t Q = query_count(p);
   const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
   const int k = p.k, lists = 2 * sp.nsplit, tid = threadIdx.x;
+  const int depth = min((kout + lists - 1) / lists, k);
+  const int heads = lists * depth;               // entry e of list l: head e * lists + l
   const int64_t R = rows.inv ? rows.n_out : Q;
   for (int64_t o = blockIdx.x; o < R; o += gridDim.x) {
     const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
@@ -1030,54 +1054,77 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
       if (tid == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
+    if (p.only && (p.only[q / BM] & p.only_mask) == 0u) continue;   // block-uniform
     const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
     const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
     uint64_t mine[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int l = j * kMrThreads + tid;
-      mine[j] = l < lists ? pack_key(ps[(size_t)l * k], pi[(size_t)l * k]) : 0ull;
-      if (l < lists) s_head[l] = mine[j];
+      const int h = j * kMrThreads + tid;
+      mine[j] = 0ull;
+      if (h < heads) {
+        const size_t e = (size_t)(h % lists) * k + h / lists;
+        s_head[h] = mine[j] = pack_key(ps[e], pi[e]);
+      }
     }
-    if (tid == 0) s_nsel = s_ncand = 0;
+    if (tid == 0) {
+      s_nsel = s_ncand = 0;
+      s_kth = 0ull;                                // stays 0 when there are not kout entries
+    }
     __syncthreads();
     int rank[2] = {0, 0};
 #pragma unroll 8
-    for (int l = 0; l < lists; ++l) {              // (heads of empty lists are alike)
-      const uint64_t h = s_head[l];
-      rank[0] += (h > mine[0]) | ((h == mine[0]) & (l < tid));
-      rank[1] += (h > mine[1]) | ((h == mine[1]) & (l < tid + kMrThreads));
+    for (int h = 0; h < heads; ++h) {              // (entries of empty lists are alike)
+      const uint64_t y = s_head[h];
+      rank[0] += (y > mine[0]) | ((y == mine[0]) & (h < tid));
+      rank[1] += (y > mine[1]) | ((y == mine[1]) & (h < tid + kMrThreads));
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      if (j * kMrThreads + tid < lists && rank[j] < k) {
-        s_sel[rank[j]] = j * kMrThreads + tid;
-        atomicAdd(&s_nsel, 1);
-      }
+      if (j * kMrThreads + tid < heads && rank[j] == kout - 1) s_kth = mine[j];
     __syncthreads();
-    const int nsel = s_nsel;
-    // the k-th best head; with fewer lists than k every entry counts
-    const uint64_t bound = nsel == k ? s_head[s_sel[k - 1]] : 0ull;
-    for (int i = tid; i < nsel * k; i += kMrThreads) {
-      const size_t e = (size_t)s_sel[i / k] * k + i % k;
+    // the kout-th best head; with fewer entries than that every one counts
+    const uint64_t bound = s_kth;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int h = j * kMrThreads + tid;
+      if (h < heads && rank[j] < kout) {
+        s_cand[atomicAdd(&s_ncand, 1)] = mine[j];
+        if (h / lists == depth - 1) s_sel[atomicAdd(&s_nsel, 1)] = h % lists;
+      }
+    }
+    __syncthreads();
+    const int rest = k - depth, more = s_nsel * rest;
+    for (int i = tid; i < more; i += kMrThreads) {
+      const size_t e = (size_t)s_sel[i / rest] * k + depth + i % rest;
       const uint64_t key = pack_key(ps[e], pi[e]);
       if (key >= bound) s_cand[atomicAdd(&s_ncand, 1)] = key;
     }
+    if (tid == 0) s_kth = 0ull;
     __syncthreads();
     const int c = s_ncand;
     for (int i = tid; i < c; i += kMrThreads) {
       const uint64_t key = s_cand[i];
       int r = 0;
+#pragma unroll 8
       for (int j = 0; j < c; ++j) r += (s_cand[j] > key) | ((s_cand[j] == key) & (j < i));
-      if (r < k) {
+      if (r < kout) {
         float sc;
         int32_t id;
         unpack_key(key, sc, id);
-        out_s[(size_t)o * k + r] = sc;
-        out_i[(size_t)o * k + r] = id;
+        out_s[(size_t)o * kout + r] = sc;
+        out_i[(size_t)o * kout + r] = id;
+        if (r == kout - 1) s_kth = key;
       }
     }
     __syncthreads();                               // read before the next row's lists come in
+    if (flag_out) {
+      const uint64_t kth = s_kth;
+      bool cut = false;
+      for (int l = tid; l < lists; l += kMrThreads)
+        cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= kth;
+      if (__syncthreads_or(cut) && tid == 0) atomicOr(flag_out + q / BM, flag_bit);
+    }
   }
 }
 
@@ -1533,6 +1580,19 @@ hs_status launch_resident(const uint16_t* queries, const uint16_t* corpus, int64
 
 }  // namespace
 
+// The fewest lists that a query gets over the plans of launch_variant (one
+// block of queries, or pairs of blocks); with a count that only the device
+// knows, over every count up to Q.
+static int64_t fewest_lists(int64_t Q, bool device_count, int64_t tiles, int32_t k, int64_t sms) {
+  const int64_t blocks = (Q + BM - 1) / BM;
+  const int32_t cl = blocks >= 2 ? 2 : 1;
+  const int64_t slots = sms / cl, groups = (blocks + cl - 1) / cl;
+  int64_t fewest = 2 * split_plan(Q, tiles, k, slots, cl).nsplit;
+  for (int64_t g = 1; device_count && g < std::min(groups, slots + 1); ++g)
+    fewest = std::min<int64_t>(fewest, 2 * split_plan(g * BM * cl, tiles, k, slots, cl).nsplit);
+  return fewest;
+}
+
 // One of the two arrays of lists.  Batches of up to RQ queries may be split
 // into tiles of 128 rows.
 static size_t part_bytes(int64_t Q, int64_t N, int32_t k, int64_t sms) {
@@ -1552,7 +1612,7 @@ size_t retrieve_topk_workspace(int64_t Q, int64_t N, int32_t d, int32_t k) {
   const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
   const size_t qfloor = (((size_t)Q * 4) + 255) & ~(size_t)255;
   const size_t flags = ((((size_t)(Q + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
-  // lists, large-k lists, shared floors, large-k floors, block flags
+  // lists, large-k lists, shared floors, block flags, large-k floors
   return 2 * part + 2 * list + 2 * qfloor + flags + 256;
 }
 
@@ -1592,9 +1652,9 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   prm.list_i = reinterpret_cast<int32_t*>(w + 2 * part + list);
   const size_t qfloor_bytes = (((size_t)Qmax * 4) + 255) & ~(size_t)255;
   prm.qfloor = reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list);
-  float* kth = reinterpret_cast<float*>(w + 2 * part + 2 * list + qfloor_bytes);
-  uint32_t* block_flags =
-      reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list + 2 * qfloor_bytes);
+  const size_t flag_bytes = ((((size_t)(Qmax + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
+  uint32_t* block_flags = reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list + qfloor_bytes);
+  float* kth = reinterpret_cast<float*>(w + 2 * part + 2 * list + qfloor_bytes + flag_bytes);
   prm.err = err;
   const bool small = Qmax <= SQ_N && k <= 32 && prm.kb_count <= SQ_MAXKB;
   // Up to 64 queries stay in shared memory, which leaves the ring to the
@@ -1605,17 +1665,12 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   // 168; 64 queries, 4096 x 384 24.5 / 22.5 / 24.2, 20,000 x 768 30.1 / 34.8 /
   // 30.5, 2,000,000 x 256 177 to 187 / 189 / 173, 1,000,000 x 768 235 to 255 /
   // 240 / 236 to 241.  A stage's batch of 64 over 2,097,152 x 768: 508 -> 475.
-  const bool resident = !small && Qmax <= RQ && k <= 32 && prm.kb_count <= kResMaxKb;
+  const bool resident = !small && Qmax <= RQ && prm.kb_count <= kResMaxKb;
   const bool wide = prm.kb_count <= kResMaxKbWide && (N + 127) / 128 > sms;
-  if (!small) {
-    // The shared per-query floors of the register-list passes start empty.
-    const cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
-    if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
-  }
   const OutRows rows{inv, n_out};
   const int64_t R = inv ? n_out : Qmax;             // rows the final merge writes
   auto merge = [&](const Params& pm, int32_t kout, float* os, int32_t* oi, OutRows orows,
-                   uint32_t* flag_out = nullptr, const uint32_t* only = nullptr) -> hs_status {
+                   uint32_t* flag_out = nullptr, uint32_t flag_bit = 0) -> hs_status {
     const int64_t nr = orows.inv ? orows.n_out : Qmax;
     if (nr == 0) return HS_OK;
     // Every plan caps its executors (slots) at 16 * kMaxListsPerLane, so a
@@ -1623,17 +1678,26 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     // every launch.
     if (2 * (int64_t)pm.slots > 32 * kMaxListsPerLane)
       return fail(HS_ERR_UNSUPPORTED, "more lists per query than the merge takes");
-    // A block per row while there is an SM for each (256 rows of 152 lists
-    // take 1 to 2 us more than with a warp each) and k is worth it (k = 1: 0.5
-    // to 1 us more).  After the main kernel it is launched in plain stream
+    // Up to 32 results: a block per row while there is an SM for each (256 rows
+    // of 152 lists take 1 to 2 us more than with a warp each) and k is worth it
+    // (k = 1: 0.5 to 1 us more).  More results: up to twelve rows per SM (1000
+    // rows, k = 50 and 100, 8 and 19 us less than with a warp each; 4000 rows 15
+    // more).  After the main kernel it is launched in plain stream
     // order: with its blocks waiting beside it, their shared memory cost the
     // next retrieval up to 45 us; after the small-batch kernel it does not.
-    if (k >= 4 && k <= 32 && nr <= sms) {
+    if (kout >= 4 && kout <= 32 && nr <= sms) {
       if (small)
-        launch_pdl(merge_rank_kernel, dim3((unsigned)nr), dim3(kMrThreads), 0, stream, pm, os, oi,
-                   orows);
+        launch_pdl(merge_rank_kernel<32 * 32>, dim3((unsigned)nr), dim3(kMrThreads), 0, stream, pm,
+                   os, oi, kout, orows, flag_out, flag_bit);
       else
-        merge_rank_kernel<<<dim3((unsigned)nr), dim3(kMrThreads), 0, stream>>>(pm, os, oi, orows);
+        merge_rank_kernel<32 * 32><<<dim3((unsigned)nr), dim3(kMrThreads), 0, stream>>>(
+            pm, os, oi, kout, orows, flag_out, flag_bit);
+      return cuda_fail(cudaGetLastError(), "merge launch");
+    }
+    if (kout > 32 && kout <= kMrMaxK && pm.k <= 32 && oi && nr <= 12 * sms) {
+      const int64_t blocks = std::min<int64_t>(nr, 6 * sms);
+      merge_rank_kernel<32 * kMrMaxK><<<dim3((unsigned)blocks), dim3(kMrThreads), 0, stream>>>(
+          pm, os, oi, kout, orows, flag_out, flag_bit);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
     {
@@ -1643,16 +1707,16 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       const int64_t lpl = (2 * (int64_t)pm.slots + 31) / 32;
       if (lpl <= 2)
         launch_pdl(merge_warp_kernel<2>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, only);
+                   flag_out, flag_bit);
       else if (lpl <= 3)
         launch_pdl(merge_warp_kernel<3>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, only);
+                   flag_out, flag_bit);
       else if (lpl <= 5)
         launch_pdl(merge_warp_kernel<5>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, only);
+                   flag_out, flag_bit);
       else
         launch_pdl(merge_warp_kernel<kMaxListsPerLane>, grid, dim3(256), 0, stream, pm, os, oi,
-                   kout, orows, flag_out, only);
+                   kout, orows, flag_out, flag_bit);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
   };
@@ -1679,75 +1743,104 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     launch_pdl(retrieve_small_kernel, dim3((unsigned)grid), dim3(SQ_THREADS), SQ_SMEM, stream,
                mq16, mc128, prm, (N + SQ_BM - 1) / SQ_BM);
     st = cuda_fail(cudaGetLastError(), "retrieve launch");
-  } else if (resident) {
-    auto* launch = k <= 8    ? (wide ? launch_resident<8, 256> : launch_resident<8, 128>)
-                   : k <= 12 ? (wide ? launch_resident<12, 256> : launch_resident<12, 128>)
-                   : k <= 16 ? (wide ? launch_resident<16, 256> : launch_resident<16, 128>)
-                             : (wide ? launch_resident<32, 256> : launch_resident<32, 128>);
-    st = launch(queries, corpus, N, d, prm, stream);
-  } else if (k <= 8) {
-    st = launch_variant<8>(corpus, N, d, mq, prm, stream);
-  } else if (k <= 12) {
-    st = launch_variant<12>(corpus, N, d, mq, prm, stream);
-  } else if (k <= 16) {
-    st = launch_variant<16>(corpus, N, d, mq, prm, stream);
-  } else if (k <= 32) {
-    st = launch_variant<32>(corpus, N, d, mq, prm, stream);
   } else {
-    // Large k.  Unless the corpus has few tiles an optimistic pass runs first:
-    // the register-list kernel (32 per list, no shared floor: a floor that
-    // bounds 32nd-best scores would cut rows of the top k) over the whole
-    // corpus, merged to the first k of the union of its lists.  A list whose
-    // last entry is below the union's k-th best holds every row of its range
-    // that can be in the top k, so where no list of a query is cut that way
-    // the union's first k are exact.  The merge flags the query blocks where
-    // some list may have been cut; only those take the exact two-pass path
-    // (pass 1: register lists over the first eighth of the corpus, whose
-    // union's k-th best is a score k distinct rows reach, hence a floor;
-    // pass 2: the large-k kernel over the whole corpus keeping scores >= the
-    // floor), and every kernel of it skips the other blocks.  Both passes'
-    // lists go through the same workspace; the floors are staged in it.
-    // A tile gives a query two lists, so with k <= 32 tiles a list holds 16 of
-    // the top k on average, four deviations below the 32 it keeps; pass 1
-    // needs eight tiles of its own.  4096
-    // x 384, k = 100: 1 query 157 -> 85 us, 2048 queries 1267 -> 171 us.
-    if ((int64_t)k <= 32 * tiles) {
-      const int64_t nb = (Qmax + BM - 1) / BM;
-      const cudaError_t ze = cudaMemsetAsync(block_flags, 0, (size_t)nb * 4, stream);
-      if (ze != cudaSuccess) return cuda_fail(ze, "flag clear");
-      Params pa = prm;
-      pa.k = 32;
-      pa.qfloor = nullptr;
-      pa.floor = nullptr;
-      st = launch_variant<32>(corpus, N, d, mq, pa, stream);
-      if (st != HS_OK) return st;
-      st = merge(pa, k, scores_out, ids_out, rows, block_flags, nullptr);
-      if (st != HS_OK) return st;
-      count_launches(2);
+    // How many of a query's k best one of its lists holds on average bounds the
+    // slots that a list needs.
+    const int64_t lists =
+        resident ? 2 * split_plan(1, wide ? tiles : (N + 127) / 128, 16, sms, 1).nsplit
+                 : fewest_lists(Qmax, count_dev != nullptr, tiles, 16, sms);
+    const int32_t few = 4 * (int64_t)k <= 5 * lists ? 12 : 2 * (int64_t)k <= 7 * lists ? 16 : 32;
+    const bool guess = k > 32 ? (int64_t)k <= 32 * tiles : k > 16 && few < 32;
+    // The shared per-query floors of the register-list passes start empty, and
+    // no query block is flagged.
+    const size_t clear = guess ? qfloor_bytes + flag_bytes : (size_t)Qmax * 4;
+    cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, clear, stream);
+    if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
+    // Whole-corpus pass of register lists.
+    auto pass = [&](Params& pm, int32_t slots) -> hs_status {
+      if (resident && !pm.only) {
+        auto* launch = slots <= 8    ? (wide ? launch_resident<8, 256> : launch_resident<8, 128>)
+                       : slots <= 12 ? (wide ? launch_resident<12, 256> : launch_resident<12, 128>)
+                       : slots <= 16 ? (wide ? launch_resident<16, 256> : launch_resident<16, 128>)
+                                     : (wide ? launch_resident<32, 256> : launch_resident<32, 128>);
+        return launch(queries, corpus, N, d, pm, stream);
+      }
+      return slots <= 8    ? launch_variant<8>(corpus, N, d, mq, pm, stream)
+             : slots <= 12 ? launch_variant<12>(corpus, N, d, mq, pm, stream)
+             : slots <= 16 ? launch_variant<16>(corpus, N, d, mq, pm, stream)
+                           : launch_variant<32>(corpus, N, d, mq, pm, stream);
+    };
+    st = HS_OK;
+    if (guess) {
+      // More than 16 results: unless the corpus has few tiles an optimistic
+      // pass runs first: the register-list kernel (no shared floor: a floor
+      // that bounds the list's last entry would cut rows of the top k) over the
+      // whole corpus with as many slots as a list is likely to need, merged to
+      // the first k of the union of its lists.  A list whose last entry is
+      // below the union's k-th best holds every row of its range that can be in
+      // the top k, so where no list of a query is cut that way the union's
+      // first k are exact.  The merge flags the query blocks where some list
+      // may have been cut, and every later kernel skips the others.
+      // With rows in no special order a list's share is binomial: 12 slots for
+      // an average of 1.25, 16 for 3.5 and 32 for 16 (k = 32 tiles, two lists a
+      // tile) leave a block of 128 queries flagged once in 1,000 batches or
+      // less, but for the last (one in 20).  Flagged blocks are run with 32
+      // slots, which for k <= 32 are always enough, and what is flagged again
+      // (a query's best rows next to one another in the corpus) exactly.
+      // The slots decide the time, as a list starts by taking nearly all it
+      // sees: 300 queries over 131,072 x 384, k = 50: 237 us with 32 slots, 146
+      // with 16, 126 with 12 (105 with the merge by rank and skipped passes that
+      // end at once), k = 32: 199 -> 104; over 4096 x 128, k = 32: 73 -> 41;
+      // 1000 over 524,288 x 384, k = 100: 637 -> 450.
+      prm.only_mask = 1;
+      auto optimistic = [&](int32_t slots, uint32_t flag_bit) -> hs_status {
+        Params pa = prm;
+        pa.k = slots;
+        pa.qfloor = nullptr;
+        hs_status os = pass(pa, slots);
+        if (os == HS_OK) os = merge(pa, k, scores_out, ids_out, rows, block_flags, flag_bit);
+        if (os == HS_OK) count_launches(2);
+        return os;
+      };
+      st = optimistic(few, 1);
       prm.only = block_flags;
-    }
-    if (tiles >= 64 && prm.only) {
-      Params p1 = prm;
-      p1.tiles = tiles / 8;
-      p1.N = p1.tiles * BN;
-      p1.k = 32;
-      p1.floor = nullptr;
-      st = launch_variant<32>(corpus, N, d, mq, p1, stream);
+      if (st == HS_OK && k > 32 && few < 32) {
+        st = optimistic(32, 2);
+        prm.only_mask = 2;
+      }
       if (st != HS_OK) return st;
-      st = merge(p1, k, kth, nullptr, OutRows{nullptr, 0}, nullptr, block_flags);
-      if (st != HS_OK) return st;
-      count_launches(2);
-      prm.floor = kth;
-      prm.floor_stride = 1;
-      prm.floor_index = 0;
-      // Pass 1's shared floors bound 32nd-best scores, not k-th best: clear.
-      const cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
-      if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
     }
-    st = launch_variant<0>(corpus, N, d, mq, prm, stream);
+    if (k <= 32) {
+      st = pass(prm, k);
+    } else {
+      // The exact path of large k, in two passes.  Pass 1: register lists over
+      // the first eighth of the corpus, whose union's k-th best is a score k
+      // distinct rows reach, hence a floor; pass 2: the large-k kernel over the
+      // whole corpus keeping scores >= the floor.  All passes' lists go through
+      // the same workspace; the floors are staged in it.  Pass 1 needs eight
+      // tiles of its own.
+      if (tiles >= 64 && prm.only) {
+        Params p1 = prm;
+        p1.tiles = tiles / 8;
+        p1.N = p1.tiles * BN;
+        p1.k = 32;
+        st = launch_variant<32>(corpus, N, d, mq, p1, stream);
+        if (st != HS_OK) return st;
+        st = merge(p1, k, kth, nullptr, OutRows{nullptr, 0});
+        if (st != HS_OK) return st;
+        count_launches(2);
+        prm.floor = kth;
+        prm.floor_stride = 1;
+        prm.floor_index = 0;
+        // Pass 1's shared floors bound 32nd-best scores, not k-th best: clear.
+        ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
+        if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
+      }
+      st = launch_variant<0>(corpus, N, d, mq, prm, stream);
+    }
   }
   if (st != HS_OK) return st;
-  st = merge(prm, k, scores_out, ids_out, rows, nullptr, prm.only);
+  st = merge(prm, k, scores_out, ids_out, rows);
   if (st != HS_OK) return st;
   count_launches(R > 0 ? 2 : 1);  // retrieve_kernel + merge_warp_kernel
   return HS_OK;

@@ -113,3 +113,22 @@ def test_resident_pipeline_wait_runs_out():
     got = hs.hs_retrieve_topk(Q, C, 10)
     hs.hs_get_device_error()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("crowd", [0, 14, 40])
+@pytest.mark.parametrize("k", [17, 32, 50, 128, 129])
+@pytest.mark.parametrize("nq", [3, 40, 600])
+def test_lists_shorter_than_k(nq, k, crowd):
+    """More than 16 results from lists of 12 to 32 slots: a query's best rows
+    spread over the corpus, or 14 and 40 of them side by side, which cuts a
+    list of the first pass, and of the second as well; only some query blocks
+    have such a query."""
+    C = synth.unit_rows(9000, 64, k)
+    Q = synth.unit_rows(nq, 64, 6)
+    if crowd:
+        q = bf16_f64(Q[nq // 2:nq // 2 + 1])
+        near = q + np.linspace(0.0, 0.3, crowd)[:, None] * bf16_f64(C[:crowd])
+        near /= np.linalg.norm(near, axis=1, keepdims=True)
+        bits = torch.from_numpy(near.astype(np.float32)).to(torch.bfloat16).view(torch.int16)
+        C[4100:4100 + crowd] = bits.numpy().view(np.uint16)
+    check(Q, C, k)

@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // The query's shared floor, as a threshold that keeps ties with it
       // (another list may hold an equal score at a higher index).
-      uint32_t qf_seen = 0;
+      uint32_t qf_seen = 0, qf_next = 0;
       float qf_theta = -FLT_MAX;
       float list_kth = -FLT_MAX;               // large k: this list's k-th best so far
       if (valid_q && p.qfloor) {               // lists of other splits may have set it
@@ -685,7 +685,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t acc = tile_i & 1u, aphase = (tile_i >> 1) & 1u;
         if (!mbar_wait_limit(tfull + acc, aphase, abort_flag, lim)) goto epi_done;
         tc_fence_after();
-        theta = fmaxf(theta, qf_theta);
         const int64_t col0 = t * BN + half * kHalfCols;
         const bool tail = col0 + kHalfCols > p.N;
         // Register lists: the candidates of the staged chunk (if any) of every
@@ -792,7 +791,14 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           }
-                };
+        };
+        // The floor asked for at the end of the last tile; its round trip has
+        // passed in the wait for this tile's scores.
+        if (qf_next > qf_seen) {
+          qf_seen = qf_next;
+          qf_theta = nextafterf(code_float(qf_next), -INFINITY);  // keep s >= floor
+        }
+        theta = fmaxf(theta, qf_theta);
         // Lists of up to 16 slots: two chunks per TMEM round trip (both loads,
         // one wait).  Longer lists and large k keep one: they need the
         // registers.
@@ -817,23 +823,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (KREG >= 32 && __any_sync(0xffffffffu, pending)) drain();
         tc_fence_before();
         __syncwarp();
-        if (valid_q && p.qfloor) {
-          // Publish this list's k-th best if it raises the query's floor,
-          // and fetch the floor for the next tile.
-          const float kth = KREG > 0 ? ls[(KREG > 0 ? KREG : 1) - 1] : list_kth;
-          const uint32_t mine = kth > -FLT_MAX ? float_code(kth) : 0u;
-          if (mine > qf_seen) atomicMax(p.qfloor + q, mine);
-          const uint32_t c = *reinterpret_cast<volatile uint32_t*>(p.qfloor + q);
-          if (c > qf_seen) {
-            qf_seen = c;
-            qf_theta = nextafterf(code_float(c), -INFINITY);  // keep s >= floor
-          }
-        }
-        if (lane == 0) {
+        if (lane == 0) {                       // the scores are read: the next MMA may have them
           if (CL == 1)
             mbar_arrive(tempty + acc);
           else
             mbar_arrive_cluster(cluster_smem_addr(tempty + acc, 0));
+        }
+        if (valid_q && p.qfloor) {
+          // Publish this list's k-th best if it raises the query's floor,
+          // and fetch the floor for the next tile.  With narrow rows a tile
+          // takes little longer than this round trip: not waiting for it, and
+          // giving the scores' place back before it, 2000 queries over 524,288
+          // x 128, k = 1: 340 -> 318 us, k = 10 500 -> 480; x 384 487 -> 468,
+          // 650 -> 635.
+          const float kth = KREG > 0 ? ls[(KREG > 0 ? KREG : 1) - 1] : list_kth;
+          const uint32_t mine = kth > -FLT_MAX ? float_code(kth) : 0u;
+          if (mine > qf_seen) atomicMax(p.qfloor + q, mine);
+          qf_next = *reinterpret_cast<volatile uint32_t*>(p.qfloor + q);
         }
       }
       if (valid_q) {

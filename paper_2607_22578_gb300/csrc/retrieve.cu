@@ -124,10 +124,13 @@ struct Params {
   // 0 = none), raised with atomicMax and read once per tile by every list of
   // the query.  Zeroed before each launch.
   uint32_t* qfloor;
-  // Optional, one word per query block: a unit whose query blocks all have no
-  // bit of only_mask here is skipped (later passes re-run only flagged blocks).
+  // Optional, one word per query block: a unit whose query blocks are all 0
+  // here is skipped (the exact large-k pass re-runs only the flagged blocks).
   const uint32_t* only;
-  uint32_t only_mask;
+  // Optional: the pass's queries are the count_dev first of a compact copy, and
+  // query q of the call (of all_dev, or Qmax) is its row slot[q] - 1, 0: not in it.
+  const uint32_t* slot;
+  const int32_t* all_dev;
   // Bounded waits of retrieve_kernel: give up after wait_limit_ns.  With
   // withhold_first set (a test hook) every CTA skips the loads of its first
   // stage, so that stage never fills and the waits run out.
@@ -213,7 +216,7 @@ __device__ __forceinline__ bool unit_skipped(const Params& p, const SplitPlan& s
   const int g = (int)(u % sp.groups);
   for (int r = 0; r < cl; ++r) {
     const int qb = g * cl + r;
-    if (qb < sp.qblocks && (p.only[qb] & p.only_mask) != 0u) return false;
+    if (qb < sp.qblocks && p.only[qb] != 0u) return false;
   }
   return true;
 }
@@ -389,14 +392,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* epi_smem = bar_base + kBarBytes;
   const uint64_t lim = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;
 
-  // A pass over flagged query blocks of which there are none, the usual case,
-  // ends here (every CTA sees the same flags): 3.4 us cold, 5 to 7.5 where it
+  // A pass over what an earlier one flagged, of which there is mostly nothing,
+  // then ends here (every CTA sees the same): 3.4 us cold, 5 to 7.5 where it
   // found no unit after the setup.
-  if ((KREG == 0 || KREG == 32) && p.only) {
+  if (p.only || p.slot) {
     pdl_wait();
-    bool any = false;
-    for (int64_t b = threadIdx.x; b < (p.Qmax + BM - 1) / BM; b += kThreads)
-      any |= (p.only[b] & p.only_mask) != 0u;
+    bool any = p.slot && query_count(p) > 0;
+    if (p.only)
+      for (int64_t b = threadIdx.x; b < (p.Qmax + BM - 1) / BM; b += kThreads) any |= p.only[b] != 0u;
     if (!__syncthreads_or(any)) return;
   }
 
@@ -882,6 +885,31 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ---- K7: merge of the per-split lists ----------------------------------------------------
+// What a merge does with a query of which a list may have been cut: flag its
+// block, or (slot set) copy it to the next row of `copy`, once.
+struct CutOut {
+  uint32_t* block;
+  uint32_t *slot, *count;
+  const uint4* queries;
+  uint4* copy;
+  int32_t row16;                        // 16-byte pieces of a query
+};
+
+// The query's row of the copy if it is to be copied now, else -1; one thread.
+__device__ __forceinline__ int64_t claim_row(const CutOut& c, int64_t q) {
+  if (!c.slot || atomicCAS(c.slot + q, 0u, 0xffffffffu) != 0u) return -1;
+  const uint32_t i = atomicAdd(c.count, 1u);
+  c.slot[q] = i + 1u;
+  return i;
+}
+
+// Queries of the call that a merge's rows are drawn from.
+__device__ __forceinline__ int64_t call_count(const Params& p, int64_t Q) {
+  if (!p.slot) return Q;
+  const int64_t c = p.all_dev ? *p.all_dev : p.Qmax;
+  return c < 0 ? 0 : (c > p.Qmax ? p.Qmax : c);
+}
+
 __device__ __forceinline__ uint64_t pack_key(float s, int32_t idx) {
   uint32_t u = __float_as_uint(s);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
@@ -916,8 +944,8 @@ constexpr int kMaxListsPerLane = 10;
 // kout <= 32; for larger kout each pick is written as it is made.  With
 // out_i NULL only the kout-th pick's score is written, to out_s[o] (the
 // floor of the second large-k pass).  With p.only set, rows whose query
-// block is not flagged there are skipped.  With `flag_out` set, a query's
-// block is flagged when one of its lists may have cut off a member of the
+// block is not flagged there are skipped.  With `cut_out` set, a query is
+// handed on when one of its lists may have cut off a member of the
 // top kout: a full list whose last (k-th) entry is not below the union's
 // kout-th pick.  A list whose last entry is below it holds every row of its
 // range that can be in the top kout, so with no list flagged the union's
@@ -929,25 +957,26 @@ template <int LPL>
 __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* __restrict__ out_s,
                                                          int32_t* __restrict__ out_i,
                                                          int32_t kout, OutRows rows,
-                                                         uint32_t* flag_out, uint32_t flag_bit) {
+                                                         const CutOut cut_out) {
   pdl_wait();
   pdl_trigger();
-  const int64_t Q = query_count(p);
+  const int64_t Q = query_count(p), Qcall = call_count(p, Q);
   const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
   const int k = p.k;
   const int lists = 2 * sp.nsplit;
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t R = rows.inv ? rows.n_out : Q;
+  const int64_t R = rows.inv ? rows.n_out : Qcall;
   for (int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; o < R; o += nwarps) {
     const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
-    if (q < 0 || q >= Q) {                         // warp-uniform
+    if (q < 0 || q >= Qcall) {                     // warp-uniform
       if (lane == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
-    if (p.only && (p.only[q / BM] & p.only_mask) == 0u) continue;   // warp-uniform
-    const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
-    const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
+    const int64_t lq = p.slot ? (int64_t)p.slot[q] - 1 : q;
+    if (lq < 0 || (p.only && p.only[q / BM] == 0u)) continue;   // warp-uniform
+    const float* __restrict__ ps = p.part_s + (size_t)lq * lists * k;
+    const int32_t* __restrict__ pi = p.part_i + (size_t)lq * lists * k;
     uint64_t head[LPL], next[LPL];
     int pos[LPL];
 #pragma unroll
@@ -1007,7 +1036,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
       if (last != 0ull) unpack_key(last, sc, id);
       out_s[o] = sc;
     }
-    if (flag_out) {
+    if (cut_out.block || cut_out.slot) {
       bool cut = false;
 #pragma unroll
       for (int j = 0; j < LPL; ++j) {
@@ -1015,7 +1044,12 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
         if (l < lists)
           cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= last;
       }
-      if (__any_sync(0xffffffffu, cut) && lane == 0) atomicOr(flag_out + q / BM, flag_bit);
+      if (__any_sync(0xffffffffu, cut)) {
+        if (lane == 0 && cut_out.block) atomicOr(cut_out.block + q / BM, 1u);
+        const int64_t to = __shfl_sync(0xffffffffu, lane == 0 ? claim_row(cut_out, q) : 0, 0);
+        for (int v = lane; to >= 0 && v < cut_out.row16; v += 32)
+          cut_out.copy[to * cut_out.row16 + v] = __ldg(cut_out.queries + q * cut_out.row16 + v);
+      }
     }
   }
 }
@@ -1029,7 +1063,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
 // shared memory in place of kout dependent rounds.  64 rows of 304 lists, k =
 // 10: 11 us cold, 14.4 with a warp each; 24 rows, k = 50: 27.8 -> 8.4 (32 lists of
 // 32 entries before, 64 of 12 now); 100 rows, k = 100: 66.9 -> 16.8.
-// Lists of at most 32 entries (p.k); CAP >= kout * p.k.  flag_out as above.
+// Lists of at most 32 entries (p.k); CAP >= kout * p.k.  cut_out as above.
 constexpr int kMrThreads = 256;
 constexpr int kMrLists = 32 * kMaxListsPerLane;
 constexpr int kMrMaxK = 128;
@@ -1041,28 +1075,30 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
                                                                 float* __restrict__ out_s,
                                                                 int32_t* __restrict__ out_i,
                                                                 int32_t kout, OutRows rows,
-                                                                uint32_t* flag_out,
-                                                                uint32_t flag_bit) {
+                                                                const CutOut cut_out) {
   pdl_wait();
   pdl_trigger();
   __shared__ uint64_t s_head[kMrLists], s_cand[CAP], s_kth;
   __shared__ int32_t s_sel[kMrLists];
   __shared__ int s_nsel, s_ncand;
+  __shared__ int64_t s_copy;
   const int64_t Q = query_count(p);
   const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
   const int k = p.k, lists = 2 * sp.nsplit, tid = threadIdx.x;
   const int depth = min((kout + lists - 1) / lists, k);
   const int heads = lists * depth;               // entry e of list l: head e * lists + l
-  const int64_t R = rows.inv ? rows.n_out : Q;
+  const int64_t Qcall = call_count(p, Q);
+  const int64_t R = rows.inv ? rows.n_out : Qcall;
   for (int64_t o = blockIdx.x; o < R; o += gridDim.x) {
     const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
-    if (q < 0 || q >= Q) {                         // block-uniform
+    if (q < 0 || q >= Qcall) {                     // block-uniform
       if (tid == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
-    if (p.only && (p.only[q / BM] & p.only_mask) == 0u) continue;   // block-uniform
-    const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
-    const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
+    const int64_t lq = p.slot ? (int64_t)p.slot[q] - 1 : q;
+    if (lq < 0 || (p.only && p.only[q / BM] == 0u)) continue;   // block-uniform
+    const float* __restrict__ ps = p.part_s + (size_t)lq * lists * k;
+    const int32_t* __restrict__ pi = p.part_i + (size_t)lq * lists * k;
     uint64_t mine[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -1124,12 +1160,22 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
       }
     }
     __syncthreads();                               // read before the next row's lists come in
-    if (flag_out) {
+    if (cut_out.block || cut_out.slot) {
       const uint64_t kth = s_kth;
       bool cut = false;
       for (int l = tid; l < lists; l += kMrThreads)
         cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= kth;
-      if (__syncthreads_or(cut) && tid == 0) atomicOr(flag_out + q / BM, flag_bit);
+      if (__syncthreads_or(cut)) {               // (block-uniform)
+        if (tid == 0) {
+          if (cut_out.block) atomicOr(cut_out.block + q / BM, 1u);
+          s_copy = claim_row(cut_out, q);
+        }
+        __syncthreads();
+        const int64_t to = s_copy;
+        for (int v = tid; to >= 0 && v < cut_out.row16; v += kMrThreads)
+          cut_out.copy[to * cut_out.row16 + v] = __ldg(cut_out.queries + q * cut_out.row16 + v);
+        __syncthreads();
+      }
     }
   }
 }
@@ -1612,14 +1658,14 @@ static size_t part_bytes(int64_t Q, int64_t N, int32_t k, int64_t sms) {
 // every batch of at most Q queries.
 size_t retrieve_topk_workspace(int64_t Q, int64_t N, int32_t d, int32_t k) {
   if (Q <= 0 || N <= 0 || k <= 0) return 256;
-  (void)d;
   const int64_t sms = num_sms();
   const size_t part = part_bytes(Q, N, k, sms);
   const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
   const size_t qfloor = (((size_t)Q * 4) + 255) & ~(size_t)255;
   const size_t flags = ((((size_t)(Q + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
-  // lists, large-k lists, shared floors, block flags, large-k floors
-  return 2 * part + 2 * list + 2 * qfloor + flags + 256;
+  // lists, large-k lists, shared floors, block flags, rows of a copy of queries
+  // and their number, large-k floors, the copy
+  return 2 * part + 2 * list + 3 * qfloor + flags + 256 + (k > 16 ? (size_t)Q * d * 2 : 0) + 256;
 }
 
 // Qmax rows of `queries` are addressable; the kernels process the first
@@ -1659,8 +1705,13 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   const size_t qfloor_bytes = (((size_t)Qmax * 4) + 255) & ~(size_t)255;
   prm.qfloor = reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list);
   const size_t flag_bytes = ((((size_t)(Qmax + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
-  uint32_t* block_flags = reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list + qfloor_bytes);
-  float* kth = reinterpret_cast<float*>(w + 2 * part + 2 * list + qfloor_bytes + flag_bytes);
+  char* wf = w + 2 * part + 2 * list + qfloor_bytes;
+  uint32_t* block_flags = reinterpret_cast<uint32_t*>(wf);
+  uint32_t* copy_slot = reinterpret_cast<uint32_t*>(wf + flag_bytes);
+  uint32_t* copy_count = reinterpret_cast<uint32_t*>(wf + flag_bytes + qfloor_bytes);
+  const size_t clear_bytes = qfloor_bytes + flag_bytes + qfloor_bytes + 256;
+  float* kth = reinterpret_cast<float*>(wf + flag_bytes + qfloor_bytes + 256);
+  uint16_t* copy = reinterpret_cast<uint16_t*>(wf + flag_bytes + 2 * qfloor_bytes + 256);
   prm.err = err;
   const bool small = Qmax <= SQ_N && k <= 32 && prm.kb_count <= SQ_MAXKB;
   // Up to 64 queries stay in shared memory, which leaves the ring to the
@@ -1676,7 +1727,7 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   const OutRows rows{inv, n_out};
   const int64_t R = inv ? n_out : Qmax;             // rows the final merge writes
   auto merge = [&](const Params& pm, int32_t kout, float* os, int32_t* oi, OutRows orows,
-                   uint32_t* flag_out = nullptr, uint32_t flag_bit = 0) -> hs_status {
+                   const CutOut cut = CutOut{}) -> hs_status {
     const int64_t nr = orows.inv ? orows.n_out : Qmax;
     if (nr == 0) return HS_OK;
     // Every plan caps its executors (slots) at 16 * kMaxListsPerLane, so a
@@ -1694,16 +1745,16 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     if (kout >= 4 && kout <= 32 && nr <= sms) {
       if (small)
         launch_pdl(merge_rank_kernel<32 * 32>, dim3((unsigned)nr), dim3(kMrThreads), 0, stream, pm,
-                   os, oi, kout, orows, flag_out, flag_bit);
+                   os, oi, kout, orows, cut);
       else
         merge_rank_kernel<32 * 32><<<dim3((unsigned)nr), dim3(kMrThreads), 0, stream>>>(
-            pm, os, oi, kout, orows, flag_out, flag_bit);
+            pm, os, oi, kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
     if (kout > 32 && kout <= kMrMaxK && pm.k <= 32 && oi && nr <= 12 * sms) {
       const int64_t blocks = std::min<int64_t>(nr, 6 * sms);
       merge_rank_kernel<32 * kMrMaxK><<<dim3((unsigned)blocks), dim3(kMrThreads), 0, stream>>>(
-          pm, os, oi, kout, orows, flag_out, flag_bit);
+          pm, os, oi, kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
     {
@@ -1713,16 +1764,16 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       const int64_t lpl = (2 * (int64_t)pm.slots + 31) / 32;
       if (lpl <= 2)
         launch_pdl(merge_warp_kernel<2>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, flag_bit);
+                   cut);
       else if (lpl <= 3)
         launch_pdl(merge_warp_kernel<3>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, flag_bit);
+                   cut);
       else if (lpl <= 5)
         launch_pdl(merge_warp_kernel<5>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   flag_out, flag_bit);
+                   cut);
       else
         launch_pdl(merge_warp_kernel<kMaxListsPerLane>, grid, dim3(256), 0, stream, pm, os, oi,
-                   kout, orows, flag_out, flag_bit);
+                   kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
   };
@@ -1758,23 +1809,24 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     const int32_t few = 4 * (int64_t)k <= 5 * lists ? 12 : 2 * (int64_t)k <= 7 * lists ? 16 : 32;
     const bool guess = k > 32 ? (int64_t)k <= 32 * tiles : k > 16 && few < 32;
     // The shared per-query floors of the register-list passes start empty, and
-    // no query block is flagged.
-    const size_t clear = guess ? qfloor_bytes + flag_bytes : (size_t)Qmax * 4;
+    // no query or block is flagged.
+    const size_t clear = guess ? clear_bytes : (size_t)Qmax * 4;
     cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, clear, stream);
     if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
     // Whole-corpus pass of register lists.
-    auto pass = [&](Params& pm, int32_t slots) -> hs_status {
-      if (resident && !pm.only) {
+    auto pass = [&](Params& pm, int32_t slots, const uint16_t* from,
+                    const CUtensorMap& map) -> hs_status {
+      if (resident) {
         auto* launch = slots <= 8    ? (wide ? launch_resident<8, 256> : launch_resident<8, 128>)
                        : slots <= 12 ? (wide ? launch_resident<12, 256> : launch_resident<12, 128>)
                        : slots <= 16 ? (wide ? launch_resident<16, 256> : launch_resident<16, 128>)
                                      : (wide ? launch_resident<32, 256> : launch_resident<32, 128>);
-        return launch(queries, corpus, N, d, pm, stream);
+        return launch(from, corpus, N, d, pm, stream);
       }
-      return slots <= 8    ? launch_variant<8>(corpus, N, d, mq, pm, stream)
-             : slots <= 12 ? launch_variant<12>(corpus, N, d, mq, pm, stream)
-             : slots <= 16 ? launch_variant<16>(corpus, N, d, mq, pm, stream)
-                           : launch_variant<32>(corpus, N, d, mq, pm, stream);
+      return slots <= 8    ? launch_variant<8>(corpus, N, d, map, pm, stream)
+             : slots <= 12 ? launch_variant<12>(corpus, N, d, map, pm, stream)
+             : slots <= 16 ? launch_variant<16>(corpus, N, d, map, pm, stream)
+                           : launch_variant<32>(corpus, N, d, map, pm, stream);
     };
     st = HS_OK;
     if (guess) {
@@ -1789,35 +1841,61 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       // may have been cut, and every later kernel skips the others.
       // With rows in no special order a list's share is binomial: 12 slots for
       // an average of 1.25, 16 for 3.5 and 32 for 16 (k = 32 tiles, two lists a
-      // tile) leave a block of 128 queries flagged once in 1,000 batches or
-      // less, but for the last (one in 20).  Flagged blocks are run with 32
-      // slots, which for k <= 32 are always enough, and what is flagged again
-      // (a query's best rows next to one another in the corpus) exactly.
+      // tile) leave one of 128 queries cut once in 1,000 batches or less, but
+      // for the last (one in 20).  Queries whose best rows lie side by side in
+      // the corpus are cut more often: they are copied together by the merge and
+      // run with 32 slots, which for k <= 32 are always enough; the blocks of
+      // those cut again, or at first with 32 slots, are run exactly.  One query
+      // in 100 with 20 neighbours among its best, 300 queries over 131,072 x 384:
+      // k = 32 208 us, k = 50 219 (whole blocks run again: 293 and 304; 32 slots
+      // from the start: 200 and 241).
       // The slots decide the time, as a list starts by taking nearly all it
       // sees: 300 queries over 131,072 x 384, k = 50: 237 us with 32 slots, 146
       // with 16, 126 with 12 (105 with the merge by rank and skipped passes that
       // end at once), k = 32: 199 -> 104; over 4096 x 128, k = 32: 73 -> 41;
       // 1000 over 524,288 x 384, k = 100: 637 -> 450.
-      prm.only_mask = 1;
-      auto optimistic = [&](int32_t slots, uint32_t flag_bit) -> hs_status {
-        Params pa = prm;
-        pa.k = slots;
-        pa.qfloor = nullptr;
-        hs_status os = pass(pa, slots);
-        if (os == HS_OK) os = merge(pa, k, scores_out, ids_out, rows, block_flags, flag_bit);
-        if (os == HS_OK) count_launches(2);
-        return os;
-      };
-      st = optimistic(few, 1);
-      prm.only = block_flags;
-      if (st == HS_OK && k > 32 && few < 32) {
-        st = optimistic(32, 2);
-        prm.only_mask = 2;
+      Params pa = prm;
+      pa.k = few;
+      pa.qfloor = nullptr;
+      CutOut cut{};
+      if (few == 32) {
+        cut.block = block_flags;
+      } else {
+        cut.slot = copy_slot;
+        cut.count = copy_count;
+        cut.queries = reinterpret_cast<const uint4*>(queries);
+        cut.copy = reinterpret_cast<uint4*>(copy);
+        cut.row16 = d / 8;
       }
+      st = pass(pa, few, queries, mq);
+      if (st == HS_OK) st = merge(pa, k, scores_out, ids_out, rows, cut);
       if (st != HS_OK) return st;
+      count_launches(2);
+      prm.only = block_flags;
+      if (few < 32) {
+        CUtensorMap mcopy;
+        if (!make_map(&mcopy, copy, Qmax, d, BM))
+          return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
+        Params pc = prm;
+        pc.k = k <= 32 ? k : 32;
+        pc.only = nullptr;
+        pc.slot = copy_slot;
+        pc.count_dev = reinterpret_cast<const int32_t*>(copy_count);
+        pc.all_dev = count_dev;
+        CutOut again{};
+        if (k > 32) {
+          pc.qfloor = nullptr;
+          again.block = block_flags;
+        }
+        st = pass(pc, pc.k, copy, mcopy);
+        if (st == HS_OK) st = merge(pc, k, scores_out, ids_out, rows, again);
+        if (st != HS_OK) return st;
+        count_launches(2);
+        if (k <= 32) return HS_OK;
+      }
     }
     if (k <= 32) {
-      st = pass(prm, k);
+      st = pass(prm, k, queries, mq);
     } else {
       // The exact path of large k, in two passes.  Pass 1: register lists over
       // the first eighth of the corpus, whose union's k-th best is a score k

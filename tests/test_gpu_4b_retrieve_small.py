@@ -132,3 +132,27 @@ def test_lists_shorter_than_k(nq, k, crowd):
         bits = torch.from_numpy(near.astype(np.float32)).to(torch.bfloat16).view(torch.int16)
         C[4100:4100 + crowd] = bits.numpy().view(np.uint16)
     check(Q, C, k)
+
+
+@pytest.mark.parametrize("k", [24, 60])
+@pytest.mark.parametrize("n_live", [1, 150, 400])
+def test_lists_shorter_than_k_with_fanout(n_live, k):
+    """The same through a device count and a fan-out map, where several rows
+    hand the same cut query on: every row gets its query's result."""
+    rng = np.random.default_rng(k)
+    C = synth.unit_rows(9000, 64, k)
+    Q = synth.unit_rows(400, 64, 6)
+    for j, q in enumerate(range(0, n_live, 7)):
+        near = bf16_f64(Q[q:q + 1]) + np.linspace(0.0, 0.3, 20)[:, None] * bf16_f64(C[:20])
+        near /= np.linalg.norm(near, axis=1, keepdims=True)
+        bits = torch.from_numpy(near.astype(np.float32)).to(torch.bfloat16).view(torch.int16)
+        C[130 * j + 100:130 * j + 120] = bits.numpy().view(np.uint16)
+    inv = rng.integers(0, n_live, size=1000).astype(np.int32)
+    dq, dc = to_dev(Q).view(torch.bfloat16), to_dev(C).view(torch.bfloat16)
+    s, i = hs.hs_retrieve_topk_fanout(dq, to_dev(np.array([n_live], np.int32)), to_dev(inv), dc, k)
+    hs.hs_get_device_error()
+    full = bf16_f64(Q[:n_live]) @ bf16_f64(C).T
+    want = -np.sort(-full, axis=1)[:, :k][inv]
+    s, i = s.cpu().numpy(), i.cpu().numpy().astype(np.int64)
+    assert np.abs(s - want).max() < 1e-3
+    assert np.abs(np.take_along_axis(full[inv], i, 1) - want).max() < 1e-3

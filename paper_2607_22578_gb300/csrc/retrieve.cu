@@ -30,7 +30,8 @@
 // once and served to the other query blocks from L2.
 //
 // Top-k state per (query, half): a sorted list in registers (KREG = 8 to 32
-// slots; more than 16 results are first looked for in lists shorter than k).
+// slots; more than 16 results are first looked for in lists shorter than k, and
+// what such a list may have cut off in one more pass over its rows).
 // A 32-column chunk whose maximum beats no lane's threshold costs one
 // max-reduction; otherwise the chunk is staged in shared memory and every lane
 // inserts its candidates in one converged loop, so the warp pays for the
@@ -100,9 +101,34 @@ static_assert(res_stages(128, kResMaxKb) >= 4 && res_stages(256, kResMaxKbWide) 
               "resident queries: a ring of a few stages");
 static_assert(128 * BK * 2 >= (int)kResQBytes, "rows past the last query block lie in the ring");
 static_assert(8 * (2 * kResMaxStages + 4 + 2) + 8 + 8 <= kBarBytes, "barrier area");
+// The pass over cut lists: 128 queries and 128 corpus rows per stage.
+constexpr int kCutRows = 128, kCutStages = 5;
+constexpr uint32_t kCutStageBytes = kABytes + kCutRows * BK * 2;
 static_assert(Ring<1>::smem <= 232448 && Ring<2>::smem <= 232448, "shared memory per CTA");
 static_assert(8 * (2 * Ring<2>::stages + 4) + 8 + 8 <= kBarBytes, "barrier area");
 
+// Lists of a query at most: kMaxListsPerLane per lane of the warp merge, and two
+// (one per column half) per split.
+constexpr int kMaxListsPerLane = 10;
+constexpr int kMaxLists = 32 * kMaxListsPerLane;
+
+// Queries of which a first pass's list may have been cut, by list: queue[l][0,
+// count[l]), in no order; count[kMaxLists] is the sum.
+struct CutQueues {
+  uint32_t *count, *queue;              // [kMaxLists + 1], [kMaxLists][Q]
+  int64_t Q, tiles;                     // the first pass: queries, tiles of ...
+  const int32_t* count_dev;             // (as in Params)
+  int32_t tile_rows, list_k;            // ... so many rows, a list's slots, ...
+  int32_t slots, cl;                    // ... executors, CTAs of each
+  int32_t most_parts;                   // parts that a list's rows are taken in, at most
+};
+
+// The same as work: list l's queries are the rows [row[l], row[l + 1]) of the pass
+// over cut lists, in the blocks of BM [block[l], block[l + 1]).
+struct CutTable {
+  uint32_t blocks, parts, lists, rows;
+  uint32_t row[kMaxLists + 1], block[kMaxLists + 1];
+};
 struct Params {
   int64_t Qmax, N, tiles;
   const int32_t* count_dev;  // queries to process: min(*count_dev, Qmax); NULL: Qmax
@@ -114,23 +140,19 @@ struct Params {
   float* list_s;     // large-k: [grid][kEpi][2][k]
   int32_t* list_i;
   unsigned* err;
-  // Optional per-query score floor (large-k path): query q only keeps scores
-  // >= floor[q * floor_stride + floor_index].  A floor never exceeds the
-  // query's final k-th best score, so it prunes without changing the result.
-  const float* floor;
-  int32_t floor_stride, floor_index;
-  // Per-query shared floor, the largest k-th best score any list of
-  // the query has reached so far (order-preserving uint32 code of the float,
-  // 0 = none), raised with atomicMax and read once per tile by every list of
-  // the query.  Zeroed before each launch.
+  // Optional per-query floor, a score that k rows of the query are known to
+  // reach (order-preserving uint32 code of the float, 0 = none): lower scores
+  // are not kept, which prunes without changing the result.  Zero before the
+  // call's first pass; the merge of a pass whose lists may be cut hands its k-th
+  // best score on in it.  With raise_floor set every list of the query raises
+  // it with atomicMax to its own last entry, and reads it once per tile.  (Not
+  // where lists are shorter than k: their last entries bound nothing.)
   uint32_t* qfloor;
+  int32_t raise_floor;
   // Optional, one word per query block: a unit whose query blocks are all 0
   // here is skipped (the exact large-k pass re-runs only the flagged blocks).
   const uint32_t* only;
-  // Optional: the pass's queries are the count_dev first of a compact copy, and
-  // query q of the call (of all_dev, or Qmax) is its row slot[q] - 1, 0: not in it.
-  const uint32_t* slot;
-  const int32_t* all_dev;
+  CutQueues cut;             // what the pass over cut lists (CUT kernels) runs
   // Bounded waits of retrieve_kernel: give up after wait_limit_ns.  With
   // withhold_first set (a test hook) every CTA skips the loads of its first
   // stage, so that stage never fills and the waits run out.
@@ -199,13 +221,95 @@ __device__ __forceinline__ int64_t query_count(const Params& p) {
   return c < 0 ? 0 : (c > p.Qmax ? p.Qmax : c);
 }
 
-__device__ __forceinline__ void unit_coords(const SplitPlan& sp, int64_t tiles, int64_t u,
-                                            int rank, int cl, int& qb, int& split, int64_t& t0,
-                                            int64_t& t1) {
-  qb = (int)(u % sp.groups) * cl + rank;
-  split = (int)(u / sp.groups);
-  t0 = (int64_t)split * tiles / sp.nsplit;
-  t1 = (int64_t)(split + 1) * tiles / sp.nsplit;
+// Unit u's queries [q0, q1) (CUT: rows of the pass, and where they are in the
+// queue), lists and tiles.
+struct Unit {
+  int64_t q0, q1, t0, t1, queue;
+  int32_t split, half;
+};
+__device__ __forceinline__ Unit unit_coords(const SplitPlan& sp, int64_t Q, int64_t tiles,
+                                            int64_t u, int rank, int cl) {
+  Unit un;
+  un.q0 = ((u % sp.groups) * cl + rank) * BM;
+  un.q1 = Q;
+  un.queue = un.half = 0;
+  un.split = (int)(u / sp.groups);
+  un.t0 = (int64_t)un.split * tiles / sp.nsplit;
+  un.t1 = (int64_t)(un.split + 1) * tiles / sp.nsplit;
+  return un;
+}
+
+// The table, in shared memory, by one warp.  The parts of a list's rows spread what
+// there is over the SMs, in as few rounds as their number allows.
+__device__ __forceinline__ void make_cut_table(const CutQueues& c, CutTable& t, int sms) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n_dev = c.count_dev ? *c.count_dev : c.Q;
+  const SplitPlan sp = split_plan(n_dev < 0 ? 0 : (n_dev > c.Q ? c.Q : n_dev), c.tiles, c.list_k,
+                                  c.slots, c.cl);
+  const int lists = 2 * sp.nsplit;
+  uint32_t rows = 0, blocks = 0;
+  for (int l0 = 0; l0 < lists; l0 += 32) {         // exclusive sums, 32 lists at a time
+    const uint32_t n = l0 + lane < lists ? c.count[l0 + lane] : 0u, nb = (n + BM - 1) / BM;
+    uint32_t r = n, b = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t yr = __shfl_up_sync(0xffffffffu, r, o);
+      const uint32_t yb = __shfl_up_sync(0xffffffffu, b, o);
+      if (lane >= o) {
+        r += yr;
+        b += yb;
+      }
+    }
+    if (l0 + lane < lists) {
+      t.row[l0 + lane] = rows + r - n;
+      t.block[l0 + lane] = blocks + b - nb;
+    }
+    rows += __shfl_sync(0xffffffffu, r, 31);
+    blocks += __shfl_sync(0xffffffffu, b, 31);
+  }
+  if (lane == 0) {
+    t.row[lists] = t.rows = rows;
+    t.block[lists] = t.blocks = blocks;
+    t.lists = lists;
+    const int room = max(1, min(c.most_parts, sp.nsplit * 3 / 8));
+    int best = 1;
+    uint32_t least = ~0u;
+    for (int n = 1; n <= room; ++n) {
+      const uint32_t cost = (blocks * n + sms - 1) / sms * 840u / n;   // 840: lcm(1 ... 8)
+      if (cost < least) {
+        least = cost;
+        best = n;
+      }
+    }
+    t.parts = best;
+  }
+}
+
+// Unit u of the pass over cut lists: block u / parts, part u % parts (which may be
+// empty) of its list's tiles; tile t is the 128 rows from
+// t * tile_rows + half * tile_rows / 2 on, `half` the list's.
+__device__ __forceinline__ Unit cut_unit(const CutTable& t, const CutQueues& c, int64_t u) {
+  const uint32_t b = (uint32_t)(u / t.parts), part = (uint32_t)(u % t.parts);
+  int lo = 0, hi = (int)t.lists;         // block[lo] <= b < block[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) / 2;
+    if (t.block[mid] <= b)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  Unit un;
+  const int64_t at = (int64_t)(b - t.block[lo]) * BM;
+  un.q0 = t.row[lo] + at;
+  un.q1 = t.row[lo + 1];
+  un.queue = lo * c.Q + at;
+  un.split = (int)part;
+  un.half = lo & 1;
+  const int64_t nsplit = t.lists / 2, a = (lo / 2) * c.tiles / nsplit;
+  const int64_t n = (lo / 2 + 1) * c.tiles / nsplit - a;
+  un.t0 = a + part * n / t.parts;
+  un.t1 = a + (part + 1) * n / t.parts;
+  return un;
 }
 
 // True when `only` is set and no query block of unit u's group is flagged.
@@ -361,19 +465,21 @@ __device__ void flush_candidates(float* cs, int32_t* ci, int et, int& cnt, float
   cnt = 0;
 }
 
-// RN > 0: resident queries (CL = 1) and corpus tiles of RN rows.
-template <int KREG, int CL, int RN>
+// RN > 0: resident queries (CL = 1) and corpus tiles of RN rows.  CUT: the units
+// are those of p.cut, single CTAs.
+template <int KREG, int CL, int RN, bool CUT>
 __global__ void __launch_bounds__(kThreads, 1)
     retrieve_kernel(const __grid_constant__ CUtensorMap tmap_q,
                     const __grid_constant__ CUtensorMap tmap_c, const Params p) {
   constexpr bool RES = RN > 0;
   static_assert(!RES || (CL == 1 && KREG > 0), "resident queries: single CTAs, register lists");
-  constexpr int BN = RES ? RN : hs::BN;
+  static_assert(!CUT || (CL == 1 && !RES && KREG == 0), "cut lists: lists in memory");
+  constexpr int BN = RES ? RN : CUT ? kCutRows : hs::BN;
   constexpr int kHalfCols = BN / 2;     // columns per epilogue thread per tile
   constexpr uint32_t kTmemCols = 2 * BN;
-  const int kStages = RES ? res_stages(RN, p.kb_count) : Ring<CL>::stages;
-  constexpr uint32_t kBLocal = RES ? RN * BK * 2 : Ring<CL>::b_bytes;
-  constexpr uint32_t kStageBytes = RES ? RN * BK * 2 : Ring<CL>::stage_bytes;
+  const int kStages = RES ? res_stages(RN, p.kb_count) : CUT ? kCutStages : Ring<CL>::stages;
+  constexpr uint32_t kBLocal = RES ? RN * BK * 2 : CUT ? kCutRows * BK * 2 : Ring<CL>::b_bytes;
+  constexpr uint32_t kStageBytes = RES ? RN * BK * 2 : CUT ? kCutStageBytes : Ring<CL>::stage_bytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -395,10 +501,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // A pass over what an earlier one flagged, of which there is mostly nothing,
   // then ends here (every CTA sees the same): 3.4 us cold, 5 to 7.5 where it
   // found no unit after the setup.
-  if (p.only || p.slot) {
+  if (CUT || p.only) {
     pdl_wait();
-    bool any = p.slot && query_count(p) > 0;
-    if (p.only)
+    bool any = CUT && p.cut.count[kMaxLists] != 0u;
+    if (!CUT)
       for (int64_t b = threadIdx.x; b < (p.Qmax + BM - 1) / BM; b += kThreads) any |= p.only[b] != 0u;
     if (!__syncthreads_or(any)) return;
   }
@@ -444,12 +550,78 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the previous kernel on the stream.
   pdl_wait();
   pdl_trigger();
+  const CutTable& cut = *reinterpret_cast<const CutTable*>(epi_smem + hs::kEpiSmem);
+  if (CUT) {
+    if (warp == 0)
+      make_cut_table(p.cut, *reinterpret_cast<CutTable*>(epi_smem + hs::kEpiSmem), gridDim.x);
+    __syncthreads();
+  }
   const int64_t Q = query_count(p);
-  const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, CL);
-  const int64_t units = Q > 0 ? (int64_t)sp.groups * sp.nsplit : 0;
+  const SplitPlan sp = CUT ? SplitPlan{0, 0, (int32_t)cut.parts}
+                           : split_plan(Q, p.tiles, p.k, p.slots, CL);
+  const int64_t units = CUT     ? (int64_t)cut.blocks * cut.parts
+                        : Q > 0 ? (int64_t)sp.groups * sp.nsplit
+                                : 0;
   const int64_t u0 = blockIdx.x / CL, ustep = gridDim.x / CL;
+  auto tile_row = [&](const Unit& un, int64_t t) {   // a tile's first corpus row
+    return CUT ? t * p.cut.tile_rows + un.half * (p.cut.tile_rows / 2) : t * BN;
+  };
+  auto unit_of = [&](int64_t u, int rank) {
+    return CUT ? cut_unit(cut, p.cut, u) : unit_coords(sp, Q, p.tiles, u, rank, CL);
+  };
 
-  if (warp == 0) {
+  if (CUT && warp == 0) {
+    // ------------------------------------------------------------ TMA producer
+    // of cut queries: each lane takes four of a block's rows from their places
+    // (whole rows of four; the rest of the 128 is whatever was there, in lanes
+    // nobody reads), lane 0 the corpus tile.
+    const uint64_t pol_c = policy_evict_first();
+    uint32_t stage = 0, phase = 0;
+    int64_t issued = 0;
+    bool ok = true;
+    for (int64_t u = u0; u < units && ok; u += ustep) {
+      const Unit un = unit_of(u, 0);
+      const int live = (int)min((int64_t)BM, un.q1 - un.q0), fours = (live + 3) / 4;
+      const uint32_t* qs = p.cut.queue + un.queue;
+      int4 mine = make_int4(0, 0, 0, 0);
+      if (lane < fours)
+        mine = make_int4((int)qs[4 * lane], (int)qs[min(4 * lane + 1, live - 1)],
+                         (int)qs[min(4 * lane + 2, live - 1)], (int)qs[min(4 * lane + 3, live - 1)]);
+      for (int64_t t = un.t0; t < un.t1 && ok; ++t) {
+        for (int kb = 0; kb < p.kb_count; ++kb) {
+          ok = __all_sync(0xffffffffu, mbar_wait_limit(empty + stage, phase ^ 1u, abort_flag, lim));
+          if (!ok) break;
+          if (!p.withhold_first || issued > 0) {   // (test hook: that stage never fills)
+            if (lane == 0) {
+              mbar_arrive_expect_tx(full + stage, (uint32_t)fours * 4 * BK * 2 + kBLocal);
+              const int64_t cy = tile_row(un, t);    // past the last row: any, masked
+              tma_load_2d_hint(sB + stage * kBLocal, &tmap_c, full + stage, kb * BK,
+                               (int32_t)(cy < p.N ? cy : 0), pol_c);
+            }
+            __syncwarp();
+            if (lane < fours)
+              tma_gather4(sA + stage * kABytes + lane * 4 * BK * 2, &tmap_q, full + stage, kb * BK,
+                          mine);
+          }
+          ++issued;
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+    }
+    if (lane == 0) {                       // no copy in flight when the CTA leaves, as below
+      volatile int keep_going = 0;
+      for (int64_t i = issued > kStages ? issued - kStages : 0; i < issued; ++i) {
+        if (p.withhold_first && i == 0) continue;
+        if (!mbar_wait_limit(full + (int)(i % kStages), (uint32_t)((i / kStages) & 1), &keep_going,
+                             lim))
+          break;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const uint64_t pol_c = policy_evict_first();
@@ -463,11 +635,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           tma_load_2d(sA + kb * kResQBytes, &tmap_q, qfull, kb * BK, 0);
       }
       for (int64_t u = u0; u < units; u += ustep) {
-        if (unit_skipped(p, sp, u, CL)) continue;
-        int qb, split;
-        int64_t t0, t1;
-        unit_coords(sp, p.tiles, u, rank, CL, qb, split, t0, t1);
-        for (int64_t t = t0; t < t1; ++t) {
+        if (!CUT && unit_skipped(p, sp, u, CL)) continue;
+        const Unit un = unit_of(u, rank);
+        for (int64_t t = un.t0; t < un.t1; ++t) {
           for (int kb = 0; kb < p.kb_count; ++kb) {
             if (!mbar_wait_limit(empty + stage, phase ^ 1u, abort_flag, lim)) goto producer_done;
             if (p.withhold_first && issued == 0) {   // test hook: this stage never fills
@@ -482,7 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // A query block past the last addressable row is loaded from
             // row 0 instead: its scores are masked, and no box lies wholly
             // outside the tensor.
-            const int32_t qy = (int64_t)qb * BM < p.Qmax ? qb * BM : 0;
+            const int32_t qy = un.q0 < p.Qmax ? (int32_t)un.q0 : 0;
             if (RES) {
               mbar_arrive_expect_tx(full + stage, kStageBytes);
               tma_load_2d_hint(sB + stage * kBLocal, &tmap_c, full + stage, kb * BK,
@@ -535,11 +705,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool any_mma = false;
       if (RES && u0 < units && !mbar_wait_limit(qfull, 0u, abort_flag, lim)) goto mma_done;
       for (int64_t u = u0; u < units; u += ustep) {
-        if (unit_skipped(p, sp, u, CL)) continue;
-        int qb, split;
-        int64_t t0, t1;
-        unit_coords(sp, p.tiles, u, rank, CL, qb, split, t0, t1);
-        for (int64_t t = t0; t < t1; ++t, ++tile_i) {
+        if (!CUT && unit_skipped(p, sp, u, CL)) continue;
+        const Unit un = unit_of(u, rank);
+        for (int64_t t = un.t0; t < un.t1; ++t, ++tile_i) {
           const uint32_t acc = tile_i & 1u, aphase = (tile_i >> 1) & 1u;
           if (!mbar_wait_limit(tempty + acc, aphase ^ 1u, abort_flag, lim)) goto mma_done;
           tc_fence_after();
@@ -607,21 +775,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     float* Ls = p.list_s + ((size_t)blockIdx.x * kEpi + et) * 2 * (size_t)k;
     int32_t* Li = p.list_i + ((size_t)blockIdx.x * kEpi + et) * 2 * (size_t)k;
     for (int64_t u = u0; u < units; u += ustep) {
-      if (unit_skipped(p, sp, u, CL)) continue;
-      int qb, split;
-      int64_t t0, t1;
-      unit_coords(sp, p.tiles, u, rank, CL, qb, split, t0, t1);
-      const int64_t q = (int64_t)qb * BM + row;
-      const bool valid_q = q < Q;
+      if (!CUT && unit_skipped(p, sp, u, CL)) continue;
+      const Unit un = unit_of(u, rank);
+      const int64_t t0 = un.t0, t1 = un.t1, q = un.q0 + row;
+      const bool valid_q = q < un.q1;
+      const int64_t qcall = CUT && valid_q ? (int64_t)p.cut.queue[un.queue + row] : q;
       const bool warp_has_query = __any_sync(0xffffffffu, valid_q);
-      // Large k: start from the query's floor (a lower bound on its final k-th
-      // best score), so only scores that can still make the top k are kept.
-      float floor_theta = -FLT_MAX;
-      if (KREG == 0 && p.floor && valid_q) {
-        const float f = p.floor[(size_t)q * p.floor_stride + p.floor_index];
-        if (f > -FLT_MAX) floor_theta = nextafterf(f, -INFINITY);  // keep s >= f
-      }
-      float theta = floor_theta;
+      float theta = -FLT_MAX;
       // Register list (k <= 32): KREG slots sorted descending, the first
       // KREG - k holding +FLT_MAX sentinels that never move, so the last
       // slot is always the k-th best score seen: the list's own threshold.
@@ -638,11 +798,37 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t qf_seen = 0, qf_next = 0;
       float qf_theta = -FLT_MAX;
       float list_kth = -FLT_MAX;               // large k: this list's k-th best so far
-      if (valid_q && p.qfloor) {               // lists of other splits may have set it
-        qf_seen = *reinterpret_cast<volatile uint32_t*>(p.qfloor + q);
+      const size_t list = ((size_t)q * lists + 2 * un.split + half) * k;
+      // Cut lists: few scores reach the floor that they start with, most of them
+      // together, so they are kept in no order, in place, and the least is looked
+      // for only once there are k.
+      int at_least = 0;
+      auto keep = [&](float sc, int32_t idx) {
+        float* os = p.part_s + list;
+        int32_t* oi = p.part_i + list;
+        const int at = cnt < k ? cnt++ : at_least;
+        os[at] = sc;
+        oi[at] = idx;
+        if (cnt < k) return;
+        float ls0 = INFINITY;
+        int32_t li0 = -1;
+        for (int i = 0; i < k; ++i) {
+          const float s = os[i];
+          const int32_t j = oi[i];
+          if (s < ls0 || (s == ls0 && j > li0) || i == 0) {
+            ls0 = s;
+            li0 = j;
+            at_least = i;
+          }
+        }
+        list_kth = ls0;
+        theta = fmaxf(theta, ls0);
+      };
+      if (valid_q && p.qfloor) {               // an earlier pass or other lists may have set it
+        qf_seen = *reinterpret_cast<volatile uint32_t*>(p.qfloor + qcall);
         if (qf_seen) qf_theta = nextafterf(code_float(qf_seen), -INFINITY);
       }
-      if (KREG == 0 && valid_q) {
+      if (KREG == 0 && !CUT && valid_q) {
         for (int i = 0; i < k; ++i) {
           Ls[i] = -FLT_MAX;
           Li[i] = -1;
@@ -688,7 +874,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t acc = tile_i & 1u, aphase = (tile_i >> 1) & 1u;
         if (!mbar_wait_limit(tfull + acc, aphase, abort_flag, lim)) goto epi_done;
         tc_fence_after();
-        const int64_t col0 = t * BN + half * kHalfCols;
+        const int64_t col0 = tile_row(un, t) + half * kHalfCols;
         const bool tail = col0 + kHalfCols > p.N;
         // Register lists: the candidates of the staged chunk (if any) of every
         // lane, inserted in one converged loop (the warp pays for the largest
@@ -772,6 +958,25 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
               __syncwarp();
             }
+          } else if (CUT) {
+            const bool any = valid_q && chunk_max(r) > theta;
+            if (__any_sync(0xffffffffu, any)) {
+              uint32_t m = 0;
+              if (any) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) m |= (__uint_as_float(r[j]) > theta ? 1u : 0u) << j;
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                  reinterpret_cast<uint4*>(stage_f)[v * kEpi + et] =
+                      make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+              }
+              for (; m; m &= m - 1) {
+                const int j = __ffs(m) - 1;
+                const float sc = stage_f[((j >> 2) * kEpi + et) * 4 + (j & 3)];
+                if (sc > theta) keep(sc, cbase + j);
+              }
+              __syncwarp();
+            }
           } else {
             // Same first test as above: a chunk whose maximum beats no
             // lane's threshold costs one max-reduction and a vote.
@@ -789,8 +994,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                   }
                 }
                 if (__any_sync(0xffffffffu, cnt > kCap - 4))
-                  flush_candidates(cand_s, cand_i, et, cnt, Ls, Li, k, cur, theta,
-                                   fmaxf(floor_theta, qf_theta), list_kth);
+                  flush_candidates(cand_s, cand_i, et, cnt, Ls, Li, k, cur, theta, qf_theta,
+                                   list_kth);
               }
             }
           }
@@ -832,7 +1037,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           else
             mbar_arrive_cluster(cluster_smem_addr(tempty + acc, 0));
         }
-        if (valid_q && p.qfloor) {
+        if (valid_q && p.raise_floor) {
           // Publish this list's k-th best if it raises the query's floor,
           // and fetch the floor for the next tile.  With narrow rows a tile
           // takes little longer than this round trip: not waiting for it, and
@@ -841,15 +1046,27 @@ __global__ void __launch_bounds__(kThreads, 1)
           // 650 -> 635.
           const float kth = KREG > 0 ? ls[(KREG > 0 ? KREG : 1) - 1] : list_kth;
           const uint32_t mine = kth > -FLT_MAX ? float_code(kth) : 0u;
-          if (mine > qf_seen) atomicMax(p.qfloor + q, mine);
-          qf_next = *reinterpret_cast<volatile uint32_t*>(p.qfloor + q);
+          if (mine > qf_seen) atomicMax(p.qfloor + qcall, mine);
+          qf_next = *reinterpret_cast<volatile uint32_t*>(p.qfloor + qcall);
         }
       }
       if (valid_q) {
-        const size_t o = ((size_t)q * lists + 2 * split + half) * k;
-        float* os = p.part_s + o;
-        int32_t* oi = p.part_i + o;
-        if (KREG > 0) {
+        float* os = p.part_s + list;
+        int32_t* oi = p.part_i + list;
+        if (CUT) {                             // the least of a full list goes last
+          if (cnt == k) {
+            const float sl = os[at_least];
+            const int32_t il = oi[at_least];
+            os[at_least] = os[k - 1];
+            oi[at_least] = oi[k - 1];
+            os[k - 1] = sl;
+            oi[k - 1] = il;
+          }
+          for (int i = cnt; i < k; ++i) {
+            os[i] = -FLT_MAX;
+            oi[i] = -1;
+          }
+        } else if (KREG > 0) {
 #pragma unroll
           for (int i = 0; i < (KREG > 0 ? KREG : 1); ++i)
             if (i >= KREG - k) {
@@ -857,8 +1074,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               oi[i - (KREG - k)] = li[i];
             }
         } else {
-          flush_candidates(cand_s, cand_i, et, cnt, Ls, Li, k, cur, theta,
-                           fmaxf(floor_theta, qf_theta), list_kth);
+          flush_candidates(cand_s, cand_i, et, cnt, Ls, Li, k, cur, theta, qf_theta,
+                           list_kth);
           for (int i = 0; i < k; ++i) {
             os[i] = Ls[(size_t)cur * k + i];
             oi[i] = Li[(size_t)cur * k + i];
@@ -885,33 +1102,33 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ---- K7: merge of the per-split lists ----------------------------------------------------
-// What a merge does with a query of which a list may have been cut: flag its
-// block, or (slot set) copy it to the next row of `copy`, once.
+// What a merge does with a query of which a list may have been cut, that is a
+// full list whose last entry is not below the k-th best: it flags the query's
+// block, or (pairs set) notes, once, which lists were cut, for the pass over
+// them.  No more than k entries are that good and a cut list has p.k of
+// them, so at most `most` = k / p.k of a query's lists are cut.  The k-th
+// best score, which k rows reach, is the later passes' floor (of every query,
+// as a flagged block is run whole).
 struct CutOut {
   uint32_t* block;
-  uint32_t *slot, *count;
-  const uint4* queries;
-  uint4* copy;
-  int32_t row16;                        // 16-byte pieces of a query
+  uint32_t* floor;                      // by query
+  uint32_t* pairs;                      // by query: lists cut
+  uint2* at;                            // [query][most]: the list, the place in its queue
+  int32_t most;
+  CutQueues queues;
 };
 
-// The query's row of the copy if it is to be copied now, else -1; one thread.
-__device__ __forceinline__ int64_t claim_row(const CutOut& c, int64_t q) {
-  if (!c.slot || atomicCAS(c.slot + q, 0u, 0xffffffffu) != 0u) return -1;
-  const uint32_t i = atomicAdd(c.count, 1u);
-  c.slot[q] = i + 1u;
-  return i;
+__device__ __forceinline__ void add_pair(const CutOut& c, int64_t q, int32_t i, int32_t list) {
+  if (i >= c.most) return;              // not reached, but after a wait that ran out
+  const uint32_t at = atomicAdd(c.queues.count + list, 1u);
+  atomicAdd(c.queues.count + kMaxLists, 1u);
+  c.queues.queue[(size_t)list * c.queues.Q + at] = (uint32_t)q;
+  c.at[(size_t)q * c.most + i] = make_uint2((uint32_t)list, at);
 }
 
-// Queries of the call that a merge's rows are drawn from.
-__device__ __forceinline__ int64_t call_count(const Params& p, int64_t Q) {
-  if (!p.slot) return Q;
-  const int64_t c = p.all_dev ? *p.all_dev : p.Qmax;
-  return c < 0 ? 0 : (c > p.Qmax ? p.Qmax : c);
-}
-
+// (-0 as +0: they are equal, and keys order as the lists do.)
 __device__ __forceinline__ uint64_t pack_key(float s, int32_t idx) {
-  uint32_t u = __float_as_uint(s);
+  uint32_t u = __float_as_uint(s + 0.0f);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((uint64_t)u << 32) | (uint64_t)(0xffffffffu - (uint32_t)idx);
 }
@@ -921,6 +1138,15 @@ __device__ __forceinline__ void unpack_key(uint64_t key, float& s, int32_t& idx)
   u = (u & 0x80000000u) ? (u ^ 0x80000000u) : ~u;
   s = __uint_as_float(u);
   idx = (int32_t)(0xffffffffu - (uint32_t)key);
+}
+
+// Is it a row's key (a list's unused entries have none)?
+__device__ __forceinline__ bool real_key(uint64_t key) { return (uint32_t)key != 0u; }
+
+// The floor that a k-th pick is: its score's code (a key's upper half), or 0
+// where it is none, with fewer rows than k in the lists.
+__device__ __forceinline__ uint32_t key_floor(uint64_t key) {
+  return real_key(key) ? (uint32_t)(key >> 32) : 0u;
 }
 
 // Largest key of the warp's: the largest high word, then the largest low word
@@ -938,45 +1164,41 @@ __device__ __forceinline__ uint64_t warp_max_key(uint64_t key) {
 // head (keys are unique: a corpus row lives in exactly one list; padding
 // keys tie, and the lowest such lane advances), so kout rounds give the kout
 // best in order.
-constexpr int kMaxListsPerLane = 10;
-
+//
 // Any kout: picks 0..31 are kept one per lane and written together when
 // kout <= 32; for larger kout each pick is written as it is made.  With
-// out_i NULL only the kout-th pick's score is written, to out_s[o] (the
-// floor of the second large-k pass).  With p.only set, rows whose query
-// block is not flagged there are skipped.  With `cut_out` set, a query is
-// handed on when one of its lists may have cut off a member of the
-// top kout: a full list whose last (k-th) entry is not below the union's
+// p.only set, rows whose query
+// block is not flagged there are skipped.  With CUT, a query is handed on to
+// `cut_out` when one of its lists may have cut off a member of the top kout: a full list whose last (k-th) entry is not below the union's
 // kout-th pick.  A list whose last entry is below it holds every row of its
-// range that can be in the top kout, so with no list flagged the union's
+// range that can be in the top kout, so with no list cut the union's
 // first kout entries are exact.  LPL lists per lane at most (the
 // launch's bound on 2 * nsplit / 32, rounded up); slots past the query's
 // list count are skipped warp-uniformly, so the per-round work and the
 // registers follow the lists a launch can have, not the largest count.
-template <int LPL>
+template <int LPL, bool CUT>
 __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* __restrict__ out_s,
                                                          int32_t* __restrict__ out_i,
                                                          int32_t kout, OutRows rows,
                                                          const CutOut cut_out) {
   pdl_wait();
   pdl_trigger();
-  const int64_t Q = query_count(p), Qcall = call_count(p, Q);
+  const int64_t Q = query_count(p);
   const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
   const int k = p.k;
   const int lists = 2 * sp.nsplit;
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t R = rows.inv ? rows.n_out : Qcall;
+  const int64_t R = rows.inv ? rows.n_out : Q;
   for (int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; o < R; o += nwarps) {
     const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
-    if (q < 0 || q >= Qcall) {                     // warp-uniform
+    if (q < 0 || q >= Q) {                         // warp-uniform
       if (lane == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
-    const int64_t lq = p.slot ? (int64_t)p.slot[q] - 1 : q;
-    if (lq < 0 || (p.only && p.only[q / BM] == 0u)) continue;   // warp-uniform
-    const float* __restrict__ ps = p.part_s + (size_t)lq * lists * k;
-    const int32_t* __restrict__ pi = p.part_i + (size_t)lq * lists * k;
+    if (p.only && p.only[q / BM] == 0u) continue;  // warp-uniform
+    const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
+    const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
     uint64_t head[LPL], next[LPL];
     int pos[LPL];
 #pragma unroll
@@ -1006,7 +1228,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
       last = mx;
       if (kout <= 32) {
         if (lane == r && mx != 0ull) unpack_key(mx, my_s, my_i);
-      } else if (out_i && lane == 0) {
+      } else if (lane == 0) {
         float sc = -FLT_MAX;
         int32_t id = -1;
         if (mx != 0ull) unpack_key(mx, sc, id);
@@ -1026,29 +1248,33 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
           }
       }
     }
-    if (out_i && kout <= 32 && lane < kout) {
+    if (kout <= 32 && lane < kout) {
       out_s[(size_t)o * kout + lane] = my_s;
       out_i[(size_t)o * kout + lane] = my_i;
     }
-    if (!out_i && lane == 0) {
-      float sc = -FLT_MAX;
-      int32_t id = -1;
-      if (last != 0ull) unpack_key(last, sc, id);
-      out_s[o] = sc;
-    }
-    if (cut_out.block || cut_out.slot) {
-      bool cut = false;
-#pragma unroll
-      for (int j = 0; j < LPL; ++j) {
-        const int l = j * 32 + lane;
-        if (l < lists)
-          cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= last;
-      }
-      if (__any_sync(0xffffffffu, cut)) {
-        if (lane == 0 && cut_out.block) atomicOr(cut_out.block + q / BM, 1u);
-        const int64_t to = __shfl_sync(0xffffffffu, lane == 0 ? claim_row(cut_out, q) : 0, 0);
-        for (int v = lane; to >= 0 && v < cut_out.row16; v += 32)
-          cut_out.copy[to * cut_out.row16 + v] = __ldg(cut_out.queries + q * cut_out.row16 + v);
+    if (CUT) {
+      if (lane == 0) cut_out.floor[q] = key_floor(last);
+      auto cut = [&](int l) {                      // is list l?
+        if (l >= lists) return false;
+        const uint64_t key = pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]);
+        return real_key(key) && key >= last;
+      };
+      bool any = false;
+#pragma unroll 1
+      for (int l = lane; l < lists; l += 32) any |= cut(l);
+      if (!__any_sync(0xffffffffu, any)) continue;
+      if (!cut_out.pairs) {
+        if (lane == 0) atomicOr(cut_out.block + q / BM, 1u);
+      } else if (__shfl_sync(0xffffffffu, lane == 0 ? atomicCAS(cut_out.pairs + q, 0u, ~0u) : 0u,
+                             0) == 0u) {
+        int32_t n = 0;
+#pragma unroll 1
+        for (int l0 = 0; l0 < lists; l0 += 32) {
+          const uint32_t m = __ballot_sync(0xffffffffu, cut(l0 + lane));
+          if ((m >> lane) & 1u) add_pair(cut_out, q, n + __popc(m & lanemask_lt()), l0 + lane);
+          n += __popc(m);
+        }
+        if (lane == 0) cut_out.pairs[q] = min(n, cut_out.most);
       }
     }
   }
@@ -1065,7 +1291,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
 // 32 entries before, 64 of 12 now); 100 rows, k = 100: 66.9 -> 16.8.
 // Lists of at most 32 entries (p.k); CAP >= kout * p.k.  cut_out as above.
 constexpr int kMrThreads = 256;
-constexpr int kMrLists = 32 * kMaxListsPerLane;
+constexpr int kMrLists = kMaxLists;
 constexpr int kMrMaxK = 128;
 static_assert(kMrLists <= 2 * kMrThreads, "two heads per thread");
 static_assert(kMrLists >= 2 * kMrMaxK, "lists * depth < kout + lists <= kMrLists");
@@ -1080,25 +1306,22 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
   pdl_trigger();
   __shared__ uint64_t s_head[kMrLists], s_cand[CAP], s_kth;
   __shared__ int32_t s_sel[kMrLists];
-  __shared__ int s_nsel, s_ncand;
-  __shared__ int64_t s_copy;
+  __shared__ int s_nsel, s_ncand, s_npairs;
   const int64_t Q = query_count(p);
   const SplitPlan sp = split_plan(Q, p.tiles, p.k, p.slots, p.cl);
   const int k = p.k, lists = 2 * sp.nsplit, tid = threadIdx.x;
   const int depth = min((kout + lists - 1) / lists, k);
   const int heads = lists * depth;               // entry e of list l: head e * lists + l
-  const int64_t Qcall = call_count(p, Q);
-  const int64_t R = rows.inv ? rows.n_out : Qcall;
+  const int64_t R = rows.inv ? rows.n_out : Q;
   for (int64_t o = blockIdx.x; o < R; o += gridDim.x) {
     const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
-    if (q < 0 || q >= Qcall) {                     // block-uniform
+    if (q < 0 || q >= Q) {                         // block-uniform
       if (tid == 0) set_error(p.err, kErrInvalidArg);
       continue;
     }
-    const int64_t lq = p.slot ? (int64_t)p.slot[q] - 1 : q;
-    if (lq < 0 || (p.only && p.only[q / BM] == 0u)) continue;   // block-uniform
-    const float* __restrict__ ps = p.part_s + (size_t)lq * lists * k;
-    const int32_t* __restrict__ pi = p.part_i + (size_t)lq * lists * k;
+    if (p.only && p.only[q / BM] == 0u) continue;  // block-uniform
+    const float* __restrict__ ps = p.part_s + (size_t)q * lists * k;
+    const int32_t* __restrict__ pi = p.part_i + (size_t)q * lists * k;
     uint64_t mine[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -1106,7 +1329,8 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
       mine[j] = 0ull;
       if (h < heads) {
         const size_t e = (size_t)(h % lists) * k + h / lists;
-        s_head[h] = mine[j] = pack_key(ps[e], pi[e]);
+        const uint64_t key = pack_key(ps[e], pi[e]);
+        s_head[h] = mine[j] = real_key(key) ? key : 0ull;
       }
     }
     if (tid == 0) {
@@ -1116,21 +1340,21 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
     __syncthreads();
     int rank[2] = {0, 0};
 #pragma unroll 8
-    for (int h = 0; h < heads; ++h) {              // (entries of empty lists are alike)
+    for (int h = 0; h < heads; ++h) {              // (missing entries are alike)
       const uint64_t y = s_head[h];
       rank[0] += (y > mine[0]) | ((y == mine[0]) & (h < tid));
       rank[1] += (y > mine[1]) | ((y == mine[1]) & (h < tid + kMrThreads));
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      if (j * kMrThreads + tid < heads && rank[j] == kout - 1) s_kth = mine[j];
+      if (mine[j] != 0ull && rank[j] == kout - 1) s_kth = mine[j];
     __syncthreads();
     // the kout-th best head; with fewer entries than that every one counts
     const uint64_t bound = s_kth;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int h = j * kMrThreads + tid;
-      if (h < heads && rank[j] < kout) {
+      if (mine[j] != 0ull && rank[j] < kout) {
         s_cand[atomicAdd(&s_ncand, 1)] = mine[j];
         if (h / lists == depth - 1) s_sel[atomicAdd(&s_nsel, 1)] = h % lists;
       }
@@ -1140,16 +1364,20 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
     for (int i = tid; i < more; i += kMrThreads) {
       const size_t e = (size_t)s_sel[i / rest] * k + depth + i % rest;
       const uint64_t key = pack_key(ps[e], pi[e]);
-      if (key >= bound) s_cand[atomicAdd(&s_ncand, 1)] = key;
+      if (real_key(key) && key >= bound) s_cand[atomicAdd(&s_ncand, 1)] = key;
     }
     if (tid == 0) s_kth = 0ull;
     __syncthreads();
     const int c = s_ncand;
+    for (int i = c + tid; i < kout; i += kMrThreads) {       // fewer rows than results
+      out_s[(size_t)o * kout + i] = -FLT_MAX;
+      out_i[(size_t)o * kout + i] = -1;
+    }
     for (int i = tid; i < c; i += kMrThreads) {
       const uint64_t key = s_cand[i];
       int r = 0;
 #pragma unroll 8
-      for (int j = 0; j < c; ++j) r += (s_cand[j] > key) | ((s_cand[j] == key) & (j < i));
+      for (int j = 0; j < c; ++j) r += s_cand[j] > key;
       if (r < kout) {
         float sc;
         int32_t id;
@@ -1160,23 +1388,129 @@ __global__ void __launch_bounds__(kMrThreads) merge_rank_kernel(const Params p,
       }
     }
     __syncthreads();                               // read before the next row's lists come in
-    if (cut_out.block || cut_out.slot) {
+    if (cut_out.floor) {
       const uint64_t kth = s_kth;
-      bool cut = false;
-      for (int l = tid; l < lists; l += kMrThreads)
-        cut |= pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]) >= kth;
-      if (__syncthreads_or(cut)) {               // (block-uniform)
+      if (tid == 0) cut_out.floor[q] = key_floor(kth);
+      uint32_t cut = 0;                            // bit j: list j * kMrThreads + tid is
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int l = j * kMrThreads + tid;
+        if (l < lists) {
+          const uint64_t key = pack_key(ps[(size_t)l * k + k - 1], pi[(size_t)l * k + k - 1]);
+          if (real_key(key) && key >= kth) cut |= 1u << j;
+        }
+      }
+      if (__syncthreads_or(cut)) {                 // block-uniform
         if (tid == 0) {
-          if (cut_out.block) atomicOr(cut_out.block + q / BM, 1u);
-          s_copy = claim_row(cut_out, q);
+          s_npairs = cut_out.pairs ? (int)(atomicCAS(cut_out.pairs + q, 0u, ~0u) != 0u) : -1;
+          if (!cut_out.pairs) atomicOr(cut_out.block + q / BM, 1u);
         }
         __syncthreads();
-        const int64_t to = s_copy;
-        for (int v = tid; to >= 0 && v < cut_out.row16; v += kMrThreads)
-          cut_out.copy[to * cut_out.row16 + v] = __ldg(cut_out.queries + q * cut_out.row16 + v);
+        const bool first = s_npairs == 0;          // block-uniform
         __syncthreads();
+        for (int j = 0; j < 2 && first; ++j)
+          if ((cut >> j) & 1u)
+            add_pair(cut_out, q, atomicAdd(&s_npairs, 1), j * kMrThreads + tid);
+        __syncthreads();
+        if (first && tid == 0) cut_out.pairs[q] = min(s_npairs, cut_out.most);
       }
     }
+  }
+}
+
+// ---- the pass over cut lists, its merge ---------------------------------------------------
+constexpr int kCutThreads = 256;
+// The results of the cut queries: the first pass's k best, and what their cut
+// lists, run again, have above the k-th of them.  A row met twice (in the results,
+// or in tiles that overlap) counts once.  More new rows than the block holds, or
+// (k > 32) a list cut again, flag the query's block.
+constexpr int kCutNew = 3072;
+constexpr int kMaxK = HS_TOPK_MAX_K;
+
+__global__ void __launch_bounds__(kCutThreads) cut_merge_kernel(
+    const Params p, float* __restrict__ out_s, int32_t* __restrict__ out_i, int32_t kout,
+    OutRows rows, const CutOut cut, int sms) {
+  pdl_wait();
+  pdl_trigger();
+  if (cut.queues.count[kMaxLists] == 0u) return;
+  __shared__ uint64_t s_res[kMaxK], s_new[kCutNew], s_kth;
+  __shared__ uint8_t s_dup[kCutNew];
+  __shared__ int s_n;
+  __shared__ CutTable t;
+  if (threadIdx.x < 32) make_cut_table(cut.queues, t, sms);
+  __syncthreads();
+  const int tid = threadIdx.x, k = p.k, per = 2 * (int)t.parts * k;
+  const int64_t n_queries = cut.queues.Q, R = rows.inv ? rows.n_out : n_queries;
+  for (int64_t o = blockIdx.x; o < R; o += gridDim.x) {
+    const int64_t q = rows.inv ? (int64_t)__ldg(rows.inv + o) : o;
+    const int np = q >= 0 && q < n_queries ? (int)cut.pairs[q] : 0;   // block-uniform
+    if (np == 0) continue;
+    for (int i = tid; i < kout; i += kCutThreads) {
+      const uint64_t key = pack_key(out_s[(size_t)o * kout + i], out_i[(size_t)o * kout + i]);
+      s_res[i] = real_key(key) ? key : 0ull;
+    }
+    if (tid == 0) {
+      s_n = 0;
+      s_kth = 0ull;
+    }
+    __syncthreads();
+    const uint64_t kth = s_res[kout - 1];
+    for (int i = tid; i < np * per; i += kCutThreads) {
+      const uint2 at = cut.at[(size_t)q * cut.most + i / per];
+      const size_t e = ((size_t)t.row[at.x] + at.y) * per + i % per;
+      const uint64_t key = pack_key(p.part_s[e], p.part_i[e]);
+      if (!real_key(key) || key <= kth) continue;
+      int lo = 0, hi = kout;                       // the first result not above it
+      while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (s_res[mid] > key)
+          lo = mid + 1;
+        else
+          hi = mid;
+      }
+      if (lo < kout && s_res[lo] == key) continue;
+      const int n = atomicAdd(&s_n, 1);
+      if (n < kCutNew) s_new[n] = key;
+    }
+    __syncthreads();
+    const int n = min(s_n, kCutNew);
+    const bool over = s_n > kCutNew;               // k > 32: k <= 32 has 1024 at most
+    for (int i = tid; i < n; i += kCutThreads) {
+      bool dup = false;
+      for (int j = 0; j < i; ++j) dup |= s_new[j] == s_new[i];
+      s_dup[i] = dup;
+    }
+    __syncthreads();
+    for (int i = tid; i < kout + n && !over; i += kCutThreads) {
+      const bool is_new = i >= kout;
+      const uint64_t key = is_new ? s_new[i - kout] : s_res[i];
+      if (key == 0ull || (is_new && s_dup[i - kout])) continue;
+      int r = is_new ? 0 : i;
+      if (is_new)
+        for (int j = 0; j < kout; ++j) r += s_res[j] > key;
+      for (int j = 0; j < n; ++j) r += s_new[j] > key && !s_dup[j];
+      if (r >= kout) continue;
+      float sc;
+      int32_t id;
+      unpack_key(key, sc, id);
+      out_s[(size_t)o * kout + r] = sc;
+      out_i[(size_t)o * kout + r] = id;
+      if (r == kout - 1) s_kth = key;
+    }
+    __syncthreads();
+    if (kout > 32) {
+      const uint64_t best = s_kth;
+      bool again = over;
+      for (int l = tid; l < np * (per / k); l += kCutThreads) {
+        const uint2 at = cut.at[(size_t)q * cut.most + l / (per / k)];
+        const size_t e = ((size_t)t.row[at.x] + at.y) * per + (l % (per / k)) * k + k - 1;
+        const uint64_t key = pack_key(p.part_s[e], p.part_i[e]);
+        again |= real_key(key) && key >= best;
+      }
+      if (__syncthreads_or(again) && tid == 0) atomicOr(cut.block + q / BM, 1u);
+      if (tid == 0 && !over) cut.floor[q] = key_floor(best);
+    }
+    __syncthreads();                               // read before the next row's
   }
 }
 
@@ -1513,13 +1847,19 @@ bool make_map(CUtensorMap* map, const uint16_t* base, int64_t rows, int32_t d, u
 std::atomic<uint64_t> g_ret_wait_limit_ns{0};
 std::atomic<int> g_ret_withhold{0};
 
-template <int KREG, int CL, int RN>
+// The pass over cut lists: the ring, as the others', and the table.
+constexpr size_t kCutSmem = 1024 + (size_t)kCutStages * kCutStageBytes + kBarBytes + kEpiSmem +
+                            sizeof(CutTable);
+static_assert(kCutSmem <= 232448 && sizeof(CutTable) % 4 == 0, "shared memory per CTA");
+static_assert(8 * (2 * kCutStages + 4 + 2) + 8 + 8 <= kBarBytes, "barrier area");
+
+template <int KREG, int CL, int RN, bool CUT = false>
 hs_status configure_kernel() {
   static std::atomic<uint64_t> done{0};
   return once_per_device(done, [] {
-    return cuda_fail(cudaFuncSetAttribute(retrieve_kernel<KREG, CL, RN>,
+    return cuda_fail(cudaFuncSetAttribute(retrieve_kernel<KREG, CL, RN, CUT>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          RN > 0 ? 232448 : (int)Ring<CL>::smem),
+                                          RN > 0 ? 232448 : CUT ? (int)kCutSmem : (int)Ring<CL>::smem),
                      "retrieve smem attribute");
   });
 }
@@ -1544,14 +1884,14 @@ int64_t max_pairs() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<KREG, 2, 0>, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<KREG, 2, 0, false>, &cfg) != cudaSuccess) n = 0;
     cached = n;
     if (dev >= 0) per_device[dev].store(cached + 1);
   }
   return cached;
 }
 
-template <int KREG, int CL, int RN>
+template <int KREG, int CL, int RN, bool CUT = false>
 hs_status launch_kernel(const CUtensorMap& mq, const CUtensorMap& mc, const Params& prm,
                         int64_t grid, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
@@ -1564,11 +1904,11 @@ hs_status launch_kernel(const CUtensorMap& mq, const CUtensorMap& mc, const Para
   attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = RN > 0 ? res_smem(RN, prm.kb_count) : Ring<CL>::smem;
+  cfg.dynamicSmemBytes = RN > 0 ? res_smem(RN, prm.kb_count) : CUT ? kCutSmem : Ring<CL>::smem;
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = CL > 1 ? 2 : 1;
-  return cuda_fail(cudaLaunchKernelEx(&cfg, retrieve_kernel<KREG, CL, RN>, mq, mc, prm),
+  return cuda_fail(cudaLaunchKernelEx(&cfg, retrieve_kernel<KREG, CL, RN, CUT>, mq, mc, prm),
                    "retrieve launch");
 }
 
@@ -1653,19 +1993,40 @@ static size_t part_bytes(int64_t Q, int64_t N, int32_t k, int64_t sms) {
   return (((size_t)lists * 2 * k * 4) + 255) & ~(size_t)255;
 }
 
+// Workspace: lists, large-k lists, then what is cleared (floors, block flags, and
+// for k > 16 how many lists of each query and queries of each list were cut), and
+// for k > 16 which they were.
 // Upper bound over every query count up to Q: a plan's split count is at most
 // max_splits() and the grid is at most the SM count, so one workspace serves
 // every batch of at most Q queries.
+struct Workspace {
+  size_t part, list;                    // sizes: two of each, at 0 and 2 * part
+  size_t floor, flags, pairs, count, clear_end, queue, at, total;
+};
+constexpr int kFewSlots = 12;           // of a first pass's lists, at the fewest
+static Workspace workspace(int64_t Q, int64_t N, int32_t k) {
+  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const int64_t sms = num_sms();
+  Workspace w{};
+  w.part = part_bytes(Q, N, k, sms);
+  w.list = k <= 32 ? 0 : up((size_t)sms * kEpi * 2 * k * 4);
+  const bool cut = k > 16;
+  size_t o = 2 * w.part + 2 * w.list;
+  w.floor = o;       o += up((size_t)Q * 4);
+  w.flags = o;       o += up((size_t)((Q + BM - 1) / BM) * 4);
+  w.pairs = o;       o += cut ? up((size_t)Q * 4) : 0;
+  w.count = o;       o += cut ? up((kMaxLists + 1) * 4) : 0;
+  w.clear_end = o;
+  w.queue = o;       o += cut ? up((size_t)kMaxLists * Q * 4) : 0;
+  w.at = o;          o += cut ? up((size_t)Q * (k / kFewSlots) * sizeof(uint2)) : 0;
+  w.total = o;
+  return w;
+}
+
 size_t retrieve_topk_workspace(int64_t Q, int64_t N, int32_t d, int32_t k) {
   if (Q <= 0 || N <= 0 || k <= 0) return 256;
-  const int64_t sms = num_sms();
-  const size_t part = part_bytes(Q, N, k, sms);
-  const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
-  const size_t qfloor = (((size_t)Q * 4) + 255) & ~(size_t)255;
-  const size_t flags = ((((size_t)(Q + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
-  // lists, large-k lists, shared floors, block flags, rows of a copy of queries
-  // and their number, large-k floors, the copy
-  return 2 * part + 2 * list + 3 * qfloor + flags + 256 + (k > 16 ? (size_t)Q * d * 2 : 0) + 256;
+  (void)d;
+  return workspace(Q, N, k).total;
 }
 
 // Qmax rows of `queries` are addressable; the kernels process the first
@@ -1680,14 +2041,12 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   if (!err) return fail(HS_ERR_CUDA, "could not resolve the device error word");
   const int64_t sms = num_sms();
   const int64_t tiles = (N + BN - 1) / BN;
-  const size_t need = retrieve_topk_workspace(Qmax, N, d, k);
-  if (ws_bytes < need)
-    return fail(HS_ERR_WORKSPACE, "retrieve workspace too small: %zu < %zu", ws_bytes, need);
+  const Workspace L = workspace(Qmax, N, k);
+  if (ws_bytes < L.total)
+    return fail(HS_ERR_WORKSPACE, "retrieve workspace too small: %zu < %zu", ws_bytes, L.total);
   CUtensorMap mq;
   if (!make_map(&mq, queries, Qmax, d, BM))
     return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
-  const size_t part = part_bytes(Qmax, N, k, sms);
-  const size_t list = k <= 32 ? 0 : ((((size_t)sms * kEpi * 2 * k * 4) + 255) & ~(size_t)255);
   char* w = static_cast<char*>(ws);
   Params prm{};
   prm.Qmax = Qmax;
@@ -1699,19 +2058,12 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   prm.wait_limit_ns = g_ret_wait_limit_ns.load();
   prm.withhold_first = g_ret_withhold.load();
   prm.part_s = reinterpret_cast<float*>(w);
-  prm.part_i = reinterpret_cast<int32_t*>(w + part);
-  prm.list_s = reinterpret_cast<float*>(w + 2 * part);
-  prm.list_i = reinterpret_cast<int32_t*>(w + 2 * part + list);
-  const size_t qfloor_bytes = (((size_t)Qmax * 4) + 255) & ~(size_t)255;
-  prm.qfloor = reinterpret_cast<uint32_t*>(w + 2 * part + 2 * list);
-  const size_t flag_bytes = ((((size_t)(Qmax + BM - 1) / BM) * 4) + 255) & ~(size_t)255;
-  char* wf = w + 2 * part + 2 * list + qfloor_bytes;
-  uint32_t* block_flags = reinterpret_cast<uint32_t*>(wf);
-  uint32_t* copy_slot = reinterpret_cast<uint32_t*>(wf + flag_bytes);
-  uint32_t* copy_count = reinterpret_cast<uint32_t*>(wf + flag_bytes + qfloor_bytes);
-  const size_t clear_bytes = qfloor_bytes + flag_bytes + qfloor_bytes + 256;
-  float* kth = reinterpret_cast<float*>(wf + flag_bytes + qfloor_bytes + 256);
-  uint16_t* copy = reinterpret_cast<uint16_t*>(wf + flag_bytes + 2 * qfloor_bytes + 256);
+  prm.part_i = reinterpret_cast<int32_t*>(w + L.part);
+  prm.list_s = reinterpret_cast<float*>(w + 2 * L.part);
+  prm.list_i = reinterpret_cast<int32_t*>(w + 2 * L.part + L.list);
+  prm.qfloor = reinterpret_cast<uint32_t*>(w + L.floor);
+  prm.raise_floor = 1;
+  uint32_t* block_flags = reinterpret_cast<uint32_t*>(w + L.flags);
   prm.err = err;
   const bool small = Qmax <= SQ_N && k <= 32 && prm.kb_count <= SQ_MAXKB;
   // Up to 64 queries stay in shared memory, which leaves the ring to the
@@ -1751,7 +2103,7 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
             pm, os, oi, kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
-    if (kout > 32 && kout <= kMrMaxK && pm.k <= 32 && oi && nr <= 12 * sms) {
+    if (kout > 32 && kout <= kMrMaxK && pm.k <= 32 && nr <= 12 * sms) {
       const int64_t blocks = std::min<int64_t>(nr, 6 * sms);
       merge_rank_kernel<32 * kMrMaxK><<<dim3((unsigned)blocks), dim3(kMrThreads), 0, stream>>>(
           pm, os, oi, kout, orows, cut);
@@ -1762,18 +2114,15 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       const dim3 grid((unsigned)(blocks < sms * 16 ? blocks : sms * 16));
       // lists per query <= 2 * slots (nsplit <= slots): lanes need that / 32
       const int64_t lpl = (2 * (int64_t)pm.slots + 31) / 32;
-      if (lpl <= 2)
-        launch_pdl(merge_warp_kernel<2>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   cut);
-      else if (lpl <= 3)
-        launch_pdl(merge_warp_kernel<3>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   cut);
-      else if (lpl <= 5)
-        launch_pdl(merge_warp_kernel<5>, grid, dim3(256), 0, stream, pm, os, oi, kout, orows,
-                   cut);
-      else
-        launch_pdl(merge_warp_kernel<kMaxListsPerLane>, grid, dim3(256), 0, stream, pm, os, oi,
-                   kout, orows, cut);
+      auto* kernel = cut.floor ? (lpl <= 2   ? merge_warp_kernel<2, true>
+                                  : lpl <= 3 ? merge_warp_kernel<3, true>
+                                  : lpl <= 5 ? merge_warp_kernel<5, true>
+                                             : merge_warp_kernel<kMaxListsPerLane, true>)
+                               : (lpl <= 2   ? merge_warp_kernel<2, false>
+                                  : lpl <= 3 ? merge_warp_kernel<3, false>
+                                  : lpl <= 5 ? merge_warp_kernel<5, false>
+                                             : merge_warp_kernel<kMaxListsPerLane, false>);
+      launch_pdl(kernel, grid, dim3(256), 0, stream, pm, os, oi, kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }
   };
@@ -1806,27 +2155,26 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     const int64_t lists =
         resident ? 2 * split_plan(1, wide ? tiles : (N + 127) / 128, 16, sms, 1).nsplit
                  : fewest_lists(Qmax, count_dev != nullptr, tiles, 16, sms);
-    const int32_t few = 4 * (int64_t)k <= 5 * lists ? 12 : 2 * (int64_t)k <= 7 * lists ? 16 : 32;
+    const int32_t few = 4 * (int64_t)k <= 5 * lists ? kFewSlots : 2 * (int64_t)k <= 7 * lists ? 16 : 32;
     const bool guess = k > 32 ? (int64_t)k <= 32 * tiles : k > 16 && few < 32;
     // The shared per-query floors of the register-list passes start empty, and
     // no query or block is flagged.
-    const size_t clear = guess ? clear_bytes : (size_t)Qmax * 4;
-    cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, clear, stream);
+    const size_t clear = guess ? L.clear_end - L.floor : (size_t)Qmax * 4;
+    const cudaError_t ze = cudaMemsetAsync(prm.qfloor, 0, clear, stream);
     if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
     // Whole-corpus pass of register lists.
-    auto pass = [&](Params& pm, int32_t slots, const uint16_t* from,
-                    const CUtensorMap& map) -> hs_status {
+    auto pass = [&](Params& pm, int32_t slots) -> hs_status {
       if (resident) {
         auto* launch = slots <= 8    ? (wide ? launch_resident<8, 256> : launch_resident<8, 128>)
                        : slots <= 12 ? (wide ? launch_resident<12, 256> : launch_resident<12, 128>)
                        : slots <= 16 ? (wide ? launch_resident<16, 256> : launch_resident<16, 128>)
                                      : (wide ? launch_resident<32, 256> : launch_resident<32, 128>);
-        return launch(from, corpus, N, d, pm, stream);
+        return launch(queries, corpus, N, d, pm, stream);
       }
-      return slots <= 8    ? launch_variant<8>(corpus, N, d, map, pm, stream)
-             : slots <= 12 ? launch_variant<12>(corpus, N, d, map, pm, stream)
-             : slots <= 16 ? launch_variant<16>(corpus, N, d, map, pm, stream)
-                           : launch_variant<32>(corpus, N, d, map, pm, stream);
+      return slots <= 8    ? launch_variant<8>(corpus, N, d, mq, pm, stream)
+             : slots <= 12 ? launch_variant<12>(corpus, N, d, mq, pm, stream)
+             : slots <= 16 ? launch_variant<16>(corpus, N, d, mq, pm, stream)
+                           : launch_variant<32>(corpus, N, d, mq, pm, stream);
     };
     st = HS_OK;
     if (guess) {
@@ -1843,12 +2191,18 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       // an average of 1.25, 16 for 3.5 and 32 for 16 (k = 32 tiles, two lists a
       // tile) leave one of 128 queries cut once in 1,000 batches or less, but
       // for the last (one in 20).  Queries whose best rows lie side by side in
-      // the corpus are cut more often: they are copied together by the merge and
-      // run with 32 slots, which for k <= 32 are always enough; the blocks of
-      // those cut again, or at first with 32 slots, are run exactly.  One query
-      // in 100 with 20 neighbours among its best, 300 queries over 131,072 x 384:
-      // k = 32 208 us, k = 50 219 (whole blocks run again: 293 and 304; 32 slots
-      // from the start: 200 and 241).
+      // the corpus, as chunks of a document do, are cut more often.  Their cut
+      // lists alone are run again, the queries of each taken from their places
+      // side by side, over that list's rows, from the k-th best score so far as
+      // a floor; with min(k, 32) slots they are enough for k <= 32.  The blocks of
+      // queries cut again, or at first with 32 slots, are run exactly, from the
+      // floor too.  300 queries over 131,072 x 384, 20 neighbours among the best of
+      // none, 1 in 100, all of the queries, us: k = 17 94 / 111 / 133, k = 32 101 /
+      // 117 / 139 (32 slots from the start 145 / 145 / 146 and 199 / 199 / 205),
+      // k = 50 of all 132 (986 with 32 slots, then exactly); 2000 over 262,144 x
+      // 768, k = 17 523 / 561 / 712 (564 / 560 / 646), k = 100 of all 882 (6100).
+      // What it can cost is one more reading of the corpus, where the best of a
+      // query crowd in nearly every list: 256 over 262,144 x 1536, k = 17 290 (194).
       // The slots decide the time, as a list starts by taking nearly all it
       // sees: 300 queries over 131,072 x 384, k = 50: 237 us with 32 slots, 146
       // with 16, 126 with 12 (105 with the merge by rank and skipped passes that
@@ -1857,69 +2211,60 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       Params pa = prm;
       pa.k = few;
       pa.qfloor = nullptr;
+      pa.raise_floor = 0;
       CutOut cut{};
-      if (few == 32) {
-        cut.block = block_flags;
-      } else {
-        cut.slot = copy_slot;
-        cut.count = copy_count;
-        cut.queries = reinterpret_cast<const uint4*>(queries);
-        cut.copy = reinterpret_cast<uint4*>(copy);
-        cut.row16 = d / 8;
+      cut.block = block_flags;
+      cut.floor = prm.qfloor;
+      if (few < 32) {
+        cut.pairs = reinterpret_cast<uint32_t*>(w + L.pairs);
+        cut.at = reinterpret_cast<uint2*>(w + L.at);
+        cut.most = k / few;
       }
-      st = pass(pa, few, queries, mq);
+      st = pass(pa, few);
+      if (few < 32) {
+        CutQueues& c = cut.queues;
+        c.count = reinterpret_cast<uint32_t*>(w + L.count);
+        c.queue = reinterpret_cast<uint32_t*>(w + L.queue);
+        c.list_k = few;
+        c.slots = pa.slots;
+        c.cl = pa.cl;
+        c.tiles = pa.tiles;
+        c.Q = Qmax;
+        c.count_dev = count_dev;
+        c.tile_rows = resident && !wide ? 128 : BN;
+        // The lists of this pass go where the first pass's were: at most
+        // Q * k / few * 2 * parts of 32 entries, where max_splits() * 2 * Q * k fit.
+        c.most_parts = (int32_t)std::min<int64_t>(8, max_splits(sms, tiles, k) * 3 / 8);
+      }
       if (st == HS_OK) st = merge(pa, k, scores_out, ids_out, rows, cut);
       if (st != HS_OK) return st;
       count_launches(2);
-      prm.only = block_flags;
       if (few < 32) {
-        CUtensorMap mcopy;
-        if (!make_map(&mcopy, copy, Qmax, d, BM))
+        CUtensorMap mq1, mc;
+        if (!make_map(&mq1, queries, Qmax, d, 1) || !make_map(&mc, corpus, N, d, kCutRows))
           return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
         Params pc = prm;
         pc.k = k <= 32 ? k : 32;
-        pc.only = nullptr;
-        pc.slot = copy_slot;
-        pc.count_dev = reinterpret_cast<const int32_t*>(copy_count);
-        pc.all_dev = count_dev;
-        CutOut again{};
-        if (k > 32) {
-          pc.qfloor = nullptr;
-          again.block = block_flags;
-        }
-        st = pass(pc, pc.k, copy, mcopy);
-        if (st == HS_OK) st = merge(pc, k, scores_out, ids_out, rows, again);
+        pc.raise_floor = k <= 32;
+        pc.cut = cut.queues;
+        st = configure_kernel<0, 1, 0, true>();
+        if (st == HS_OK) st = launch_kernel<0, 1, 0, true>(mq1, mc, pc, sms, stream);
+        if (st != HS_OK) return st;
+        launch_pdl(cut_merge_kernel,
+                   dim3((unsigned)std::min<int64_t>(std::max<int64_t>(R, 1), 4 * sms)),
+                   dim3(kCutThreads), 0, stream, pc, scores_out, ids_out, k, rows, cut, (int)sms);
+        st = cuda_fail(cudaGetLastError(), "cut merge launch");
         if (st != HS_OK) return st;
         count_launches(2);
         if (k <= 32) return HS_OK;
       }
+      prm.only = block_flags;
     }
     if (k <= 32) {
-      st = pass(prm, k, queries, mq);
+      st = pass(prm, k);
     } else {
-      // The exact path of large k, in two passes.  Pass 1: register lists over
-      // the first eighth of the corpus, whose union's k-th best is a score k
-      // distinct rows reach, hence a floor; pass 2: the large-k kernel over the
-      // whole corpus keeping scores >= the floor.  All passes' lists go through
-      // the same workspace; the floors are staged in it.  Pass 1 needs eight
-      // tiles of its own.
-      if (tiles >= 64 && prm.only) {
-        Params p1 = prm;
-        p1.tiles = tiles / 8;
-        p1.N = p1.tiles * BN;
-        p1.k = 32;
-        st = launch_variant<32>(corpus, N, d, mq, p1, stream);
-        if (st != HS_OK) return st;
-        st = merge(p1, k, kth, nullptr, OutRows{nullptr, 0});
-        if (st != HS_OK) return st;
-        count_launches(2);
-        prm.floor = kth;
-        prm.floor_stride = 1;
-        prm.floor_index = 0;
-        // Pass 1's shared floors bound 32nd-best scores, not k-th best: clear.
-        ze = cudaMemsetAsync(prm.qfloor, 0, (size_t)Qmax * 4, stream);
-        if (ze != cudaSuccess) return cuda_fail(ze, "floor clear");
-      }
+      // The exact path of large k: of the flagged blocks, whose queries start
+      // with the floor that the merges gave, or of all.
       st = launch_variant<0>(corpus, N, d, mq, prm, stream);
     }
   }

@@ -223,15 +223,19 @@ def test_device_count_zero_and_clamped():
     assert torch.equal(s2, ref_s) and torch.equal(i2, ref_i)
 
 
-def test_large_k_floor_with_ties_beyond_k():
-    # 60 exact copies of each query, some inside the first eighth of the
-    # corpus (the floor sample): the floor equals the copies' score, every
-    # copy ties with it, and the top 40 must be the 40 lowest-index copies.
+@pytest.mark.parametrize("spread", [True, False])
+def test_large_k_floor_with_ties_beyond_k(spread):
+    # 60 exact copies of each query: the k-th best score so far, which later
+    # passes take as their floor, is the copies' score, every copy ties with
+    # it, and the top 40 must be the 40 lowest-index copies.  Spread over the
+    # corpus no list is cut and there are no later passes; side by side, in one
+    # list's rows, the first pass's list is cut, and so is the one run again
+    # (32 slots), so that the exact pass runs from the floor.
     nq, N, d, k = 6, 40000, 128, 40
     Q, C = unit_pair(nq, N, d, 21)
     rng = np.random.default_rng(3)
     for q in range(nq):
-        pos = rng.choice(N, size=60, replace=False)
+        pos = rng.choice(N, size=60, replace=False) if spread else 256 * (3 + 20 * q) + np.arange(60)
         C[pos] = Q[q]
     gs, gi = gpu_topk(to_dev(Q), to_dev(C), k)
     parity(Q, C, k, gs, gi, range(nq))
@@ -239,9 +243,9 @@ def test_large_k_floor_with_ties_beyond_k():
     assert (gi == oi).all()
 
 
-def test_large_k_best_rows_outside_the_sample():
-    # The best rows of every query sit in the last part of the corpus, so the
-    # floor from the first eighth is far below the final k-th score.
+def test_large_k_best_rows_at_the_end():
+    # The best rows of every query sit side by side in the last part of the
+    # corpus, 200 in a row, so a list and the list run again are both cut.
     nq, N, d, k = 5, 40000, 128, 64
     Q, C = unit_pair(nq, N, d, 22)
     for q in range(nq):

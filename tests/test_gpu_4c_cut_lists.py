@@ -194,3 +194,19 @@ def test_cut_lists_cost_their_own_rows():
         us.append(_us(lambda: hs.hs_retrieve_topk(dq, c, k, workspace=ws, out=out)))
     hs.hs_get_device_error()
     assert us[1] < 1.9 * us[0], us
+
+
+def test_many_results_for_few_queries():
+    """The merge of more than 128 results takes a round per result, by the number of
+    lists: wide rows (1024), whose ring allows tiles of 128 only, do not get more of
+    them than rows of 768 (1.24 times the time with twice as many; 1.02 without)."""
+    us = []
+    for d in (768, 1024):
+        q, c = dev(synth.unit_rows(3, d, 1)), dev(synth.unit_rows(32768, d, 2))
+        ws = torch.empty(hs.hs_retrieve_topk_workspace(3, 32768, d, 500), dtype=torch.uint8,
+                         device="cuda")
+        out = (torch.empty((3, 500), device="cuda"),
+               torch.empty((3, 500), dtype=torch.int32, device="cuda"))
+        us.append(_us(lambda: hs.hs_retrieve_topk(q, c, 500, workspace=ws, out=out)))
+    hs.hs_get_device_error()
+    assert us[1] < 1.12 * us[0], us

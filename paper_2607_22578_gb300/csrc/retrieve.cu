@@ -1126,9 +1126,9 @@ __device__ __forceinline__ void add_pair(const CutOut& c, int64_t q, int32_t i, 
   c.at[(size_t)q * c.most + i] = make_uint2((uint32_t)list, at);
 }
 
-// (-0 as +0: they are equal, and keys order as the lists do.)
+// Keys order as the lists do: scores are sums that start from +0, so none is -0.
 __device__ __forceinline__ uint64_t pack_key(float s, int32_t idx) {
-  uint32_t u = __float_as_uint(s + 0.0f);
+  uint32_t u = __float_as_uint(s);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((uint64_t)u << 32) | (uint64_t)(0xffffffffu - (uint32_t)idx);
 }
@@ -2093,14 +2093,23 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     if (2 * (int64_t)pm.slots > 32 * kMaxListsPerLane)
       return fail(HS_ERR_UNSUPPORTED, "more lists per query than the merge takes");
     // Up to 32 results: a block per row while there is an SM for each (256 rows
-    // of 152 lists take 1 to 2 us more than with a warp each) and k is worth it
-    // (k = 1: 0.5 to 1 us more).  More results: up to twelve rows per SM (1000
-    // rows, k = 50 and 100, 8 and 19 us less than with a warp each; 4000 rows 15
-    // more).  After the main kernel it is launched in plain stream
-    // order: with its blocks waiting beside it, their shared memory cost the
-    // next retrieval up to 45 us; after the small-batch kernel it does not.
-    if (kout >= 4 && kout <= 32 && nr <= sms) {
-      if (small)
+    // of 152 lists take 1 to 2 us more than with a warp each), and k is worth it:
+    // a block ranks the lists' heads, a warp takes k rounds.  us, block / warp, after
+    // the small-batch kernel: 16 lists, k = 4 7.4 / 7.3; 64, k = 6 9.2 / 9.0, k = 8
+    // 9.5 / 9.8; 152, k = 8 23.6 / 22.9, k = 16 28.3 / 29.4; after the main kernel:
+    // 30, k = 4 16.4 / 16.5; 152, k = 6 61.7 / 62.5; 304, k = 8 43.2 to 47.2 / 41.2 to
+    // 46.9, k = 10 48.1 to 53.0 / 47.5 to 53.4, k = 16 67.8 / 71.2.
+    // More results: up to twelve rows per SM (1000 rows, k = 50 and 100, 8 and 19
+    // us less than with a warp each; 4000 rows 15 more).
+    // After the main kernel it is launched in plain stream order: with its
+    // blocks waiting beside it, their shared memory cost the next retrieval up to
+    // 45 us.  After the small-batch kernel it is launched early, 0.4 us less, but
+    // not where that leaves too few SMs free for a block each, as all of them then
+    // wait there (8 queries over 19,000 x 128, k = 16: 27.0 early, 17.2 plain).
+    const int64_t lists = 2 * split_plan(Qmax, pm.tiles, pm.k, pm.slots, pm.cl).nsplit;
+    const bool ranked = small ? 30 * (int64_t)(kout - 4) >= lists : 60 * (int64_t)(kout - 3) >= lists;
+    if (ranked && kout <= 32 && nr <= sms) {
+      if (small && (lists >= sms || nr <= sms - lists))
         launch_pdl(merge_rank_kernel<32 * 32>, dim3((unsigned)nr), dim3(kMrThreads), 0, stream, pm,
                    os, oi, kout, orows, cut);
       else

@@ -19,6 +19,27 @@ def to_dev(a: np.ndarray):
     return torch.from_numpy(a).cuda()
 
 
+def graph_us(f, n=10, replays=8) -> float:
+    """GPU time of one call of f, n calls in a captured graph: the least of a few
+    replays, so that a test can hold two calls against each other."""
+    import torch
+    f()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(n):
+            f()
+    best = float("inf")
+    for _ in range(replays):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        g.replay()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / n)
+    return best
+
+
 def fp_host(t) -> np.ndarray:
     return t.cpu().numpy().view(np.uint64)
 

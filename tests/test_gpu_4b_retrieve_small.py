@@ -8,7 +8,7 @@ import torch
 
 import paper_2607_22578_gb300 as hs
 import synth
-from hs_testutil import bf16_f64, to_dev
+from hs_testutil import bf16_f64, graph_us, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -156,3 +156,18 @@ def test_lists_shorter_than_k_with_fanout(n_live, k):
     s, i = s.cpu().numpy(), i.cpu().numpy().astype(np.int64)
     assert np.abs(s - want).max() < 1e-3
     assert np.abs(np.take_along_axis(full[inv], i, 1) - want).max() < 1e-3
+
+
+def test_small_batch_merge_with_few_sms_free():
+    """8 queries over 19,000 rows, whose 150 CTAs leave 2 SMs free: no dearer than over
+    20,480 (1.4 times with the merge's blocks launched early, all onto those two)."""
+    us = []
+    for n in (19000, 20480):
+        q, c = (to_dev(synth.unit_rows(m, 128, m)).view(torch.bfloat16) for m in (8, n))
+        ws = torch.empty(hs.hs_retrieve_topk_workspace(8, n, 128, 10), dtype=torch.uint8,
+                         device="cuda")
+        out = (torch.empty((8, 10), device="cuda"),
+               torch.empty((8, 10), dtype=torch.int32, device="cuda"))
+        us.append(graph_us(lambda: hs.hs_retrieve_topk(q, c, 10, workspace=ws, out=out)))
+    hs.hs_get_device_error()
+    assert us[0] < 1.15 * us[1], us

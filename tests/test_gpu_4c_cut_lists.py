@@ -7,7 +7,7 @@ import torch
 
 import paper_2607_22578_gb300 as hs
 import synth
-from hs_testutil import bf16_f64, to_dev
+from hs_testutil import bf16_f64, graph_us, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -157,24 +157,6 @@ def test_wait_runs_out_with_cut_lists(k):
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
 
 
-def _us(f, n=10):
-    f()
-    torch.cuda.synchronize()
-    g = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(g):
-        for _ in range(n):
-            f()
-    best_us = 1e9
-    for _ in range(8):
-        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        a.record()
-        g.replay()
-        b.record()
-        b.synchronize()
-        best_us = min(best_us, a.elapsed_time(b) * 1e3 / n)
-    return best_us
-
-
 def test_cut_lists_cost_their_own_rows():
     """300 queries whose 20 best rows are neighbours, k = 17, against the same batch
     on a corpus in random order: 1.4 times the time (2.5 times with a second pass of
@@ -191,7 +173,7 @@ def test_cut_lists_cost_their_own_rows():
                          device="cuda")
         out = (torch.empty((300, k), device="cuda"),
                torch.empty((300, k), dtype=torch.int32, device="cuda"))
-        us.append(_us(lambda: hs.hs_retrieve_topk(dq, c, k, workspace=ws, out=out)))
+        us.append(graph_us(lambda: hs.hs_retrieve_topk(dq, c, k, workspace=ws, out=out)))
     hs.hs_get_device_error()
     assert us[1] < 1.9 * us[0], us
 
@@ -207,6 +189,6 @@ def test_many_results_for_few_queries():
                          device="cuda")
         out = (torch.empty((3, 500), device="cuda"),
                torch.empty((3, 500), dtype=torch.int32, device="cuda"))
-        us.append(_us(lambda: hs.hs_retrieve_topk(q, c, 500, workspace=ws, out=out)))
+        us.append(graph_us(lambda: hs.hs_retrieve_topk(q, c, 500, workspace=ws, out=out)))
     hs.hs_get_device_error()
     assert us[1] < 1.12 * us[0], us

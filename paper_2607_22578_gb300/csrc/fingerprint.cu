@@ -30,14 +30,15 @@ using namespace fnv;
 // exactly as if the padding had not been there.  So every lane runs the same
 // straight-line hash whatever its row's start and length, in one pass.
 //
-// Bound by the memory system: 16 warps an SM each keep one 128-byte chunk per
-// lane in flight, in as many places as there are rows.  400,000 rows of 64 to
-// 512 tokens: 115 us, 4.0 TB/s (116 us as a pass over full chunks and a second
-// one over the rests); 200,000 rows of 512: 82 us, 5.0 TB/s (86); 400,000 rows
-// of at most 36: 20 us (26); 20,011 rows at a stride of 333: 23 us cold (132 us
-// hashing word by word).  Rests queued and hashed 32 at a time, steps left
-// out by a vote of the warp, and loads with a 256-byte prefetch or a bulk
-// prefetch to L2 were each slower.
+// Bound by the memory system where there are rows enough: 16 warps an SM each keep
+// one 128-byte chunk per lane in flight, in as many places as there are rows.
+// 200,000 rows of 512 tokens: 81 us, 5.0 TB/s; 400,000 rows of 8 to 36: 19.6 us
+// (23.6 as a pass over full chunks and a second one over the rests); 20,011 rows at a
+// stride of 333: 19 us (75 hashing word by word), where the chain bounds it.  Rests
+// queued and hashed 32 at a time, masks or steps left out by a vote of the warp
+// (400,000 rows of 64 to 512: 113 -> 125), and loads with a 256-byte prefetch or a
+// bulk prefetch to L2 were each slower.  Long rows of unequal lengths go in those two
+// passes (two_passes below), rows of less than a chunk to the second alone.
 //
 // A chunk whose tokens are all below 65536 (in every live lane) takes the
 // two-round small-token hash; otherwise the whole chunk takes the octet-wise
@@ -58,7 +59,6 @@ __device__ __forceinline__ void load_vec(const int32_t* p, uint32_t* x) {
 }
 
 constexpr int kChunk = 32;      // T: tokens per chunk
-constexpr int kStep = 8;        // tokens per step that rows shorter than a chunk can leave out
 constexpr int kFpThreads = 256;
 
 // kUnpad.v[t] = prime^-(4 t): undoes t zero tokens.
@@ -74,8 +74,8 @@ constexpr Unpad make_unpad() {
 static_assert(make_unpad().v[1] * kPrime * kPrime * kPrime * kPrime == 1, "inverse of the prime");
 __constant__ Unpad kUnpad = make_unpad();
 
-// VB bytes per load, K loads per chunk, NB register buffers.  MASK: a chunk
-// may hold tokens that are not the row's (lengths, or a stride that is no
+// VB bytes per load, K loads per chunk, NB register buffers; stride >= T.  MASK: a
+// chunk may hold tokens that are not the row's (lengths, or a stride that is no
 // multiple of T); HEAD: and rows may start off a 16-byte boundary (4-byte
 // aligned), VB is then 16.
 template <int VB, int K, int NB, bool MASK, bool HEAD>
@@ -95,9 +95,6 @@ __global__ void __launch_bounds__(kFpThreads) fingerprint_kernel(
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t seed_lo = (uint32_t)seed, seed_hi = (uint32_t)(seed >> 32);
   const int32_t* const tokens_end = tokens + n * (int64_t)stride;
-  // Rows of fewer than T tokens (the same for every row): steps past them are
-  // left out.
-  const int used = MASK ? min(T, (stride + (HEAD ? 3 : 0) + kStep - 1) / kStep * kStep) : T;
 
   // Issue side: the row being loaded, its next chunk's first token (-3 ... -1
   // in a first chunk that starts before the row), its length.
@@ -206,22 +203,14 @@ __global__ void __launch_bounds__(kFpThreads) fingerprint_kernel(
     for (int t = 0; t < T; ++t) any |= buf[b][t];
     if (__all_sync(0xffffffffu, !live || (any >> 16) == 0u)) {
 #pragma unroll
-      for (int t0 = 0; t0 < T; t0 += kStep)
-        if (!MASK || t0 < used) {
-#pragma unroll
-          for (int t = t0; t < t0 + kStep; ++t) hash_word_small(lo, hi, buf[b][t]);
-        }
+      for (int t = 0; t < T; ++t) hash_word_small(lo, hi, buf[b][t]);
     } else {
 #pragma unroll
-      for (int t0 = 0; t0 < T; t0 += kStep)
-        if (!MASK || t0 < used) {
-#pragma unroll
-          for (int t = t0; t < t0 + kStep; ++t) hash_word_full(lo, hi, buf[b][t]);
-        }
+      for (int t = 0; t < T; ++t) hash_word_full(lo, hi, buf[b][t]);
     }
     if (live && blast[b]) {
       const uint64_t h = ((uint64_t)hi << 32) | lo;
-      fp_out[brow[b]] = MASK ? h * kUnpad.v[used - bend[b]] : h;
+      fp_out[brow[b]] = MASK ? h * kUnpad.v[T - bend[b]] : h;
     }
     brow[b] = -1;
   };
@@ -249,10 +238,9 @@ __global__ void __launch_bounds__(kFpThreads) fingerprint_kernel(
 
 // ---- few rows: a warp per row -------------------------------------------------------------
 // Bound by the latency of one row, which a warp cuts to eight prefix xors and
-// 32 rounds per 1024 octets (fnv.cuh).  It costs about three times the
+// 32 rounds per 1024 octets (fnv_warp.cuh).  It costs about three times the
 // instructions of a lane per row, so it is for batches that leave most of the
-// GPU idle.  A row of
-// 1536 octets takes 3.5 us with its launch where the chain takes 14.4.
+// GPU idle.  A row of 1536 octets takes 3.5 us with its launch where the chain takes 14.4.
 template <bool VEC>
 __global__ void __launch_bounds__(128) fingerprint_warp_kernel(
     const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
@@ -272,6 +260,34 @@ __global__ void __launch_bounds__(128) fingerprint_warp_kernel(
       if (bad) set_error(err, kErrInvalidArg);
       fp_out[r] = h;
     }
+  }
+}
+
+// ---- the tokens past a row's full chunks, or all of a short row: a thread per row ------
+// MAX tokens at most.  chunks: the chunk pass below has run, and left the state of
+// rows of a chunk and more.
+template <int MAX, bool VEC>
+__global__ void __launch_bounds__(kFpThreads) fingerprint_rests_kernel(
+    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
+    const int32_t* __restrict__ lens, uint64_t seed, bool chunks, uint64_t* __restrict__ fp_out,
+    unsigned* err) {
+  pdl_wait();
+  pdl_trigger();
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n;
+       r += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t L = lens ? __ldg(lens + r) : stride;
+    if (L < 0 || L > stride) {                             // reported, fingerprint 0
+      set_error(err, kErrInvalidArg);
+      fp_out[r] = 0ull;
+      continue;
+    }
+    const bool on = chunks && L >= kChunk;
+    const int32_t rest = on ? L % kChunk : L;
+    if (on && rest == 0) continue;
+    const uint64_t h = on ? fp_out[r] : seed;
+    uint32_t lo = (uint32_t)h, hi = (uint32_t)(h >> 32);
+    hash_tokens<MAX, VEC>(lo, hi, tokens + r * (int64_t)stride + (L - rest), rest);
+    fp_out[r] = ((uint64_t)hi << 32) | lo;
   }
 }
 
@@ -472,6 +488,20 @@ hs_status launch_fingerprint_chunks(const int32_t* tokens, int64_t n, int32_t st
   return st;
 }
 
+// Aligned rows in a pass over full chunks and one over the rests, or in one that
+// masks: masks cost every step of a chain, the second pass a launch and its own
+// reads.  us, one pass / two: lengths up to 1024, 12,000 rows 27.7 / 26.0, 40,000
+// 57.1 / 49.3, 200,000 117 / 108; up to 512, 12,000 15.4 / 16.0, 40,000 30.1 / 28.0,
+// 400,000 105 / 101; up to 256, 65,536 16.9 / 19.5, 100,000 23.6 / 22.2, 400,000 58.5 /
+// 58.2; up to 128, 100,000 14.8 / 16.1, 700,000 53.8 / 59.8; all of 36 tokens, 40,000
+// 6.9 / 8.6, 400,000 26.8 / 22.4, 700,000 38.3 / 36.8; all of 200, 6500 8.2 / 8.3, 40,000
+// 15.8 / 13.3, 400,000 75.9 / 72.8, 700,000 114 / 118.
+bool two_passes(int64_t n, int32_t stride, bool lens) {
+  if (stride >= 640) return true;
+  if (n > 80000) return lens ? stride >= 256 && n <= 1000 * (int64_t)stride : n < 600000;
+  return n >= 16384 && stride >= (lens ? 512 : 200);
+}
+
 // 32-byte loads where every row starts on such a boundary, else 16-byte loads.
 hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
                              const int32_t* lens, uint64_t seed, uint64_t* fp_out,
@@ -480,6 +510,26 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
   if (!err) return fail(HS_ERR_CUDA, "could not resolve the device error word");
   const uintptr_t base = reinterpret_cast<uintptr_t>(tokens);
   const bool vec16 = (base & 15u) == 0 && stride % 4 == 0;
+  auto rests = [&](bool chunks) {
+    auto* kernel = vec16 ? (stride <= 8    ? fingerprint_rests_kernel<8, true>
+                            : stride <= 16 ? fingerprint_rests_kernel<16, true>
+                            : stride <= 24 ? fingerprint_rests_kernel<24, true>
+                                           : fingerprint_rests_kernel<kChunk, true>)
+                         : (stride <= 8    ? fingerprint_rests_kernel<8, false>
+                            : stride <= 16 ? fingerprint_rests_kernel<16, false>
+                            : stride <= 24 ? fingerprint_rests_kernel<24, false>
+                                           : fingerprint_rests_kernel<kChunk, false>);
+    launch_pdl(kernel,
+               dim3((unsigned)std::min<int64_t>((n + kFpThreads - 1) / kFpThreads, num_sms() * 64)),
+               dim3(kFpThreads), 0, stream, tokens, n, stride, lens, seed, chunks, fp_out, err);
+    count_launches(1);
+    return cuda_fail(cudaGetLastError(), "fingerprint launch");
+  };
+  // Rows of fewer tokens than a chunk have a thread each: 1,000,000 rows of up to 4
+  // tokens 7 us (20 in the lanes' chunks), of 8 8.7 to 9.4 (19 to 26), of 16 15 to 21
+  // (24 to 32), of 28 31 to 41 (33 to 40).  Few rows of more than 16 have a warp
+  // (100 rows of 31: 3.1 us, 3.8 with a thread).
+  if (stride <= 16) return rests(false);
   // A warp per row takes 0.7 ns per row and 256 tokens at full size; a lane
   // per row the chain of the longest row, 17 ns per token (33 where rows are
   // not aligned), while that many lanes fit the GPU.  Measured, us, warp / lane:
@@ -495,7 +545,13 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "fingerprint launch");
   }
+  if (stride < kChunk) return rests(false);
   const bool whole = !lens && stride % kChunk == 0 && stride > 0;   // no masks needed
+  if (vec16 && !whole && two_passes(n, stride, lens != nullptr)) {
+    bool ran = false;
+    const hs_status st = launch_fingerprint_chunks(tokens, n, stride, lens, seed, fp_out, &ran, stream);
+    return st == HS_OK ? rests(ran) : st;
+  }
   if ((base & 31u) == 0 && stride % 8 == 0)
     return whole ? launch_rows<32, 4, 2, false, false>(tokens, n, stride, lens, seed, fp_out, err, stream)
                  : launch_rows<32, 4, 2, true, false>(tokens, n, stride, lens, seed, fp_out, err, stream);

@@ -58,5 +58,32 @@ __device__ __forceinline__ void hash_word(uint32_t& lo, uint32_t& hi, uint32_t w
     hash_word_full(lo, hi, w);
 }
 
+// The m < T tokens at src, every load issued before the first round.  VEC: src is
+// 16-byte aligned and its last piece may be read whole.
+template <int T, bool VEC>
+__device__ __forceinline__ void hash_tokens(uint32_t& lo, uint32_t& hi,
+                                            const int32_t* __restrict__ src, int m) {
+  uint32_t v[T];
+#pragma unroll
+  for (int t = 0; t < T; t += 4) {
+    if (VEC) {
+      if (t < m) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + t));
+        v[t] = x.x;
+        v[t + 1] = x.y;
+        v[t + 2] = x.z;
+        v[t + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int i = t; i < t + 4; ++i)
+        if (i < m) v[i] = (uint32_t)__ldg(src + i);
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (t < m) hash_word(lo, hi, v[t]);
+}
+
 }  // namespace fnv
 }  // namespace hs

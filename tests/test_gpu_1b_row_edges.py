@@ -8,7 +8,7 @@ import torch
 
 import oracle
 import paper_2607_22578_gb300 as hs
-from hs_testutil import to_dev
+from hs_testutil import graph_us, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -52,6 +52,76 @@ def test_fingerprint_on_both_sides_of_the_row_count(stride, big):
             hs.hs_get_device_error()
             want = oracle.fingerprint(tokens, L, seed=0xFFFFFFFFFFFFFFFF)
             assert (fp.cpu().numpy().view(np.uint64) == want).all(), (offset, n)
+
+
+@pytest.mark.parametrize("stride", [2, 8, 9, 12, 16, 17, 20, 24, 25, 28, 31])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_fingerprint_of_rows_shorter_than_a_chunk(offset, stride):
+    """A thread per row, with room for 8, 16, 24 or 32 tokens; few rows of more than
+    16 by a warp each."""
+    rng = np.random.default_rng(stride)
+    for n in (3, 700, 5003):
+        tokens, dev = rows_at(offset, n, stride, rng, bool(n % 2))
+        lens = rng.integers(0, stride + 1, size=n).astype(np.int32)
+        lens[[0, n - 1]] = stride
+        for L in (None, lens):
+            want = oracle.fingerprint(tokens, L)
+            fp = hs.hs_fingerprint(dev, None if L is None else to_dev(L))
+            hs.hs_get_device_error()
+            assert (fp.cpu().numpy().view(np.uint64) == want).all(), (n, L is None)
+        bad = lens.copy()
+        bad[1] = stride + 1
+        fp = hs.hs_fingerprint(dev, to_dev(bad))
+        with pytest.raises(hs.HsError):
+            hs.hs_get_device_error()
+        want[1] = 0
+        assert (fp.cpu().numpy().view(np.uint64) == want).all()
+
+
+@pytest.mark.parametrize("n,stride", [(7000, 644), (16384, 512), (16384, 200), (80001, 256),
+                                      (80001, 36), (16383, 508), (80000, 252)])
+def test_fingerprint_in_two_passes(n, stride):
+    """Aligned rows of which many have full chunks: chunks first, then the rests;
+    and beside each rule's line, in one pass."""
+    rng = np.random.default_rng(stride)
+    tokens, dev = rows_at(0, n, stride, rng, False)
+    lens = rng.integers(0, stride + 1, size=n).astype(np.int32)
+    lens[:4] = [0, 32, stride, 31]
+    for L in (None, lens):
+        fp = hs.hs_fingerprint(dev, None if L is None else to_dev(L), 7)
+        hs.hs_get_device_error()
+        assert (fp.cpu().numpy().view(np.uint64) == oracle.fingerprint(tokens, L, seed=7)).all()
+    bad = lens.copy()
+    bad[[1, n - 1]] = [-5, stride + 32]
+    fp = hs.hs_fingerprint(dev, to_dev(bad), 7)
+    with pytest.raises(hs.HsError) as e:
+        hs.hs_get_device_error()
+    assert e.value.status == hs.HS_ERR_INVALID_ARG
+    want = oracle.fingerprint(tokens, lens, seed=7)
+    want[[1, n - 1]] = 0
+    assert (fp.cpu().numpy().view(np.uint64) == want).all()
+
+
+def _ragged_us(n, stride, low):
+    t = torch.zeros((n, stride), dtype=torch.int32, device="cuda")
+    lens = torch.randint(low, stride + 1, (n,), dtype=torch.int32, device="cuda")
+    fp = torch.empty(n, dtype=torch.int64, device="cuda")
+    return graph_us(lambda: hs.hs_fingerprint(t, lens, fp_out=fp))
+
+
+def test_short_rows_cost_no_chunk():
+    """A million rows of up to 8 tokens take less than the half of as many of 24 to 28
+    (0.28; 0.56 where each took a lane's chunk)."""
+    assert _ragged_us(1000000, 8, 1) < 0.43 * _ragged_us(1000000, 28, 24)
+
+
+def test_long_ragged_rows_cost_no_masks():
+    """40,000 rows of up to 2048 tokens against as many of exactly 1024: 2.05 times the
+    time (2.5 times where every chunk is masked; the longest chain is twice as long)."""
+    t = torch.zeros((40000, 1024), dtype=torch.int32, device="cuda")
+    fp = torch.empty(40000, dtype=torch.int64, device="cuda")
+    whole = graph_us(lambda: hs.hs_fingerprint(t, fp_out=fp))
+    assert _ragged_us(40000, 2048, 1) < 2.25 * whole, whole
 
 
 def test_fingerprint_mixes_small_and_large_tokens_and_bad_lengths():

@@ -530,14 +530,15 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
   // (24 to 32), of 28 31 to 41 (33 to 40).  Few rows of more than 16 have a warp
   // (100 rows of 31: 3.1 us, 3.8 with a thread).
   if (stride <= 16) return rests(false);
-  // A warp per row takes 0.7 ns per row and 256 tokens at full size; a lane
-  // per row the chain of the longest row, 17 ns per token (33 where rows are
-  // not aligned), while that many lanes fit the GPU.  Measured, us, warp / lane:
-  // 4096 rows of 256 tokens 4.9 / 6.6, 8192 7.4 / 6.6; 2048 of 384 (octet-wise)
-  // 5.1 / 14.4; 2048 of 64 3.1 / 2.8; 1024 of 64 2.7 / 2.7; 8192 of 333 on any
-  // word 13.1 / 18.3, 16384 23.4 / 18.4.
+  // A warp per row takes 0.7 ns per row and 256 tokens at full size; a lane per
+  // row the chain of the longest row while that many lanes fit the GPU, 17 to 23 ns
+  // per token (50 where rows are not aligned).  us, warp / lane: aligned, 4096 rows
+  // of 256 tokens 4.9 / 6.6, 8192 7.4 / 6.6, 2048 of 384 (octet-wise) 5.1 / 14.4; on
+  // any word, all of 333 10,000 rows 15.9 / 18.9, 12,288 19.0 / 18.9, 16,384 24.0 /
+  // 18.9, of 128 10,000 9.0 / 9.9, 12,288 10.6 / 9.8, of 1024 16,384 44.9 / 51.0, 20,011
+  // 54.2 / 54.0.
   const int64_t work = n * (((int64_t)stride + 255) / 256);
-  if (n < (1 << 20) && work <= (vec16 ? 24 : 48) * (int64_t)stride) {
+  if (n < (1 << 20) && work <= (vec16 ? 24 : 72) * (int64_t)stride) {
     const int64_t blocks = (n + 3) / 4;
     launch_pdl(vec16 ? fingerprint_warp_kernel<true> : fingerprint_warp_kernel<false>,
                dim3((unsigned)std::min<int64_t>(blocks, num_sms() * 64)), dim3(128), 0, stream,

@@ -518,8 +518,11 @@ __global__ void __launch_bounds__(256) finalize_kernel(const int32_t* __restrict
 // lengths.  VEC: pieces of 16 bytes (16-byte aligned rows, stride % 4 == 0),
 // the tokens of a pair's last piece past its length masked.  Otherwise the
 // rows may start on any word and a piece is one word, coalesced over the
-// lanes, with twice as many in flight: 20,011 rows at a stride of 333, a third
-// of them copies, take 21 us cold (40 us as two rows per warp round).  Batches
+// lanes: 20,011 rows at a stride of 333, a third of them copies, take 21 us cold (40
+// us as two rows per warp round).  As many in flight as of the others: with eight,
+// whose registers cost a block in six, 1,000,000 rows of 31 words, a tenth of them
+// copies, take 106 us from fingerprints to inverse, 96 so, and the small batches are
+// no faster.  Batches
 // that do not fill the GPU with 32 rows per warp take fewer, down to 4, so a
 // warp's chain of rounds is shorter: with the scan's smaller tiles 20,011 rows
 // take 25 us from fingerprints to inverse (35), 65,536 rows of 256 tokens 33 (38).
@@ -541,7 +544,7 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
     unsigned* err) {
   pdl_wait();
   pdl_trigger();
-  constexpr int kPieces = VEC ? 4 : 8;
+  constexpr int kPieces = 4;
   __shared__ int32_t s_pre[kVerifyThreads / 32][32];
   __shared__ int32_t s_a[kVerifyThreads / 32][32];
   __shared__ int32_t s_b[kVerifyThreads / 32][32];

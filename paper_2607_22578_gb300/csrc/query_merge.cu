@@ -25,7 +25,7 @@
 // Bound by the launch and its dependent round trips (keys, verify, gather); at
 // 256 rows of 768 by each CTA's reading of all rows.  us with the launch, where
 // one thread hashed each row first: 1 row of 768 3.6 (15.0), 64 rows 7.0
-// (17.6), 256 rows 16.6 (28.1).  256 threads instead of 512: 64 rows 8.6.
+// (17.6), 256 rows 16.6 (28.1).
 //
 // Exactness: rows are grouped by key (the table keeps the smallest row index
 // per key), then every row whose group leader is another row is compared with
@@ -41,9 +41,8 @@ namespace {
 
 using namespace table;
 
-constexpr int kQmThreads = 512;
 constexpr int kQmMaxRows = 256;             // the first threads take a row each
-static_assert(kQmMaxRows <= kQmThreads && kQmMaxRows >= HS_MERGE_QUERIES_MAX, "a thread per row");
+static_assert(kQmMaxRows <= 256 && kQmMaxRows >= HS_MERGE_QUERIES_MAX, "a thread per row");
 constexpr int kQmLog2 = table_log2(kQmMaxRows);
 constexpr int kQmSlots = (1 << kQmLog2) + 1;
 constexpr int kQmMaxCtas = 32;
@@ -65,7 +64,8 @@ __device__ __forceinline__ uint64_t piece_key(const uint4& x, int v) {
 }
 
 // CTAs [0, merge_ctas) merge; the others hash rows (fp_in NULL, fp_out not).
-__global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) merge_queries_kernel(
     const uint4* __restrict__ q, int n, int nv, uint64_t seed, const uint64_t* __restrict__ fp_in,
     uint64_t* __restrict__ fp_out, int32_t* __restrict__ n_unique,
     int32_t* __restrict__ unique_idx, int32_t* __restrict__ inverse, uint4* __restrict__ uq,
@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
   pdl_wait();
   pdl_trigger();
   if ((int)blockIdx.x >= merge_ctas) {
-    const int warps = ((int)gridDim.x - merge_ctas) * (kQmThreads / 32);
-    for (int r = ((int)blockIdx.x - merge_ctas) * (kQmThreads / 32) + (int)(threadIdx.x >> 5);
+    const int warps = ((int)gridDim.x - merge_ctas) * (THREADS / 32);
+    for (int r = ((int)blockIdx.x - merge_ctas) * (THREADS / 32) + (int)(threadIdx.x >> 5);
          r < n; r += warps) {
       const uint64_t h = fnv::hash_row_warp<true>(
           reinterpret_cast<const uint32_t*>(q + (size_t)r * nv), nv * 4, seed);
@@ -90,14 +90,14 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
   __shared__ int32_t s_uidx[kQmMaxRows];
   __shared__ int32_t s_list[kQmMaxRows];
   __shared__ uint8_t s_diff[kQmMaxRows];
-  __shared__ int32_t s_warp[kQmThreads / 32];
+  __shared__ int32_t s_warp[THREADS / 32];
   __shared__ int32_t s_nlist, s_ncoll;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int log2T = table_log2(n);
   const int T1 = (1 << log2T) + 1;
   const bool row = tid < n;
 
-  for (int s = tid; s < T1; s += kQmThreads) {
+  for (int s = tid; s < T1; s += THREADS) {
     s_keys[s] = kEmpty;
     s_idx[s] = kNoRow;
   }
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
     // rows side by side.
     int group = 32;
     while (group > 1 && group / 2 >= nv) group /= 2;
-    const int groups = kQmThreads / group, gl = tid & (group - 1);
+    const int groups = THREADS / group, gl = tid & (group - 1);
     for (int base = 0; base < n; base += groups * kQmRows) {     // the same for every lane
       const int r0 = base + tid / group;
       uint64_t h[kQmRows];
@@ -165,12 +165,12 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
   // 3. verify every listed row against its leader, all 16-byte pairs in flight
   const int m = s_nlist;
   const int items = m * nv;
-  for (int b = tid; b < items; b += kQmThreads * kQmUnroll) {
+  for (int b = tid; b < items; b += THREADS * kQmUnroll) {
     uint4 x[kQmUnroll], y[kQmUnroll];
     int ra[kQmUnroll];
 #pragma unroll
     for (int u = 0; u < kQmUnroll; ++u) {
-      const int it = b + u * kQmThreads;
+      const int it = b + u * THREADS;
       ra[u] = -1;
       if (it < items) {
         const int li = it / nv, v = it - li * nv;
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
   __syncthreads();
   int32_t off = 0, total = 0;
 #pragma unroll
-  for (int w = 0; w < kQmThreads / 32; ++w) {
+  for (int w = 0; w < THREADS / 32; ++w) {
     off += w < warp ? s_warp[w] : 0;
     total += s_warp[w];
   }
@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(kQmThreads) merge_queries_kernel(
 
   // 6. gather the unique rows, split over the CTAs
   const int gitems = total * nv;
-  const int gstride = merge_ctas * kQmThreads;
-  for (int b = blockIdx.x * kQmThreads + tid; b < gitems; b += gstride * kQmUnroll) {
+  const int gstride = merge_ctas * THREADS;
+  for (int b = blockIdx.x * THREADS + tid; b < gitems; b += gstride * kQmUnroll) {
     uint4 x[kQmUnroll];
     int dst[kQmUnroll];
 #pragma unroll
@@ -271,10 +271,15 @@ hs_status launch_merge_queries(const uint16_t* queries, int64_t n, int32_t dim, 
     return cuda_fail(cudaMemsetAsync(n_unique, 0, sizeof(int32_t), stream), "n_unique clear");
   const int nv = dim / 8;                     // 16-byte vectors per row
   const int64_t work = n * (int64_t)nv;
-  int64_t grid = (work + kQmThreads * kQmUnroll - 1) / (kQmThreads * kQmUnroll);
+  // Few pieces leave most of 512 threads idle at every barrier.  us, 256 / 512: 1 row
+  // of 8 3.1 / 3.4, 64 of 16 4.0 / 4.2, 7 of 768 (672 pieces) 4.0 / 4.1, 64 of 128 (1024)
+  // 5.1 / 4.9, 64 of 768 9.4 / 7.3.
+  const int threads = work <= 640 ? 256 : 512;
+  int64_t grid = (work + threads * kQmUnroll - 1) / (threads * kQmUnroll);
   grid = grid < 1 ? 1 : (grid > kQmMaxCtas ? kQmMaxCtas : grid);
-  const int hash = !fp_in && fp_out ? (int)((n + kQmThreads / 32 - 1) / (kQmThreads / 32)) : 0;
-  launch_pdl(merge_queries_kernel, dim3((unsigned)(grid + hash)), dim3(kQmThreads), 0, stream,
+  const int hash = !fp_in && fp_out ? (int)((n + threads / 32 - 1) / (threads / 32)) : 0;
+  launch_pdl(threads == 256 ? merge_queries_kernel<256> : merge_queries_kernel<512>,
+             dim3((unsigned)(grid + hash)), dim3(threads), 0, stream,
              reinterpret_cast<const uint4*>(queries), (int)n, nv, seed, fp_in, fp_out, n_unique,
              unique_idx, inverse, reinterpret_cast<uint4*>(uq), (int)grid);
   count_launches(1);

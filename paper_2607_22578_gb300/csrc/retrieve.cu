@@ -865,9 +865,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc_fence_before();
         sort_desc<kGroups>(gm);
-        float kth = -FLT_MAX;
-#pragma unroll
-        for (int i = 0; i < kGroups; ++i) kth = i == k - 1 ? gm[i] : kth;
+        float kth = INFINITY;                  // the least of the first k, not gm[k - 1]:
+#pragma unroll                                 // an index would put gm in local memory
+        for (int i = 0; i < kGroups; ++i) kth = i < k ? fminf(kth, gm[i]) : kth;
         if (kth > -FLT_MAX) qf_theta = fmaxf(qf_theta, nextafterf(kth, -INFINITY));
       }
       for (int64_t t = t0; t < t1; ++t, ++tile_i) {

@@ -1912,29 +1912,38 @@ hs_status launch_kernel(const CUtensorMap& mq, const CUtensorMap& mc, const Para
                    "retrieve launch");
 }
 
-// Plan and launch for one register-list size.  Clusters of two when there
-// are at least two query blocks (they share corpus tiles), else single CTAs.
+// Unit executors of a launch: pairs of CTAs where there are two query blocks (they
+// share corpus tiles) and pairs can be resident, else single CTAs; at most kMaxLists
+// / 2, so every query's lists (2 per split, nsplit <= slots) fit the merges.
+struct Executors {
+  int cl;
+  int64_t slots;
+};
+template <int KREG>
+hs_status executors(int64_t Qmax, Executors* out) {
+  const int64_t sms = num_sms();
+  hs_status st = configure_kernel<KREG, 1, 0>();
+  if (st != HS_OK) return st;
+  *out = Executors{1, std::min<int64_t>(sms, kMaxLists / 2)};
+  if (Qmax > BM) {
+    st = configure_kernel<KREG, 2, 0>();
+    if (st != HS_OK) return st;
+    const int64_t pairs =
+        std::min<int64_t>(std::min<int64_t>(max_pairs<KREG>(), sms / 2), kMaxLists / 2);
+    if (pairs >= 1) *out = Executors{2, pairs};
+  }
+  return HS_OK;
+}
+
+// Plan and launch for one register-list size.
 template <int KREG>
 hs_status launch_variant(const uint16_t* corpus, int64_t N, int32_t d, const CUtensorMap& mq,
                          Params& prm, cudaStream_t stream) {
-  const int64_t sms = num_sms();
-  const int64_t qblocks_max = (prm.Qmax + BM - 1) / BM;
-  hs_status st = configure_kernel<KREG, 1, 0>();
+  Executors ex;
+  const hs_status st = executors<KREG>(prm.Qmax, &ex);
   if (st != HS_OK) return st;
-  int cl = 1;
-  // Unit executors: at most 16 * kMaxListsPerLane, so every query's lists
-  // (2 per split, nsplit <= slots) fit the warp merge.
-  int64_t slots = std::min<int64_t>(sms, 16 * kMaxListsPerLane);
-  if (qblocks_max >= 2) {
-    st = configure_kernel<KREG, 2, 0>();
-    if (st != HS_OK) return st;
-    const int64_t pairs = std::min<int64_t>(std::min<int64_t>(max_pairs<KREG>(), sms / 2),
-                                            16 * kMaxListsPerLane);
-    if (pairs >= 1) {
-      cl = 2;
-      slots = pairs;
-    }
-  }
+  const int cl = ex.cl;
+  const int64_t slots = ex.slots;
   CUtensorMap mc;
   if (!make_map(&mc, corpus, N, d, BN / cl))
     return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
@@ -1964,7 +1973,7 @@ hs_status launch_resident(const uint16_t* queries, const uint16_t* corpus, int64
   if (!make_map(&mq, queries, prm.Qmax, d, RQ) || !make_map(&mc, corpus, N, d, RN))
     return fail(HS_ERR_CUDA, "cuTensorMapEncodeTiled failed (driver entry point or arguments)");
   prm.tiles = (N + RN - 1) / RN;
-  prm.slots = (int32_t)std::min<int64_t>(num_sms(), 16 * kMaxListsPerLane);
+  prm.slots = (int32_t)std::min<int64_t>(num_sms(), kMaxLists / 2);
   prm.cl = 1;
   const SplitPlan sp = split_plan(1, prm.tiles, prm.k, prm.slots, 1);
   return launch_kernel<KREG, 1, RN>(mq, mc, prm, sp.nsplit, stream);
@@ -1972,16 +1981,14 @@ hs_status launch_resident(const uint16_t* queries, const uint16_t* corpus, int64
 
 }  // namespace
 
-// The fewest lists that a query gets over the plans of launch_variant (one
-// block of queries, or pairs of blocks); with a count that only the device
-// knows, over every count up to Q.
-static int64_t fewest_lists(int64_t Q, bool device_count, int64_t tiles, int32_t k, int64_t sms) {
-  const int64_t blocks = (Q + BM - 1) / BM;
-  const int32_t cl = blocks >= 2 ? 2 : 1;
-  const int64_t slots = sms / cl, groups = (blocks + cl - 1) / cl;
-  int64_t fewest = 2 * split_plan(Q, tiles, k, slots, cl).nsplit;
-  for (int64_t g = 1; device_count && g < std::min(groups, slots + 1); ++g)
-    fewest = std::min<int64_t>(fewest, 2 * split_plan(g * BM * cl, tiles, k, slots, cl).nsplit);
+// The fewest lists that a query gets from these executors; with a count that only
+// the device knows, over every count up to Q.
+static int64_t fewest_lists(int64_t Q, bool device_count, int64_t tiles, const Executors& ex) {
+  const int64_t groups = ((Q + BM - 1) / BM + ex.cl - 1) / ex.cl;
+  auto lists = [&](int64_t q) { return 2 * split_plan(q, tiles, 16, ex.slots, ex.cl).nsplit; };
+  int64_t fewest = lists(Q);
+  for (int64_t g = 1; device_count && g < std::min(groups, ex.slots + 1); ++g)
+    fewest = std::min<int64_t>(fewest, lists(g * BM * ex.cl));
   return fewest;
 }
 
@@ -2087,10 +2094,9 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
                    const CutOut cut = CutOut{}) -> hs_status {
     const int64_t nr = orows.inv ? orows.n_out : Qmax;
     if (nr == 0) return HS_OK;
-    // Every plan caps its executors (slots) at 16 * kMaxListsPerLane, so a
-    // query has at most 32 * kMaxListsPerLane lists: the warp merge takes
+    // Every plan caps its executors (slots) at kMaxLists / 2: the warp merge takes
     // every launch.
-    if (2 * (int64_t)pm.slots > 32 * kMaxListsPerLane)
+    if (2 * (int64_t)pm.slots > kMaxLists)
       return fail(HS_ERR_UNSUPPORTED, "more lists per query than the merge takes");
     // Up to 32 results: a block per row while there is an SM for each (256 rows
     // of 152 lists take 1 to 2 us more than with a warp each), and k is worth it:
@@ -2156,7 +2162,7 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
     if (cst != HS_OK) return cst;
     // Lists per query = 2 * nsplit of the plan the merge kernel recomputes
     // (one query block, one group: nsplit = min(slots, tiles, 8192 / k)).
-    prm.slots = (int32_t)std::max<int64_t>(1, std::min<int64_t>(sms / 2, 16 * kMaxListsPerLane));
+    prm.slots = (int32_t)std::max<int64_t>(1, std::min<int64_t>(sms / 2, kMaxLists / 2));
     prm.cl = 1;
     const SplitPlan sp = split_plan(1, tiles, k, prm.slots, 1);
     const int64_t grid = 2 * (int64_t)sp.nsplit;
@@ -2164,11 +2170,18 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
                mq16, mc128, prm, (N + SQ_BM - 1) / SQ_BM);
     st = cuda_fail(cudaGetLastError(), "retrieve launch");
   } else {
-    // How many of a query's k best one of its lists holds on average bounds the
-    // slots that a list needs.
-    const int64_t lists =
-        resident ? 2 * split_plan(1, wide ? tiles : (N + 127) / 128, 16, sms, 1).nsplit
-                 : fewest_lists(Qmax, count_dev != nullptr, tiles, 16, sms);
+    // k > 16: how many of a query's k best one of its lists holds on average bounds
+    // the slots that a list needs.
+    int64_t lists = 0;
+    if (k > 16) {
+      Executors ex{1, std::min<int64_t>(sms, kMaxLists / 2)};
+      if (!resident) {
+        st = executors<16>(Qmax, &ex);
+        if (st != HS_OK) return st;
+      }
+      lists = fewest_lists(Qmax, !resident && count_dev,
+                           resident && !wide ? (N + 127) / 128 : tiles, ex);
+    }
     const int32_t few = 4 * (int64_t)k <= 5 * lists ? kFewSlots : 2 * (int64_t)k <= 7 * lists ? 16 : 32;
     const bool guess = k > 32 ? (int64_t)k <= 32 * tiles : k > 16 && few < 32;
     // The shared per-query floors of the register-list passes start empty, and

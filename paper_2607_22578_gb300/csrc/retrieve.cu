@@ -246,43 +246,47 @@ __device__ __forceinline__ void make_cut_table(const CutQueues& c, CutTable& t, 
   const int64_t n_dev = c.count_dev ? *c.count_dev : c.Q;
   const SplitPlan sp = split_plan(n_dev < 0 ? 0 : (n_dev > c.Q ? c.Q : n_dev), c.tiles, c.list_k,
                                   c.slots, c.cl);
-  const int lists = 2 * sp.nsplit;
-  uint32_t rows = 0, blocks = 0;
-  for (int l0 = 0; l0 < lists; l0 += 32) {         // exclusive sums, 32 lists at a time
-    const uint32_t n = l0 + lane < lists ? c.count[l0 + lane] : 0u, nb = (n + BM - 1) / BM;
-    uint32_t r = n, b = nb;
+  // A lane takes `per` lists in a row: their sums, then the warp's.
+  const int lists = 2 * sp.nsplit, per = (lists + 31) / 32, first = lane * per;
+  uint32_t n[kMaxListsPerLane], rows = 0, blocks = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t yr = __shfl_up_sync(0xffffffffu, r, o);
-      const uint32_t yb = __shfl_up_sync(0xffffffffu, b, o);
-      if (lane >= o) {
-        r += yr;
-        b += yb;
-      }
-    }
-    if (l0 + lane < lists) {
-      t.row[l0 + lane] = rows + r - n;
-      t.block[l0 + lane] = blocks + b - nb;
-    }
-    rows += __shfl_sync(0xffffffffu, r, 31);
-    blocks += __shfl_sync(0xffffffffu, b, 31);
+  for (int j = 0; j < kMaxListsPerLane; ++j) {
+    n[j] = j < per && first + j < lists ? c.count[first + j] : 0u;
+    rows += n[j];
+    blocks += (n[j] + BM - 1) / BM;
   }
-  if (lane == 0) {
-    t.row[lists] = t.rows = rows;
-    t.block[lists] = t.blocks = blocks;
+  uint32_t r = rows, b = blocks;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t yr = __shfl_up_sync(0xffffffffu, r, o);
+    const uint32_t yb = __shfl_up_sync(0xffffffffu, b, o);
+    if (lane >= o) {
+      r += yr;
+      b += yb;
+    }
+  }
+  const uint32_t all = __shfl_sync(0xffffffffu, b, 31);
+  const int room = max(1, min(c.most_parts, sp.nsplit * 3 / 8));       // at most 8
+  const uint32_t parts = lane + 1;
+  const uint32_t cost =
+      (int)parts <= room ? (all * parts + sms - 1) / sms * 840u / parts : ~0u >> 5;  // lcm(1 ... 8)
+  const uint32_t best = __reduce_min_sync(0xffffffffu, cost * 32 + lane);
+  if (lane == 31) {
+    t.row[lists] = t.rows = r;
+    t.block[lists] = t.blocks = b;
     t.lists = lists;
-    const int room = max(1, min(c.most_parts, sp.nsplit * 3 / 8));
-    int best = 1;
-    uint32_t least = ~0u;
-    for (int n = 1; n <= room; ++n) {
-      const uint32_t cost = (blocks * n + sms - 1) / sms * 840u / n;   // 840: lcm(1 ... 8)
-      if (cost < least) {
-        least = cost;
-        best = n;
-      }
-    }
-    t.parts = best;
+    t.parts = (best & 31) + 1;
   }
+  r -= rows;
+  b -= blocks;
+#pragma unroll
+  for (int j = 0; j < kMaxListsPerLane; ++j)
+    if (j < per && first + j < lists) {
+      t.row[first + j] = r;
+      t.block[first + j] = b;
+      r += n[j];
+      b += (n[j] + BM - 1) / BM;
+    }
 }
 
 // Unit u of the pass over cut lists: block u / parts, part u % parts (which may be
@@ -2224,12 +2228,14 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       // a floor; with min(k, 32) slots they are enough for k <= 32.  The blocks of
       // queries cut again, or at first with 32 slots, are run exactly, from the
       // floor too.  300 queries over 131,072 x 384, 20 neighbours among the best of
-      // none, 1 in 100, all of the queries, us: k = 17 94 / 111 / 133, k = 32 101 /
-      // 117 / 139 (32 slots from the start 145 / 145 / 146 and 199 / 199 / 205),
+      // none, 1 in 100, all of the queries, us: k = 17 94 / 110 / 132, k = 32 101 /
+      // 117 / 138 (32 slots from the start 145 / 145 / 146 and 199 / 199 / 205),
       // k = 50 of all 132 (986 with 32 slots, then exactly); 2000 over 262,144 x
-      // 768, k = 17 523 / 561 / 712 (564 / 560 / 646), k = 100 of all 882 (6100).
-      // What it can cost is one more reading of the corpus, where the best of a
-      // query crowd in nearly every list: 256 over 262,144 x 1536, k = 17 290 (194).
+      // 768, k = 17 513 / 555 / 709 (558 / 560 / 643), k = 100 of all 868 (6100).
+      // What it can cost is one more reading of the corpus, where some query's best
+      // crowd in nearly every list: 256 over 262,144 x 1536, k = 17 all 243 (192); and
+      // two launches that find work, where a call is short: 256 over 12,000 x 768,
+      // k = 17 of half 84 (65).
       // The slots decide the time, as a list starts by taking nearly all it
       // sees: 300 queries over 131,072 x 384, k = 50: 237 us with 32 slots, 146
       // with 16, 126 with 12 (105 with the merge by rank and skipped passes that

@@ -264,12 +264,12 @@ __global__ void __launch_bounds__(128) fingerprint_warp_kernel(
 }
 
 // ---- the tokens past a row's full chunks, or all of a short row: a thread per row ------
-// MAX tokens at most.  chunks: the chunk pass below has run, and left the state of
-// rows of a chunk and more.
+// MAX tokens at most.  The chunk pass below has left the state of rows of a chunk and
+// more, where there can be any.
 template <int MAX, bool VEC>
 __global__ void __launch_bounds__(kFpThreads) fingerprint_rests_kernel(
     const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
-    const int32_t* __restrict__ lens, uint64_t seed, bool chunks, uint64_t* __restrict__ fp_out,
+    const int32_t* __restrict__ lens, uint64_t seed, uint64_t* __restrict__ fp_out,
     unsigned* err) {
   pdl_wait();
   pdl_trigger();
@@ -281,10 +281,9 @@ __global__ void __launch_bounds__(kFpThreads) fingerprint_rests_kernel(
       fp_out[r] = 0ull;
       continue;
     }
-    const bool on = chunks && L >= kChunk;
-    const int32_t rest = on ? L % kChunk : L;
-    if (on && rest == 0) continue;
-    const uint64_t h = on ? fp_out[r] : seed;
+    const int32_t rest = L % kChunk;
+    if (L >= kChunk && rest == 0) continue;
+    const uint64_t h = L >= kChunk ? fp_out[r] : seed;
     uint32_t lo = (uint32_t)h, hi = (uint32_t)(h >> 32);
     hash_tokens<MAX, VEC>(lo, hi, tokens + r * (int64_t)stride + (L - rest), rest);
     fp_out[r] = ((uint64_t)hi << 32) | lo;
@@ -472,20 +471,16 @@ hs_status launch_chunks(const int32_t* tokens, int64_t n, int32_t stride, const 
 }  // namespace
 
 // The full 32-token chunks only (the first pass of hs_merge_rows, whose
-// second pass finishes the tails): 16-byte aligned rows with stride % 4 == 0.
-// Sets *ran = false when no row can have a full chunk (stride < 32).
+// second pass finishes the tails; nothing where no row can have one): 16-byte
+// aligned rows with stride % 4 == 0.
 hs_status launch_fingerprint_chunks(const int32_t* tokens, int64_t n, int32_t stride,
                                     const int32_t* lens, uint64_t seed, uint64_t* fp_out,
-                                    bool* ran, cudaStream_t stream) {
-  *ran = false;
+                                    cudaStream_t stream) {
   if (stride < kChunk) return HS_OK;
   const bool vec32 = (reinterpret_cast<uintptr_t>(tokens) & 31u) == 0 && stride % 8 == 0;
   const int64_t sms = num_sms();
-  const hs_status st =
-      vec32 ? launch_chunks<32, 4, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream)
-            : launch_chunks<16, 8, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream);
-  if (st == HS_OK) *ran = true;
-  return st;
+  return vec32 ? launch_chunks<32, 4, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream)
+               : launch_chunks<16, 8, 2>(tokens, n, stride, lens, seed, fp_out, sms, stream);
 }
 
 // Aligned rows in a pass over full chunks and one over the rests, or in one that
@@ -510,7 +505,7 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
   if (!err) return fail(HS_ERR_CUDA, "could not resolve the device error word");
   const uintptr_t base = reinterpret_cast<uintptr_t>(tokens);
   const bool vec16 = (base & 15u) == 0 && stride % 4 == 0;
-  auto rests = [&](bool chunks) {
+  auto rests = [&] {
     auto* kernel = vec16 ? (stride <= 8    ? fingerprint_rests_kernel<8, true>
                             : stride <= 16 ? fingerprint_rests_kernel<16, true>
                             : stride <= 24 ? fingerprint_rests_kernel<24, true>
@@ -521,7 +516,7 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
                                            : fingerprint_rests_kernel<kChunk, false>);
     launch_pdl(kernel,
                dim3((unsigned)std::min<int64_t>((n + kFpThreads - 1) / kFpThreads, num_sms() * 64)),
-               dim3(kFpThreads), 0, stream, tokens, n, stride, lens, seed, chunks, fp_out, err);
+               dim3(kFpThreads), 0, stream, tokens, n, stride, lens, seed, fp_out, err);
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "fingerprint launch");
   };
@@ -529,7 +524,7 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
   // tokens 7 us (20 in the lanes' chunks), of 8 8.7 to 9.4 (19 to 26), of 16 15 to 21
   // (24 to 32), of 28 31 to 41 (33 to 40).  Few rows of more than 16 have a warp
   // (100 rows of 31: 3.1 us, 3.8 with a thread).
-  if (stride <= 16) return rests(false);
+  if (stride <= 16) return rests();
   // A warp per row takes 0.7 ns per row and 256 tokens at full size; a lane per
   // row the chain of the longest row while that many lanes fit the GPU, 17 to 23 ns
   // per token (50 where rows are not aligned).  us, warp / lane: aligned, 4096 rows
@@ -546,12 +541,11 @@ hs_status launch_fingerprint(const int32_t* tokens, int64_t n, int32_t stride,
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "fingerprint launch");
   }
-  if (stride < kChunk) return rests(false);
+  if (stride < kChunk) return rests();
   const bool whole = !lens && stride % kChunk == 0 && stride > 0;   // no masks needed
   if (vec16 && !whole && two_passes(n, stride, lens != nullptr)) {
-    bool ran = false;
-    const hs_status st = launch_fingerprint_chunks(tokens, n, stride, lens, seed, fp_out, &ran, stream);
-    return st == HS_OK ? rests(ran) : st;
+    const hs_status st = launch_fingerprint_chunks(tokens, n, stride, lens, seed, fp_out, stream);
+    return st == HS_OK ? rests() : st;
   }
   if ((base & 31u) == 0 && stride % 8 == 0)
     return whole ? launch_rows<32, 4, 2, false, false>(tokens, n, stride, lens, seed, fp_out, err, stream)

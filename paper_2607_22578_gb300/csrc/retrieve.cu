@@ -1171,15 +1171,15 @@ __device__ __forceinline__ uint64_t warp_max_key(uint64_t key) {
 //
 // Any kout: picks 0..31 are kept one per lane and written together when
 // kout <= 32; for larger kout each pick is written as it is made.  With
-// p.only set, rows whose query
-// block is not flagged there are skipped.  With CUT, a query is handed on to
-// `cut_out` when one of its lists may have cut off a member of the top kout: a full list whose last (k-th) entry is not below the union's
+// p.only set, rows whose query block is not flagged there are skipped.  With CUT, a
+// query is handed on to `cut_out` when one of its lists may have cut off a member
+// of the top kout: a full list whose last (k-th) entry is not below the union's
 // kout-th pick.  A list whose last entry is below it holds every row of its
-// range that can be in the top kout, so with no list cut the union's
-// first kout entries are exact.  LPL lists per lane at most (the
-// launch's bound on 2 * nsplit / 32, rounded up); slots past the query's
-// list count are skipped warp-uniformly, so the per-round work and the
-// registers follow the lists a launch can have, not the largest count.
+// range that can be in the top kout, so with no list cut the union's first kout
+// entries are exact.  LPL lists per lane at most (the launch's bound on 2 *
+// nsplit / 32, rounded up); slots past the query's list count are skipped
+// warp-uniformly, so the per-round work and the registers follow the lists a
+// launch can have, not the largest count.
 template <int LPL, bool CUT>
 __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* __restrict__ out_s,
                                                          int32_t* __restrict__ out_i,

@@ -8,9 +8,10 @@
 //   1. insert: every row offers (fp, i); equal fingerprints within a warp are
 //      combined first, the slot keeps the minimum index (atomicMin);
 //   2. lookup + verify: rep[i] = the slot's index; a row with rep[i] != i is
-//      compared in full (length + tokens) with row rep[i] (two rows per warp
-//      round, 16 lanes each).  A mismatch — rows with equal fingerprints but
-//      different contents — sends the row to a collision list;
+//      compared in full (length + tokens) with row rep[i]: the pairs of a warp's
+//      rows as one flat list of pieces, or, in the one-launch path, two pairs per
+//      warp round of 16 lanes each.  A mismatch — rows with equal fingerprints
+//      but different contents — sends the row to a collision list;
 //   3. collision list (empty unless fingerprints collide): exact regrouping
 //      in linear work — the listed rows are grouped again by a second key
 //      (a different hash of the row, mixed with its fingerprint) in the now
@@ -397,7 +398,9 @@ __device__ __forceinline__ uint64_t wait_status(const volatile unsigned long lon
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_kernel(
-    const int32_t* __restrict__ rep, int64_t n, int32_t* __restrict__ uid, unsigned long long* status, uint32_t* ctr, int32_t* total_out, unsigned* err, uint64_t limit_ns, int64_t withhold_tile) {
+    const int32_t* __restrict__ rep, int64_t n, int32_t* __restrict__ uid,
+    unsigned long long* status, uint32_t* ctr, int32_t* total_out, unsigned* err,
+    uint64_t limit_ns, int64_t withhold_tile) {
   pdl_wait();
   pdl_trigger();
   constexpr int kWarps = kScanThreads / 32;
@@ -613,69 +616,35 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
 }
 
 // ---- hs_merge_rows: second pass of the fingerprint, fused with the insert ---------------------
-// One thread per row finishes the fingerprint (the last L mod 32 tokens,
-// from the state the chunk kernel left in fp_out, or the whole row when it
-// is shorter than 32 tokens or the chunk kernel did not run), writes it,
-// and offers (fp & key_mask, row) to the table in the same pass: rows of a
-// warp with equal keys are combined and the smallest index inserts
-// (atomicMin), as insert_kernel does.  An invalid length sets the error
-// word and a zero fingerprint, as hs_fingerprint does.  Rows [row0,
-// row_end); row0 is a multiple of 32 (warps combine their rows' inserts).
+// One thread per row finishes the fingerprint (the last L mod 32 tokens, from the
+// state the chunk kernel left in fp_out, or all of a row shorter than 32 tokens;
+// the chunk kernel runs where any row can be as long), writes it, and offers
+// (fp & key_mask, row) to the table in the same pass: rows of a warp with equal
+// keys are combined and the smallest index inserts (atomicMin), as insert_kernel
+// does.  An invalid length sets the error word and a zero fingerprint, as
+// hs_fingerprint does.
 __global__ void __launch_bounds__(256) tails_insert_kernel(
-    const int32_t* __restrict__ tokens, int64_t row0, int64_t row_end, int32_t stride,
-    const int32_t* __restrict__ lens, uint64_t seed, bool chunks_ran, uint64_t key_mask,
+    const int32_t* __restrict__ tokens, int64_t n, int32_t stride,
+    const int32_t* __restrict__ lens, uint64_t seed, uint64_t key_mask,
     uint64_t* __restrict__ fp_out, uint64_t* keys, uint32_t* idx, int log2T, unsigned* err) {
   pdl_wait();
   pdl_trigger();
   constexpr int T = 32;
-  for (int64_t base = row0 + (int64_t)blockIdx.x * blockDim.x; base < row_end;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
        base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = base + threadIdx.x;
-    const bool valid = r < row_end;
+    const bool valid = r < n;
     uint64_t f = 0;
     if (valid) {
       const int32_t L = lens ? __ldg(lens + r) : stride;
       if (L < 0 || L > stride) {
         set_error(err, kErrInvalidArg);
       } else {
-        const int32_t m = L % T;
-        const bool from_chunks = chunks_ran && L >= T;
-        if (from_chunks && m == 0) {
-          f = fp_out[r];                           // the chunk kernel wrote the final value
-        } else {
-          uint32_t lo = (uint32_t)seed, hi = (uint32_t)(seed >> 32);
-          int32_t t0 = 0;
-          if (from_chunks) {
-            const uint64_t st = fp_out[r];
-            lo = (uint32_t)st;
-            hi = (uint32_t)(st >> 32);
-            t0 = L - m;
-          }
-          // at most 31 tokens remain past the full chunks (fewer than 32 in a
-          // short row): all their 16-byte pieces are loaded before hashing
-          const int32_t* src = tokens + r * (int64_t)stride + t0;
-          const int32_t m2 = L - t0;               // tokens to hash here
-          if (m2 < T) {
-            uint4 v[T / 4];
-#pragma unroll
-            for (int q = 0; q < T / 4; ++q)
-              if (4 * q < m2) v[q] = __ldg(reinterpret_cast<const uint4*>(src + 4 * q));
-#pragma unroll
-            for (int q = 0; q < T / 4; ++q) {
-              if (4 * q < m2) fnv::hash_word(lo, hi, v[q].x);
-              if (4 * q + 1 < m2) fnv::hash_word(lo, hi, v[q].y);
-              if (4 * q + 2 < m2) fnv::hash_word(lo, hi, v[q].z);
-              if (4 * q + 3 < m2) fnv::hash_word(lo, hi, v[q].w);
-            }
-          } else {                                 // a whole row (no chunk pass ran)
-            for (int32_t t = 0; t < m2; t += 4) {  // 16-byte pieces, the last one masked
-              const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + t));
-              fnv::hash_word(lo, hi, v.x);
-              if (t + 1 < m2) fnv::hash_word(lo, hi, v.y);
-              if (t + 2 < m2) fnv::hash_word(lo, hi, v.z);
-              if (t + 3 < m2) fnv::hash_word(lo, hi, v.w);
-            }
-          }
+        const int32_t rest = L % T;
+        f = L >= T ? fp_out[r] : seed;
+        if (rest > 0) {
+          uint32_t lo = (uint32_t)f, hi = (uint32_t)(f >> 32);
+          fnv::hash_tokens<T, true>(lo, hi, tokens + r * (int64_t)stride + (L - rest), rest);
           f = ((uint64_t)hi << 32) | lo;
         }
       }
@@ -941,7 +910,7 @@ hs_status launch_unique_inverse(const uint64_t* fp, const int32_t* tokens, int64
 hs_status launch_fingerprint(const int32_t*, int64_t, int32_t, const int32_t*, uint64_t,
                              uint64_t*, cudaStream_t);
 hs_status launch_fingerprint_chunks(const int32_t*, int64_t, int32_t, const int32_t*, uint64_t,
-                                    uint64_t*, bool*, cudaStream_t);
+                                    uint64_t*, cudaStream_t);
 
 // Test hook of hs_merge_rows (hs_debug_merge_key_mask): the table key is
 // fp & mask, so a narrow mask forces fingerprint collisions.
@@ -976,12 +945,10 @@ hs_status launch_merge_rows(const int32_t* tokens, int64_t n, int32_t stride, co
   int32_t* coll_list = reinterpret_cast<int32_t*>(w + L.coll_list);
   const int sms = num_sms();
   launch_clear(w, L, sms, stream);
-  bool ran = false;
-  const hs_status st =
-      launch_fingerprint_chunks(tokens, n, stride, lens, seed, fp_out, &ran, stream);
+  const hs_status st = launch_fingerprint_chunks(tokens, n, stride, lens, seed, fp_out, stream);
   if (st != HS_OK) return st;
-  launch_pdl(tails_insert_kernel, dim3(grid_for(n, 256, sms * 16)), dim3(256), 0, stream, tokens,
-             (int64_t)0, n, stride, lens, seed, ran, mask, fp_out, keys, idx, L.log2T, err);
+  launch_pdl(tails_insert_kernel, dim3(grid_for(n, 256, sms * 16)), dim3(256), 0, stream, tokens, n,
+             stride, lens, seed, mask, fp_out, keys, idx, L.log2T, err);
   const int vr = verify_rows(n, sms);
   launch_pdl(verify_flat_kernel<true>, dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)),
              dim3(kVerifyThreads), 0, stream, (const uint64_t*)fp_out, mask, n,

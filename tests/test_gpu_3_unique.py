@@ -168,7 +168,7 @@ def test_lookback_wait_runs_out_and_reports_timeout():
     and the next call on the same stream is exact again."""
     import time
     w = configs.build_dedup_heavy(scale=0.2)
-    tok, ln = w["tokens"][:70000], w["lens"][:70000]     # five scan tiles
+    tok, ln = w["tokens"][:70000], w["lens"][:70000]     # 18 scan tiles
     t, L = to_dev(tok), to_dev(ln)
     f = hs.hs_fingerprint(t, L)
     hs.hs_get_device_error()

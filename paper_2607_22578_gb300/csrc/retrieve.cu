@@ -2086,12 +2086,12 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
   // 30.5, 2,000,000 x 256 177 to 187 / 189 / 173, 1,000,000 x 768 235 to 255 /
   // 240 / 236 to 241.  A stage's batch of 64 over 2,097,152 x 768: 508 -> 475.
   // Where the merge takes k rounds over its lists, tiles of 128 are taken only if
-  // those of 256 give too few lists for short ones (3 queries, 32,768 x 1024, k =
-  // 500: 296 with 304 lists, 238 with 256; 1 query, 4096 x 1024, k = 200: 107 with
-  // 64 lists of 16, 125 with 32 of 32).
+  // those of 256 give as many lists, or too few for short ones (3 queries, 32,768 x
+  // 1024, k = 500: 296 with 304 lists, 238 with 256; 1 query, 4096 x 1024, k = 200:
+  // 107 with 64 lists of 16, 125 with 32 of 32).
   const bool wide = prm.kb_count <= kResMaxKbWide && (N + 127) / 128 > sms;
   const bool resident = !small && Qmax <= RQ && prm.kb_count <= kResMaxKb &&
-                        (wide || k <= kMrMaxK || (int64_t)k > 7 * std::min<int64_t>(sms, tiles));
+                        (wide || k <= kMrMaxK || tiles >= sms || (int64_t)k > 7 * tiles);
   const OutRows rows{inv, n_out};
   const int64_t R = inv ? n_out : Qmax;             // rows the final merge writes
   auto merge = [&](const Params& pm, int32_t kout, float* os, int32_t* oi, OutRows orows,

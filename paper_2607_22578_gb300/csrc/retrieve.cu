@@ -1171,8 +1171,8 @@ __device__ __forceinline__ uint64_t warp_max_key(uint64_t key) {
 //
 // Any kout: picks 0..31 are kept one per lane and written together when
 // kout <= 32; for larger kout each pick is written as it is made.  With
-// p.only set, rows whose query block is not flagged there are skipped.  With CUT, a
-// query is handed on to `cut_out` when one of its lists may have cut off a member
+// p.only set, rows whose query block is not flagged there are skipped.  With CUT and
+// cut_out.floor set, a query is handed on to `cut_out` when one of its lists may have cut off a member
 // of the top kout: a full list whose last (k-th) entry is not below the union's
 // kout-th pick.  A list whose last entry is below it holds every row of its
 // range that can be in the top kout, so with no list cut the union's first kout
@@ -1256,7 +1256,7 @@ __global__ void __launch_bounds__(256) merge_warp_kernel(const Params p, float* 
       out_s[(size_t)o * kout + lane] = my_s;
       out_i[(size_t)o * kout + lane] = my_i;
     }
-    if (CUT) {
+    if (CUT && cut_out.floor) {
       if (lane == 0) cut_out.floor[q] = key_floor(last);
       auto cut = [&](int l) {                      // is list l?
         if (l >= lists) return false;
@@ -2138,14 +2138,15 @@ hs_status launch_retrieve_topk(const uint16_t* queries, int64_t Qmax, const int3
       const dim3 grid((unsigned)(blocks < sms * 16 ? blocks : sms * 16));
       // lists per query <= 2 * slots (nsplit <= slots): lanes need that / 32
       const int64_t lpl = (2 * (int64_t)pm.slots + 31) / 32;
-      auto* kernel = cut.floor ? (lpl <= 2   ? merge_warp_kernel<2, true>
-                                  : lpl <= 3 ? merge_warp_kernel<3, true>
-                                  : lpl <= 5 ? merge_warp_kernel<5, true>
-                                             : merge_warp_kernel<kMaxListsPerLane, true>)
-                               : (lpl <= 2   ? merge_warp_kernel<2, false>
-                                  : lpl <= 3 ? merge_warp_kernel<3, false>
-                                  : lpl <= 5 ? merge_warp_kernel<5, false>
-                                             : merge_warp_kernel<kMaxListsPerLane, false>);
+      // The hand-on costs only the longest lists registers that they need: without
+      // it <5> has 78 instead of 114, a third block fits an SM, and the blocks that
+      // wait for a retrieval's first free SMs crowd there (256 queries over 20,000 x
+      // 384, k = 10: 39.6 us, 37.7 with 114).
+      auto* kernel = lpl <= 2    ? merge_warp_kernel<2, true>
+                     : lpl <= 3  ? merge_warp_kernel<3, true>
+                     : lpl <= 5  ? merge_warp_kernel<5, true>
+                     : cut.floor ? merge_warp_kernel<kMaxListsPerLane, true>
+                                 : merge_warp_kernel<kMaxListsPerLane, false>;
       launch_pdl(kernel, grid, dim3(256), 0, stream, pm, os, oi, kout, orows, cut);
       return cuda_fail(cudaGetLastError(), "merge launch");
     }

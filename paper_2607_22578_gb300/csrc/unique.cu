@@ -522,13 +522,14 @@ __global__ void __launch_bounds__(256) finalize_kernel(const int32_t* __restrict
 // the tokens of a pair's last piece past its length masked.  Otherwise the
 // rows may start on any word and a piece is one word, coalesced over the
 // lanes: 20,011 rows at a stride of 333, a third of them copies, take 21 us cold (40
-// us as two rows per warp round).  As many in flight as of the others: with eight,
-// whose registers cost a block in six, 1,000,000 rows of 31 words, a tenth of them
-// copies, take 106 us from fingerprints to inverse, 96 so, and the small batches are
-// no faster.  Batches
-// that do not fill the GPU with 32 rows per warp take fewer, down to 4, so a
-// warp's chain of rounds is shorter: with the scan's smaller tiles 20,011 rows
-// take 25 us from fingerprints to inverse (35), 65,536 rows of 256 tokens 33 (38).
+// us as two rows per warp round).  Eight of these are in flight per lane; four in
+// rows of fewer than 64, where the registers of eight cost a block in six and more
+// than they give.  Fingerprints to inverse, us, four / eight: 1,000,000 rows of 31, a
+// tenth copies, 96 / 106; 400,000 of 64, half copies, 59.4 / 58.8; 200,000 of 128 54.2 /
+// 49.2, of 333 102 / 90.  Batches that do not fill the GPU with 32 rows per warp take
+// fewer, down to 4, so a warp's chain of rounds is shorter: with the scan's smaller
+// tiles 20,011 rows take 25 us from fingerprints to inverse (35), 65,536 rows of 256
+// tokens 33 (38).
 constexpr int kVerifyThreads = 256;
 
 // Do the first `live` tokens of two 16-byte pieces, or two words, differ?
@@ -538,7 +539,7 @@ __device__ __forceinline__ bool piece_differs(const uint4& x, const uint4& y, in
 }
 __device__ __forceinline__ bool piece_differs(uint32_t x, uint32_t y, int) { return x != y; }
 
-template <bool VEC>
+template <bool VEC, int kPieces>
 __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
     const uint64_t* __restrict__ fp, uint64_t key_mask, int64_t n,
     const uint64_t* __restrict__ keys, const uint32_t* __restrict__ idx, int log2T,
@@ -547,7 +548,6 @@ __global__ void __launch_bounds__(kVerifyThreads) verify_flat_kernel(
     unsigned* err) {
   pdl_wait();
   pdl_trigger();
-  constexpr int kPieces = 4;
   __shared__ int32_t s_pre[kVerifyThreads / 32][32];
   __shared__ int32_t s_a[kVerifyThreads / 32][32];
   __shared__ int32_t s_b[kVerifyThreads / 32][32];
@@ -888,7 +888,9 @@ hs_status launch_unique_inverse(const uint64_t* fp, const int32_t* tokens, int64
   launch_pdl(insert_kernel, dim3(grid_for(n, 256, sms * 8)), dim3(256), 0, stream, fp, n, keys, idx,
              L.log2T);
   const int vr = verify_rows(n, sms);
-  launch_pdl(vec ? verify_flat_kernel<true> : verify_flat_kernel<false>,
+  launch_pdl(vec           ? verify_flat_kernel<true, 4>
+             : stride < 64 ? verify_flat_kernel<false, 4>
+                           : verify_flat_kernel<false, 8>,
              dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)), dim3(kVerifyThreads), 0, stream,
              fp, ~0ull, n, (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride,
              lens, vr, rep, coll_list, ctr, err);
@@ -950,7 +952,7 @@ hs_status launch_merge_rows(const int32_t* tokens, int64_t n, int32_t stride, co
   launch_pdl(tails_insert_kernel, dim3(grid_for(n, 256, sms * 16)), dim3(256), 0, stream, tokens, n,
              stride, lens, seed, mask, fp_out, keys, idx, L.log2T, err);
   const int vr = verify_rows(n, sms);
-  launch_pdl(verify_flat_kernel<true>, dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)),
+  launch_pdl(verify_flat_kernel<true, 4>, dim3(grid_for(n, vr * (kVerifyThreads / 32), sms * 8)),
              dim3(kVerifyThreads), 0, stream, (const uint64_t*)fp_out, mask, n,
              (const uint64_t*)keys, (const uint32_t*)idx, L.log2T, tokens, stride, lens, vr, rep,
              coll_list, ctr, err);

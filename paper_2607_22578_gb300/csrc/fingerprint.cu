@@ -30,9 +30,10 @@ using namespace fnv;
 // exactly as if the padding had not been there.  So every lane runs the same
 // straight-line hash whatever its row's start and length, in one pass.
 //
-// Bound by the memory system where there are rows enough: 16 warps an SM each keep
-// one 128-byte chunk per lane in flight, in as many places as there are rows.
-// 200,000 rows of 512 tokens: 81 us, 5.0 TB/s; 400,000 rows of 8 to 36: 19.6 us
+// Where there are rows enough, 16 warps an SM (all that the two buffers' registers
+// leave) share their time between a chunk's arrival and its chain: issue slots 56 to
+// 59 % busy, DRAM at 3.2 to 4.2 TB/s (400,000 unaligned rows of 333 words, aligned
+// ones of 64 to 256).  200,000 rows of 512 tokens: 81 us, 5.0 TB/s; 400,000 of 8 to 36: 19.6 us
 // (23.6 as a pass over full chunks and a second one over the rests); 20,011 rows at a
 // stride of 333: 19 us (75 hashing word by word), where the chain bounds it.  Rests
 // queued and hashed 32 at a time, masks or steps left out by a vote of the warp
